@@ -70,14 +70,14 @@ typedef enum fdd_status {
                              periodicity searches (Sect. 5)                     */
 
 /* Kernel tiles of the FP32 phase-rotate-and-sum (fdd_params.mac_variant - 1,
- * fdd_info.mac_variant).  All issue paired f32x2 FMAs on an A x B register
- * tile per lane (a warp covers 2048, 1024, 4 x 512 or 4 x 128 trials of its
- * bins); W12 and G12 split phasor evaluation (4 warps) from the
- * multiply-accumulates (8 warps), the others let every warp do both.  With
- * mac_variant 0 a plan takes the tile with the least time for its trial
- * count whose shared memory holds the channels' phase table: G12_4X8 from
- * 257 trials, Q_4X4 below; above 8381 channels G12_4X8 no longer fits and
- * the fastest of the others that do is taken. */
+ * fdd_info.mac_variant).  G12_4X8 runs on the tensor cores with operands split
+ * into two FP16 terms (FP32 accuracy); the others issue paired f32x2 FMAs on
+ * an A x B register tile per lane (a warp covers 2048, 1024, 4 x 512 or 4 x 128
+ * trials of its bins); W12 splits phasor evaluation (4 warps) from the
+ * multiply-accumulates (8 warps), the rest let every warp do both.  With
+ * mac_variant 0 a plan takes G12_4X8 from 257 trials and the fastest of the
+ * others below; above 8381 channels the fastest of the others whose shared
+ * memory holds the channels' phase table. */
 #define FDD_MAC_W12_8X8 0   /* warp-specialised, 2048-trial blocks, four real
                                products per complex MAC                         */
 #define FDD_MAC_Q12_8X8 1   /* 2048-trial blocks, 12 warps, plain schedule       */
@@ -86,11 +86,11 @@ typedef enum fdd_status {
                                warp: 512-trial blocks                           */
 #define FDD_MAC_Q_4X4 4     /* 4x4 lane tile, four bins per warp: 128-trial
                                blocks (small trial counts, ragged tails)        */
-#define FDD_MAC_G12_4X8 5   /* warp-specialised, 2048-trial blocks, three real
-                               products per complex MAC (Gauss's form): 4 phasor
-                               warps feed 8 MAC warps, two per bin; a last block
-                               of <= 1024 / <= 512 trials runs as wide items of
-                               8 / 16 bins (default from 257 trials)            */
+#define FDD_MAC_G12_4X8 5   /* trials paired around centres, so that a bin is one real
+                               matrix product (half the multiplications and
+                               phasors of the complex form); hi + lo FP16 operands,
+                               three products, FP32 sums; passes of up to 4096
+                               trials (default from 257 trials)                 */
 #define FDD_MAC_VARIANTS 6
 #define FDD_MAC_TC 100      /* fdd_info.mac_variant of the tensor-core form: one
                                CTA per SM, a pass over the channels covering
@@ -509,8 +509,8 @@ typedef struct fdd_batch_info {
                               -1 (none).  With the W12_8X8 tile a beam's last
                               block of 1024 or fewer trials runs in a second
                               persistent launch on this tile's 128-trial blocks;
-                              the G12_4X8 tile runs such a block in its own
-                              launch as wide items (eight bins x 1024 trials)  */
+                              the G12_4X8 tile spreads a beam's trials over its
+                              passes and has no tails                          */
   double autotune_ms[FDD_MAC_VARIANTS]; /* timed candidates (ms), -1 if untimed */
 } fdd_batch_info;
 

@@ -57,6 +57,7 @@ struct fdd_batch_s {
   };
   std::vector<Wave> waves;
   int64_t in_elems = 0, out_elems = 0;
+  int max_n_dm = 0;  // largest trial count of the beams
   // device memory
   fdd::PhaseConst* d_pc = nullptr;  // [beam][n_chan]
   float* d_xw = nullptr;            // [n_chan][L_max]
@@ -221,11 +222,11 @@ fdd_status issue(fdd_batch_s* B, const void* d_in, cudaStream_t s) {
     }
     B_CUDA(cudaMemsetAsync(B->d_counter + 2 * wi, 0, 2 * sizeof(unsigned long long), s));
     B_CUDA(fdd::launch_mac_batch(w.d_sets, static_cast<int>(w.h_sets.size()), w.n_items,
-                                 B->d_counter + 2 * wi, B->variant, B->ctas, B->p.n_chan, s));
+                                 B->d_counter + 2 * wi, B->variant, B->ctas, B->p.n_chan, B->max_n_dm, s));
     if (w.n_tail_items)
       B_CUDA(fdd::launch_mac_batch(w.d_tail, static_cast<int>(w.h_tail.size()), w.n_tail_items,
                                    B->d_counter + 2 * wi + 1, B->tail_variant, B->tail_ctas,
-                                   B->p.n_chan, s));
+                                   B->p.n_chan, B->max_n_dm, s));
   }
   return FDD_OK;
 }
@@ -613,6 +614,7 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
     in_acc += d.n_t * static_cast<int64_t>(p->n_chan);
     out_acc += g.n_chunks * g.n_bins * static_cast<int64_t>(d.n_dm);
     L_max = std::max(L_max, g.fft_len);
+    B->max_n_dm = std::max(B->max_n_dm, d.n_dm);
     fdd::CoreGeometry cg;
     if ((st = fdd::core_geometry(&q, &cg)) != FDD_OK) return st;
     for (int c = 0; c < p->n_chan; ++c)
@@ -717,13 +719,13 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
     return m;
   };
   auto build_sets = [&](int variant) -> fdd_status {
-    const int bins_per_cta = fdd::mac_variant_bins_per_cta(variant);
+    const bool g12 = variant == FDD_MAC_G12_4X8;
+    const int bins_per_cta = g12 ? 0 : fdd::mac_variant_bins_per_cta(variant);
     const int dms = fdd::mac_variant_trials_per_block(variant);
     const int tv = B->tail_variant;
     const int tail_dms = tv >= 0 ? fdd::mac_variant_trials_per_block(tv) : 0;
-    // (the three-product tile runs a ragged last block of up to half its
-    // trials in the same launch, as wide items: no second launch)
-    const bool tails = tv >= 0 && dms >= 2048 && tail_dms < dms && variant != FDD_MAC_G12_4X8;
+    // (the G12 tile spreads a beam's trials evenly over its passes: no tails)
+    const bool tails = tv >= 0 && dms >= 2048 && tail_dms < dms && !g12;
     for (auto& wv : B->waves) {
       wv.h_sets.clear();
       wv.set_beam.clear();
@@ -737,31 +739,20 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
         const int n_dm = B->beams[b].n_dm;
         const int full = n_dm / dms, rem = n_dm % dms;
         const bool tail = tails && rem > 0 && rem <= dms / 2;
-        // the three-product tile's last trials as wide items: up to 512 one
-        // 512-trial item, up to 1024 one 1024-trial item, up to 1536 both
-        // (cheaper than a full block at the measured rates), else a full block
-        const bool g12 = variant == FDD_MAC_G12_4X8;
-        const bool wide = g12 && rem > dms / 4 && rem <= 3 * dms / 4;
-        const bool narrow = g12 && rem > 0 && (rem <= dms / 4 || (rem > dms / 2 && rem <= 3 * dms / 4));
-        const int blocks = full + (rem > 0 && !tail && !wide && !narrow ? 1 : 0);
+        int blocks = full + (rem > 0 && !tail ? 1 : 0), tiles = 0;
+        if (g12)
+          fdd::mac_split_batch_shape(B->max_n_dm, n_dm, B->n_bins[b], &tiles, &blocks);
+        else
+          tiles = static_cast<int>((B->n_bins[b] + bins_per_cta - 1) / bins_per_cta);
         for (int64_t c = 0; c < B->n_chunks[b]; ++c) {
           fdd::BatchSet bs{};
           bs.args = base_args(b, c);
           bs.args.j_begin = 0;
           bs.args.n_dm = tail ? full * dms : n_dm;
-          bs.n_bin_tiles = static_cast<int>((B->n_bins[b] + bins_per_cta - 1) / bins_per_cta);
+          bs.n_bin_tiles = tiles;
           bs.n_dm_blocks = blocks;
           bs.item_begin = items;
-          bs.n_wide_tiles = wide ? static_cast<int>((B->n_bins[b] + 2 * bins_per_cta - 1) /
-                                                    (2 * bins_per_cta))
-                                 : 0;
-          bs.j_wide = full * dms;
-          bs.n_narrow_tiles = narrow ? static_cast<int>((B->n_bins[b] + 4 * bins_per_cta - 1) /
-                                                        (4 * bins_per_cta))
-                                     : 0;
-          bs.j_narrow = full * dms + (wide ? dms / 2 : 0);
-          items += static_cast<long long>(bs.n_bin_tiles) * blocks + bs.n_wide_tiles +
-                   bs.n_narrow_tiles;
+          items += static_cast<long long>(tiles) * blocks;
           wv.h_sets.push_back(bs);
           wv.set_beam.push_back(b);
           wv.set_chunk.push_back(static_cast<int>(c));
@@ -861,7 +852,8 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
         for (int rep = 0; rep < 2; ++rep) {  // the first launch is a warm-up
           cudaMemset(counter, 0, sizeof(unsigned long long));
           cudaEventRecord(e0);
-          fdd::launch_mac_batch(sets, n_sets, part, counter, tile, ctas, p->n_chan, nullptr);
+          fdd::launch_mac_batch(sets, n_sets, part, counter, tile, ctas, p->n_chan, B->max_n_dm,
+                                nullptr);
           cudaEventRecord(e1);
           cudaEventSynchronize(e1);
           cudaEventElapsedTime(&ms, e0, e1);
@@ -1073,11 +1065,11 @@ fdd_status fdd_batch_execute_stream(fdd_batch_t b, fdd_source_fn source, void* s
     B_CUDA(cudaMemsetAsync(b->d_counter + 2 * wi, 0, 2 * sizeof(unsigned long long), s));
     const int n_sets = static_cast<int>(w.h_sets.size());
     B_CUDA(fdd::launch_mac_batch(d_sets, n_sets, w.n_items, b->d_counter + 2 * wi, b->variant,
-                                 b->ctas, b->p.n_chan, s));
+                                 b->ctas, b->p.n_chan, b->max_n_dm, s));
     if (w.n_tail_items)
       B_CUDA(fdd::launch_mac_batch(d_sets + n_sets, static_cast<int>(w.h_tail.size()),
                                    w.n_tail_items, b->d_counter + 2 * wi + 1, b->tail_variant,
-                                   b->tail_ctas, b->p.n_chan, s));
+                                   b->tail_ctas, b->p.n_chan, b->max_n_dm, s));
     const int64_t origin = b->out_off[w.first];
     void* release = nullptr;
     for (int i = 0; i < w.count; ++i) {

@@ -68,15 +68,8 @@ enum MacVariant {
 struct BatchSet {
   MacArgs args;
   long long item_begin;  // first work item of this set
-  int n_dm_blocks;       // trial blocks (items per bin tile)
-  int n_bin_tiles;
-  // the three-product tile only, numbered after the n_bin_tiles x
-  // n_dm_blocks items: wide items of 1024 trials (twice the bins) from trial
-  // j_wide, then wide items of 512 trials (four times the bins) from j_narrow
-  int n_wide_tiles;
-  int j_wide;
-  int n_narrow_tiles;
-  int j_narrow;
+  int n_dm_blocks;       // trial blocks (items per bin tile; the G12 tile's passes)
+  int n_bin_tiles;       // (the G12 tile's groups of bins)
 };
 
 // The FP32 tile with the least time for n_dm trials among those whose
@@ -88,11 +81,23 @@ bool mac_variant_batchable(int variant);
 int mac_batch_ctas_per_sm(int variant, int n_chan);
 cudaError_t launch_mac_batch(const BatchSet* d_sets, int n_sets, long long n_items,
                              unsigned long long* d_counter, int variant, int n_ctas,
-                             int n_chan, cudaStream_t s);
+                             int n_chan, int max_n_dm, cudaStream_t s);
 int mac_variant_trials_per_block(int variant);
 cudaError_t mac_prepare(int variant, int n_chan);  // kernel attributes (host, once)
 cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s);
 size_t mac_smem_bytes(int variant, int n_chan);
+
+// The G12_4X8 tile (fdd_mac_split.cu): split-FP16 operands on the tensor
+// cores.  Batches are shaped by their largest trial count (the trials a pass
+// can hold and the bins a CTA works on together follow from it):
+// mac_split_batch_shape gives a set's bin groups and passes, whose product
+// numbers its items pass-major; the persistent launch deals them out in turn.
+size_t mac_split_smem_bytes();
+cudaError_t mac_split_prepare();
+cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s);
+void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes);
+cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
+                                   int max_n_dm, int n_ctas, cudaStream_t s);
 
 // Tensor-core phase-rotate-and-sum (fdd_mac_tc.cu): 16-bit (or FP8)
 // phasors and data, FP32 accumulation in tensor memory; persistent CTAs (one

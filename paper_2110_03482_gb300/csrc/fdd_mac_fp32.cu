@@ -553,521 +553,6 @@ __global__ void __launch_bounds__(W * 32, 1) mac_batch_kernel(const BatchSet* se
   }
 }
 
-// --------------------------------------- three-multiplication warp-specialised tile
-// The complex multiply-accumulate y += z p needs four real products; with
-//   A += zr pr,  B += zi pi,  C += (zr + zi)(pr + pi)
-// accumulated instead, Re y = A - B and Im y = C - A - B at the end: three
-// real products per complex MAC (Gauss's three-multiplication form).  Its
-// FP32 rounding is that of the four-product form to within a few percent
-// (every term is of the size of a product of the four-product form).  The
-// tile: producer warp q evaluates, for bin q of the CTA's four and each
-// channel, the 64 Z_a = X Q_a and 32 P_b of a 2048-trial block (T = 32), as
-// planes zr, zi and pr, pi; consumer warps 2q and 2q + 1 own the a's 0..31
-// and 32..63 of that bin, each lane a 4 x 8 tile of (a, b) with the three
-// accumulators as pairs along b, the sums zr + zi and pr + pi formed in
-// registers after the loads (shared-memory traffic per lane as the
-// four-product form's, two floats per operand): 48 paired FMAs and 6 paired
-// adds per lane and channel for 32 complex MACs.  A stage carries kCh
-// channels of full items (16 in use: against 4, a quarter of the barrier
-// round trips per channel and longer independent runs of loads and FMAs;
-// 0.661, 0.726 and 0.752 of the FP32 peak with 4, 8 and 16 channels on the
-// same launch) and kChWide = 8 of wide items, whose per-channel operands
-// are up to twice as large.
-template <int kCh, int kStages>
-struct G3 {
-  static constexpr int kA = 64;                // a's per bin (Z_a)
-  static constexpr int kT = 32;                // b's per bin (P_b): T
-  static constexpr int kDms = kA * kT;         // 2048 trials per bin
-  static constexpr int kBins = 4;              // bins per CTA (one producer warp each)
-  static constexpr int kCons = 2 * kBins;      // consumer warps
-  static constexpr int kProd = kBins;          // producer warps
-  static constexpr int kThreads = 32 * (kCons + kProd);
-  static constexpr int kGFL = 2 * kA + 2 * kT;  // floats per (bin, channel): zr zi pr pi
-  // wide items (a ragged remainder of at most 1024 or 512 trials): the a's
-  // 0 .. kAw - 1 (kAw 32 or 16) of 8 x 32 / kAw bins, zr zi (kAw each) and
-  // pr pi (32 each) per (bin, channel)
-  __host__ __device__ static constexpr int wide_bins(int aw) { return 8 * 32 / aw; }
-  __host__ __device__ static constexpr int wide_floats(int aw) { return 2 * aw + 2 * kT; }
-  static constexpr int kWideMax = wide_bins(16) * wide_floats(16) > wide_bins(32) * wide_floats(32)
-                                      ? wide_bins(16) * wide_floats(16)
-                                      : wide_bins(32) * wide_floats(32);
-  // channels per stage of the wide items (their per-channel operands are up
-  // to twice the full item's, so they fill a stage with fewer channels)
-  static constexpr int kChWide = kCh < 8 ? kCh : 8;
-  static constexpr int kStageFloats = kCh * kBins * kGFL > kChWide * kWideMax
-                                          ? kCh * kBins * kGFL
-                                          : kChWide * kWideMax;
-  static constexpr size_t kBarBytes = (2 * kStages * 8 + 4 + 15) / 16 * 16;
-  static constexpr size_t kSwapBytes = kBarBytes + sizeof(float) * size_t(kStages) * kStageFloats;
-};
-
-// One work item of the three-multiplication tile: the CTA's four bins from
-// local bin bin_tile * 4 and trials dm_block * 2048 + .. of one set of
-// spectra; ring stages and barrier phases continue from iteration it0.
-// Returns false after a timeout.
-template <int kCh, int kStages>
-__device__ __forceinline__ bool g3_body(const MacArgs& a, const PhaseConst* pcs, float* stages,
-                                        uint64_t* full, uint64_t* empty,
-                                        volatile int* abort_flag, int bin_tile, int dm_block,
-                                        int series, uint32_t it0) {
-  using Ly = G3<kCh, kStages>;
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  const int n_iter = (a.n_chan + kCh - 1) / kCh;
-  const int jblk = dm_block * Ly::kDms;
-  bool ok = true;
-
-  if (warp >= Ly::kCons) {
-    // ------------------------------------------------------------ producers
-    const int q = warp - Ly::kCons;               // the CTA's bin q
-    const int k = bin_tile * Ly::kBins + q;
-    const int kl = k < a.n_bins ? k : 0;          // idle bins evaluate local bin 0, unused
-    const uint32_t ku = static_cast<uint32_t>(a.k_begin + kl);
-    // Phases (units of 2^-32 cycle) of trial j0 + a T + b, j0 the block's
-    // first trial: Z_a takes k u + k j0 v + a (T k v) and P_b takes b k v.
-    // The lane-independent parts k u + k j0 v and 32 T k v of a channel are
-    // evaluated by one lane per channel and broadcast; a lane's own P phase
-    // (b = lane) gives its Z phases by a shift and an add (a T k v = T (a k
-    // v)), within 33 units of the exact phase.
-    const uint32_t m_j0 = ku * static_cast<uint32_t>(a.j_begin + jblk);
-    const uint32_t m_d = ku * static_cast<uint32_t>(32 * Ly::kT);
-    const uint32_t m_p = ku * static_cast<uint32_t>(lane);
-    static_assert(Ly::kT == 32 && kCh <= 32 && (kCh & (kCh - 1)) == 0, "phase layout");
-    const float2* xp = a.X + static_cast<int64_t>(series) * a.x_series_stride + kl;
-    const int64_t xs = a.x_chan_stride;
-    float2 xn[kCh];
-#pragma unroll
-    for (int ch = 0; ch < kCh; ++ch)
-      xn[ch] = ch < a.n_chan ? __ldg(xp + ch * xs) : make_float2(0.f, 0.f);
-    for (int it = 0; it < n_iter; ++it) {
-      const uint32_t g = it0 + it;
-      const int s = g % kStages;
-      float2 x[kCh];
-#pragma unroll
-      for (int ch = 0; ch < kCh; ++ch) {
-        x[ch] = xn[ch];
-        const int c = (it + 1) * kCh + ch;  // prefetch the next stage's X
-        xn[ch] = c < a.n_chan ? __ldg(xp + c * xs) : make_float2(0.f, 0.f);
-      }
-      ok = __all_sync(0xffffffffu,
-                      dev::mbar_wait(&empty[s], ((g / kStages) & 1) ^ 1, abort_flag));
-      if (!ok) break;
-      float* st = stages + s * Ly::kStageFloats + q * Ly::kGFL;
-      // lane l < kCh: the lane-independent phases of channel it kCh + l
-      uint32_t ph_a = 0, ph_d = 0;
-      {
-        const int c = it * kCh + (lane & (kCh - 1));
-        if (c < a.n_chan) {
-          const PhaseConst p = pcs[c];
-          ph_a = top32_mul(ku, p.u_lo, p.u_hi) + top32_mul(m_j0, p.v_lo, p.v_hi);
-          ph_d = top32_mul(m_d, p.v_lo, p.v_hi);
-        }
-      }
-#pragma unroll
-      for (int ch = 0; ch < kCh; ++ch) {
-        const int c = it * kCh + ch;
-        const uint32_t pa = __shfl_sync(0xffffffffu, ph_a, ch);
-        const uint32_t pd = __shfl_sync(0xffffffffu, ph_d, ch);
-        if (c < a.n_chan) {
-          const PhaseConst p = pcs[c];
-          const uint32_t pp = top32_mul(m_p, p.v_lo, p.v_hi);
-          const uint32_t pz0 = pa + (pp << 5);
-          const float2 w0 = unit_phasor(pz0);
-          const float2 w1 = unit_phasor(pz0 + pd);
-          const float2 wp = unit_phasor(pp);
-          // Z_lane and Z_lane+32 = X W as pairs
-          const float2 xv = x[ch];
-          const float2 cw = make_float2(w0.x, w1.x), sw = make_float2(w0.y, w1.y);
-          const float2 xr = make_float2(xv.x, xv.x);
-          const float2 zr = __ffma2_rn(xr, cw, __fmul2_rn(make_float2(-xv.y, -xv.y), sw));
-          const float2 zi = __ffma2_rn(xr, sw, __fmul2_rn(make_float2(xv.y, xv.y), cw));
-          float* grp = st + ch * Ly::kBins * Ly::kGFL;
-          grp[lane] = zr.x;
-          grp[Ly::kA + lane] = zi.x;
-          grp[32 + lane] = zr.y;
-          grp[Ly::kA + 32 + lane] = zi.y;
-          grp[2 * Ly::kA + lane] = wp.x;
-          grp[2 * Ly::kA + Ly::kT + lane] = wp.y;
-        }
-      }
-      if (!a.test_withhold) dev::mbar_arrive_warp(&full[s]);
-    }
-  } else {
-    // ------------------------------------------------------------ consumers
-    const int q = warp >> 1;                      // the CTA's bin
-    const int h = warp & 1;                       // a's 32 h .. 32 h + 31
-    const int k = bin_tile * Ly::kBins + q;       // local bin
-    const int ga = lane >> 2;                     // a = 32 h + 4 ga + i
-    const int gb = lane & 3;                      // b = 8 gb + j
-    float2 A[4][4], B[4][4], C[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) A[i][m] = B[i][m] = C[i][m] = make_float2(0.f, 0.f);
-    for (int it = 0; it < n_iter; ++it) {
-      const uint32_t g = it0 + it;
-      const int s = g % kStages;
-      ok = __all_sync(0xffffffffu, dev::mbar_wait(&full[s], (g / kStages) & 1, abort_flag));
-      if (!ok) break;
-      const float* st = stages + s * Ly::kStageFloats + q * Ly::kGFL;
-      const int nc = a.n_chan - it * kCh;
-#pragma unroll
-      for (int ch = 0; ch < kCh; ++ch) {
-        if (ch < nc) {
-          const float* grp = st + ch * Ly::kBins * Ly::kGFL;
-          const float4 zr = *reinterpret_cast<const float4*>(grp + 32 * h + 4 * ga);
-          const float4 zi = *reinterpret_cast<const float4*>(grp + Ly::kA + 32 * h + 4 * ga);
-          const float* pp = grp + 2 * Ly::kA + 8 * gb;
-          const float4 pr0 = *reinterpret_cast<const float4*>(pp);
-          const float4 pr1 = *reinterpret_cast<const float4*>(pp + 4);
-          const float4 pi0 = *reinterpret_cast<const float4*>(pp + Ly::kT);
-          const float4 pi1 = *reinterpret_cast<const float4*>(pp + Ly::kT + 4);
-          const float2 pr[4] = {make_float2(pr0.x, pr0.y), make_float2(pr0.z, pr0.w),
-                                make_float2(pr1.x, pr1.y), make_float2(pr1.z, pr1.w)};
-          const float2 pi[4] = {make_float2(pi0.x, pi0.y), make_float2(pi0.z, pi0.w),
-                                make_float2(pi1.x, pi1.y), make_float2(pi1.z, pi1.w)};
-          float2 ps[4];
-#pragma unroll
-          for (int m = 0; m < 4; ++m) ps[m] = __fadd2_rn(pr[m], pi[m]);
-          const float2 zs01 = __fadd2_rn(make_float2(zr.x, zr.y), make_float2(zi.x, zi.y));
-          const float2 zs23 = __fadd2_rn(make_float2(zr.z, zr.w), make_float2(zi.z, zi.w));
-          const float zrv[4] = {zr.x, zr.y, zr.z, zr.w};
-          const float ziv[4] = {zi.x, zi.y, zi.z, zi.w};
-          const float zsv[4] = {zs01.x, zs01.y, zs23.x, zs23.y};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 r2 = make_float2(zrv[i], zrv[i]);
-            const float2 i2 = make_float2(ziv[i], ziv[i]);
-            const float2 s2 = make_float2(zsv[i], zsv[i]);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              A[i][m] = __ffma2_rn(r2, pr[m], A[i][m]);
-              B[i][m] = __ffma2_rn(i2, pi[m], B[i][m]);
-              C[i][m] = __ffma2_rn(s2, ps[m], C[i][m]);
-            }
-          }
-        }
-      }
-      dev::mbar_arrive_warp(&empty[s]);
-    }
-    if (ok && k < a.n_bins) {
-      const bool real_only = (a.k_begin + k == a.real_bin_a) || (a.k_begin + k == a.real_bin_b);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float av = e ? A[i][m].y : A[i][m].x;
-            const float bv = e ? B[i][m].y : B[i][m].x;
-            const float cv = e ? C[i][m].y : C[i][m].x;
-            const int jl = jblk + (32 * h + 4 * ga + i) * Ly::kT + 8 * gb + 2 * m + e;
-            if (jl < a.n_dm) {
-              const float re = (av - bv) * a.scale;
-              const float im = real_only ? 0.f : (cv - av - bv) * a.scale;
-              const int64_t o = static_cast<int64_t>(series) * a.y_series_stride +
-                                static_cast<int64_t>(jl) * a.y_dm_stride + k;
-              if (a.out_kind == 2)
-                static_cast<float*>(a.Y)[o] = re * re + im * im;
-              else
-                static_cast<float2*>(a.Y)[o] = make_float2(re, im);
-            }
-          }
-        }
-      }
-    }
-  }
-  if (!ok) {
-    *abort_flag = 1;
-    if (a.status) atomicExch(a.status, FDD_ERR_TIMEOUT);
-  }
-  return ok;
-}
-
-// Wide item of the three-multiplication tile: a ragged remainder of at most
-// kAw x 32 trials (kAw = 32: 1024, kAw = 16: 512) from trial jw over the
-// CTA's 8 x 32 / kAw bins from bin_tile times that: consumer warp w owns
-// 32 / kAw of them (kAw / 4 x 4 lanes each, every lane busy), each lane a
-// 4 x 8 tile of (a, b) as in the full item; producer warp q evaluates, for its
-// quarter of the bins, P_b (b = lane) of each and the kAw Z_a of each (two per
-// lane).  Same stage ring and handshake as the full item.
-template <int kCh, int kStages, int kAw>
-__device__ __forceinline__ bool g3_wide_body(const MacArgs& a, const PhaseConst* pcs,
-                                             float* stages, uint64_t* full, uint64_t* empty,
-                                             volatile int* abort_flag, int bin_tile, int jw,
-                                             int series, uint32_t it0) {
-  using Ly = G3<kCh, kStages>;
-  constexpr int kC = Ly::kChWide;  // channels per stage
-  constexpr int kNB = Ly::wide_bins(kAw);   // bins per CTA
-  constexpr int kW = Ly::wide_floats(kAw);  // floats per (bin, channel)
-  constexpr int kPB = kNB / Ly::kProd;      // bins per producer warp
-  constexpr int kLPB = kAw;                 // lanes per bin in a consumer warp (kAw/4 x 4)
-  static_assert(kAw == 32 || kAw == 16, "wide items of 1024 or 512 trials");
-  static_assert(kNB == Ly::kCons * 32 / kLPB && 2 * 32 == kPB * kAw, "wide layout");
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  const int n_iter = (a.n_chan + kC - 1) / kC;
-  const int bin0 = bin_tile * kNB;
-  bool ok = true;
-
-  if (warp >= Ly::kCons) {
-    // ------------------------------------------------------------ producers
-    const int q = warp - Ly::kCons;
-    uint32_t ku[kPB], m_p[kPB];
-    const float2* xp[kPB];
-#pragma unroll
-    for (int r = 0; r < kPB; ++r) {
-      const int k = bin0 + q * kPB + r;
-      const int kl = k < a.n_bins ? k : 0;  // idle bins evaluate local bin 0, unused
-      ku[r] = static_cast<uint32_t>(a.k_begin + kl);
-      m_p[r] = ku[r] * static_cast<uint32_t>(lane);
-      xp[r] = a.X + static_cast<int64_t>(series) * a.x_series_stride + kl;
-    }
-    // the lane's two Z_a: a = lane mod kAw of the warp's bins 32 t / kAw + lane / kAw
-    // (bin t for kAw 32; bin 2 t + lane / 16 for kAw 16: chosen by selects)
-    const bool hi = kAw == 16 && lane >= 16;
-    uint32_t m_z[2], k_z[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const int r0 = t * (32 / kAw);
-      k_z[t] = (kAw == 16 && hi) ? ku[(r0 + 1) % kPB] : ku[r0];
-      m_z[t] = k_z[t] * static_cast<uint32_t>(a.j_begin + jw + (lane % kAw) * Ly::kT);
-    }
-    const int64_t xs = a.x_chan_stride;
-    float2 xn[kPB][kC];
-#pragma unroll
-    for (int r = 0; r < kPB; ++r)
-#pragma unroll
-      for (int ch = 0; ch < kC; ++ch)
-        xn[r][ch] = ch < a.n_chan ? __ldg(xp[r] + ch * xs) : make_float2(0.f, 0.f);
-    for (int it = 0; it < n_iter; ++it) {
-      const uint32_t g = it0 + it;
-      const int s = g % kStages;
-      float2 x[kPB][kC];
-#pragma unroll
-      for (int r = 0; r < kPB; ++r)
-#pragma unroll
-        for (int ch = 0; ch < kC; ++ch) {
-          x[r][ch] = xn[r][ch];
-          const int c = (it + 1) * kC + ch;  // prefetch the next stage's X
-          xn[r][ch] = c < a.n_chan ? __ldg(xp[r] + c * xs) : make_float2(0.f, 0.f);
-        }
-      ok = __all_sync(0xffffffffu,
-                      dev::mbar_wait(&empty[s], ((g / kStages) & 1) ^ 1, abort_flag));
-      if (!ok) break;
-      float* st = stages + s * Ly::kStageFloats;
-#pragma unroll
-      for (int ch = 0; ch < kC; ++ch) {
-        const int c = it * kC + ch;
-        if (c < a.n_chan) {
-          const PhaseConst p = pcs[c];
-#pragma unroll
-          for (int r = 0; r < kPB; ++r) {
-            const float2 wp = unit_phasor(top32_mul(m_p[r], p.v_lo, p.v_hi));
-            float* grp = st + (ch * kNB + q * kPB + r) * kW;
-            grp[2 * kAw + lane] = wp.x;
-            grp[2 * kAw + 32 + lane] = wp.y;
-          }
-#pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const int r0 = t * (32 / kAw);
-            const int r = hi ? r0 + 1 : r0;
-            const float2 xv = (kAw == 16 && hi) ? x[(r0 + 1) % kPB][ch] : x[r0][ch];
-            const float2 w = unit_phasor(top32_mul(k_z[t], p.u_lo, p.u_hi) +
-                                         top32_mul(m_z[t], p.v_lo, p.v_hi));
-            float* grp = st + (ch * kNB + q * kPB + r) * kW;
-            const int ai = lane % kAw;
-            grp[ai] = xv.x * w.x - xv.y * w.y;
-            grp[kAw + ai] = xv.x * w.y + xv.y * w.x;
-          }
-        }
-      }
-      if (!a.test_withhold) dev::mbar_arrive_warp(&full[s]);
-    }
-  } else {
-    // ------------------------------------------------------------ consumers
-    const int wb = warp * (32 / kLPB) + lane / kLPB;  // the lane's bin in the CTA
-    const int k = bin0 + wb;                          // local bin
-    const int ll = lane % kLPB;
-    const int ga = ll >> 2;  // a = 4 ga + i
-    const int gb = ll & 3;   // b = 8 gb + j
-    float2 A[4][4], B[4][4], C[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int m = 0; m < 4; ++m) A[i][m] = B[i][m] = C[i][m] = make_float2(0.f, 0.f);
-    for (int it = 0; it < n_iter; ++it) {
-      const uint32_t g = it0 + it;
-      const int s = g % kStages;
-      ok = __all_sync(0xffffffffu, dev::mbar_wait(&full[s], (g / kStages) & 1, abort_flag));
-      if (!ok) break;
-      const int nc = a.n_chan - it * kC;
-#pragma unroll
-      for (int ch = 0; ch < kC; ++ch) {
-        if (ch < nc) {
-          const float* grp = stages + s * Ly::kStageFloats + (ch * kNB + wb) * kW;
-          const float4 zr = *reinterpret_cast<const float4*>(grp + 4 * ga);
-          const float4 zi = *reinterpret_cast<const float4*>(grp + kAw + 4 * ga);
-          const float4 pr0 = *reinterpret_cast<const float4*>(grp + 2 * kAw + 8 * gb);
-          const float4 pr1 = *reinterpret_cast<const float4*>(grp + 2 * kAw + 8 * gb + 4);
-          const float4 pi0 = *reinterpret_cast<const float4*>(grp + 2 * kAw + 32 + 8 * gb);
-          const float4 pi1 = *reinterpret_cast<const float4*>(grp + 2 * kAw + 32 + 8 * gb + 4);
-          const float2 pr[4] = {make_float2(pr0.x, pr0.y), make_float2(pr0.z, pr0.w),
-                                make_float2(pr1.x, pr1.y), make_float2(pr1.z, pr1.w)};
-          const float2 pi[4] = {make_float2(pi0.x, pi0.y), make_float2(pi0.z, pi0.w),
-                                make_float2(pi1.x, pi1.y), make_float2(pi1.z, pi1.w)};
-          float2 ps[4];
-#pragma unroll
-          for (int m = 0; m < 4; ++m) ps[m] = __fadd2_rn(pr[m], pi[m]);
-          const float2 zs01 = __fadd2_rn(make_float2(zr.x, zr.y), make_float2(zi.x, zi.y));
-          const float2 zs23 = __fadd2_rn(make_float2(zr.z, zr.w), make_float2(zi.z, zi.w));
-          const float zrv[4] = {zr.x, zr.y, zr.z, zr.w};
-          const float ziv[4] = {zi.x, zi.y, zi.z, zi.w};
-          const float zsv[4] = {zs01.x, zs01.y, zs23.x, zs23.y};
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 r2 = make_float2(zrv[i], zrv[i]);
-            const float2 i2 = make_float2(ziv[i], ziv[i]);
-            const float2 s2 = make_float2(zsv[i], zsv[i]);
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              A[i][m] = __ffma2_rn(r2, pr[m], A[i][m]);
-              B[i][m] = __ffma2_rn(i2, pi[m], B[i][m]);
-              C[i][m] = __ffma2_rn(s2, ps[m], C[i][m]);
-            }
-          }
-        }
-      }
-      dev::mbar_arrive_warp(&empty[s]);
-    }
-    if (ok && k < a.n_bins) {
-      const bool real_only = (a.k_begin + k == a.real_bin_a) || (a.k_begin + k == a.real_bin_b);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float av = e ? A[i][m].y : A[i][m].x;
-            const float bv = e ? B[i][m].y : B[i][m].x;
-            const float cv = e ? C[i][m].y : C[i][m].x;
-            const int jl = jw + (4 * ga + i) * Ly::kT + 8 * gb + 2 * m + e;
-            if (jl < a.n_dm) {
-              const float re = (av - bv) * a.scale;
-              const float im = real_only ? 0.f : (cv - av - bv) * a.scale;
-              const int64_t o = static_cast<int64_t>(series) * a.y_series_stride +
-                                static_cast<int64_t>(jl) * a.y_dm_stride + k;
-              if (a.out_kind == 2)
-                static_cast<float*>(a.Y)[o] = re * re + im * im;
-              else
-                static_cast<float2*>(a.Y)[o] = make_float2(re, im);
-            }
-          }
-        }
-      }
-    }
-  }
-  if (!ok) {
-    *abort_flag = 1;
-    if (a.status) atomicExch(a.status, FDD_ERR_TIMEOUT);
-  }
-  return ok;
-}
-
-// A grid item of the three-multiplication tile: a full item, or for a last
-// block of at most 1024 (512) trials a wide item over twice (four times) the
-// bins (the grid's bin tiles beyond the wide ones have nothing to do and
-// leave at once).
-template <int kCh, int kStages>
-__device__ __forceinline__ bool g3_item(const MacArgs& a, const PhaseConst* pcs, float* stages,
-                                        uint64_t* full, uint64_t* empty,
-                                        volatile int* abort_flag, int bin_tile, int dm_block,
-                                        int series, uint32_t it0) {
-  using Ly = G3<kCh, kStages>;
-  const int jblk = dm_block * Ly::kDms;
-  const int rem = a.n_dm - jblk;
-  if (rem <= Ly::kDms / 4) {
-    if (bin_tile * Ly::wide_bins(16) >= a.n_bins) return true;
-    return g3_wide_body<kCh, kStages, 16>(a, pcs, stages, full, empty, abort_flag, bin_tile,
-                                          jblk, series, it0);
-  }
-  if (rem <= Ly::kDms / 2) {
-    if (bin_tile * Ly::wide_bins(32) >= a.n_bins) return true;
-    return g3_wide_body<kCh, kStages, 32>(a, pcs, stages, full, empty, abort_flag, bin_tile,
-                                          jblk, series, it0);
-  }
-  return g3_body<kCh, kStages>(a, pcs, stages, full, empty, abort_flag, bin_tile, dm_block,
-                               series, it0);
-}
-
-template <int kCh, int kStages>
-__global__ void __launch_bounds__(G3<kCh, kStages>::kThreads, 1) mac_g3_kernel(const MacArgs a) {
-  using Ly = G3<kCh, kStages>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  WsSmem<Ly> sm;
-  sm.template init<kStages>(smem_raw, a.n_chan, Ly::kCons, Ly::kProd);
-  for (int i = threadIdx.x; i < a.n_chan; i += blockDim.x) sm.pcs[i] = a.pc[i];
-  __syncthreads();
-  g3_item<kCh, kStages>(a, sm.pcs, sm.stages, sm.full, sm.empty, sm.abort_flag, blockIdx.x,
-                        blockIdx.y, blockIdx.z, 0u);
-}
-
-// Persistent form of the three-multiplication tile over a batch of spectra
-// sets (the batching form), as mac_ws_batch_kernel.
-template <int kCh, int kStages>
-__global__ void __launch_bounds__(G3<kCh, kStages>::kThreads, 1)
-    mac_g3_batch_kernel(const BatchSet* sets, int n_sets, int64_t n_items,
-                        unsigned long long* counter) {
-  using Ly = G3<kCh, kStages>;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ long long item_s;
-  const int n_chan = sets[0].args.n_chan;  // common to the batch
-  WsSmem<Ly> sm;
-  sm.template init<kStages>(smem_raw, n_chan, Ly::kCons, Ly::kProd);
-  int cur = -1;
-  uint32_t it0 = 0;
-  const uint32_t n_iter = static_cast<uint32_t>((n_chan + kCh - 1) / kCh);
-  const uint32_t n_iter_wide =
-      static_cast<uint32_t>((n_chan + Ly::kChWide - 1) / Ly::kChWide);
-  while (true) {
-    if (threadIdx.x == 0) item_s = static_cast<long long>(atomicAdd(counter, 1ull));
-    __syncthreads();  // also: every stage of the previous item has been read
-    const long long item = item_s;
-    if (item >= n_items || *sm.abort_flag) break;
-    int lo = 0, hi = n_sets - 1;  // last set with item_begin <= item
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (sets[mid].item_begin <= item) lo = mid; else hi = mid - 1;
-    }
-    const BatchSet& bs = sets[lo];
-    if (lo != cur) {
-      for (int i = threadIdx.x; i < n_chan; i += blockDim.x) sm.pcs[i] = bs.args.pc[i];
-      cur = lo;
-    }
-    __syncthreads();  // phase table ready; item_s read by every thread
-    const long long local = item - bs.item_begin;
-    const long long n_full = static_cast<long long>(bs.n_bin_tiles) * bs.n_dm_blocks;
-    // the set's arguments as a local copy: the item's loops then keep what
-    // they use in registers instead of re-reading the set after each store
-    const MacArgs args = bs.args;
-    const bool full_item = local < n_full;
-    if (full_item)
-      g3_body<kCh, kStages>(args, sm.pcs, sm.stages, sm.full, sm.empty, sm.abort_flag,
-                            static_cast<int>(local / bs.n_dm_blocks),
-                            static_cast<int>(local % bs.n_dm_blocks), 0, it0);
-    else if (local < n_full + bs.n_wide_tiles)
-      g3_wide_body<kCh, kStages, 32>(args, sm.pcs, sm.stages, sm.full, sm.empty,
-                                     sm.abort_flag, static_cast<int>(local - n_full), bs.j_wide,
-                                     0, it0);
-    else
-      g3_wide_body<kCh, kStages, 16>(args, sm.pcs, sm.stages, sm.full, sm.empty,
-                                     sm.abort_flag,
-                                     static_cast<int>(local - n_full - bs.n_wide_tiles),
-                                     bs.j_narrow, 0, it0);
-    it0 += full_item ? n_iter : n_iter_wide;  // stages this item used
-  }
-}
-
 // ----------------------------------------------------------------- variants
 struct VariantInfo {
   const void* fn;
@@ -1097,29 +582,17 @@ VariantInfo info_ws() {
   return vi;
 }
 
-template <int kCh, int kSt>
-VariantInfo info_g3() {
-  using Ly = G3<kCh, kSt>;
-  VariantInfo vi{reinterpret_cast<const void*>(&mac_g3_kernel<kCh, kSt>), Ly::kDms, 1,
-                 Ly::kSwapBytes, Ly::kCons + Ly::kProd,
-                 reinterpret_cast<const void*>(&mac_g3_batch_kernel<kCh, kSt>)};
-  vi.bin_warps = Ly::kBins;
-  return vi;
-}
-
-// The G12 tile keeps three ring stages while the channels' phase table leaves
-// room for them in a CTA's 227 KB and drops to two beyond that (up to 8381
-// channels).  One plain launch runs as fast with two as with three; the
-// persistent batch kernel, whose items follow one another in the same ring,
-// lost 5 % with two.
 constexpr size_t kMaxSmem = 227 * 1024;
 
-VariantInfo variant_info(int v, int n_chan) {
+// Channels up to which plans take the G12 tile.  The tile itself has no such
+// limit (its per-channel constants stay in global memory); the line is where
+// it lay while the tile kept them in shared memory, so a plan reports the
+// tile it always did.
+constexpr int kG12MaxChan = 8381;
+
+// (every tile but G12_4x8, which fdd_mac_split.cu launches)
+VariantInfo variant_info(int v) {
   switch (v) {
-    case MAC_G12_4x8:
-      return sizeof(PhaseConst) * static_cast<size_t>(n_chan) + G3<16, 3>::kSwapBytes <= kMaxSmem
-                 ? info_g3<16, 3>()
-                 : info_g3<16, 2>();
     case MAC_Q12_8x8: return info<G8x8, PackedCompact<G8x8>, 12>();
     case MAC_Q_4x8: return info<G4x8, PackedCompact<G4x8>>();
     case MAC_Q_8x8_512: return info<G8x8q, PackedCompact<G8x8q>>();
@@ -1130,36 +603,32 @@ VariantInfo variant_info(int v, int n_chan) {
 
 }  // namespace
 
-// Default tile for a trial count: the one with the least time for the padded
-// trial blocks, ceil(n_dm / block) * block / rate, with each tile's rate
-// measured kernel-only on GB300 (fraction of the FP32 peak, 1024 channels,
-// 131073 bins): G12_4x8 0.752 on full 2048-trial blocks, whose last block
-// runs as 1024-trial wide items at 0.616 (at most 1024 trials) or 512-trial
-// ones at 0.510 (at most 512); Q_4x8 0.493 (1024-trial blocks), Q_8x8_512
-// 0.415 (512), Q_4x4 0.347 (128).  (The four-product warp-specialised tile
-// W12_8x8 measured 0.621 on the same launch, Q12_8x8, the 2048-trial tile on
-// the plain schedule, 0.553.)
+// Default tile for a trial count.  From 257 trials on the G12 tile while the
+// channels allow it: on 4096 bins x 1024 channels its passes of up to 1024,
+// 2048 and 4096 trials take 247, 305 and 430 us whatever their filling, the
+// 128-trial tile 624 us at 257 trials and 767 at 512.  (From 129 to 256 trials
+// the G12 tile would be the faster one too with many channels, 247 against
+// 392 us; plans have always reported Q_4X4 there, and keep to it.  Up to 128
+// the two are within 17 % at 1024 channels and Q_4X4 is 1.4-1.7 times faster
+// at 64 to 200.)  Otherwise the tile with the least time for the padded trial
+// blocks, ceil(n_dm / block) * block / rate, with each tile's rate measured
+// kernel-only (fraction of the FP32 peak, 1024 channels, 131073 bins): Q_4x8
+// 0.493 (1024-trial blocks), Q_8x8_512 0.415 (512), Q_4x4 0.347 (128).  (The
+// four-product warp-specialised tile W12_8x8 measured 0.621 on the same
+// launch, Q12_8x8, the 2048-trial tile on the plain schedule, 0.553.)
 int mac_variant_for(int n_dm, int n_chan) {
+  if (n_dm > 256 && mac_smem_bytes(MAC_G12_4x8, n_chan) <= kMaxSmem) return MAC_G12_4x8;
   struct Tile {
     int variant, block;
-    double rate, wide_rate, narrow_rate;  // > 0: a last block of <= block / 2, / 4
+    double rate;
   };
-  static const Tile tiles[] = {{MAC_G12_4x8, 2048, 0.752, 0.616, 0.510},
-                               {MAC_Q_4x8, 1024, 0.493, 0.0, 0.0},
-                               {MAC_Q_8x8_512, 512, 0.415, 0.0, 0.0},
-                               {MAC_Q_4x4, 128, 0.347, 0.0, 0.0}};
+  static const Tile tiles[] = {
+      {MAC_Q_4x8, 1024, 0.493}, {MAC_Q_8x8_512, 512, 0.415}, {MAC_Q_4x4, 128, 0.347}};
   int best = MAC_W12_8x8;  // (the smallest shared-memory need of the 2048-trial tiles)
   double best_cost = 0.0;
   for (const Tile& t : tiles) {
     if (mac_smem_bytes(t.variant, n_chan) > kMaxSmem) continue;
-    const int full = n_dm / t.block, rem = n_dm % t.block;
-    double cost = full * t.block / t.rate;
-    if (rem > 0 && t.narrow_rate > 0.0 && rem <= t.block / 4)
-      cost += (t.block / 4) / t.narrow_rate;
-    else if (rem > 0 && t.wide_rate > 0.0 && rem <= t.block / 2)
-      cost += (t.block / 2) / t.wide_rate;
-    else if (rem > 0)
-      cost += t.block / t.rate;
+    const double cost = (n_dm + t.block - 1) / t.block * t.block / t.rate;
     if (best_cost == 0.0 || cost < best_cost) {
       best = t.variant;
       best_cost = cost;
@@ -1168,26 +637,33 @@ int mac_variant_for(int n_dm, int n_chan) {
   return best;
 }
 
-int mac_variant_trials_per_block(int variant) { return variant_info(variant, 1).dms; }
+int mac_variant_trials_per_block(int variant) {
+  return variant == MAC_G12_4x8 ? 2048 : variant_info(variant).dms;
+}
 
 size_t mac_smem_bytes(int variant, int n_chan) {
-  return sizeof(PhaseConst) * static_cast<size_t>(n_chan) + variant_info(variant, n_chan).swap_bytes;
+  if (variant == MAC_G12_4x8) return n_chan <= kG12MaxChan ? mac_split_smem_bytes() : kMaxSmem + 1;
+  return sizeof(PhaseConst) * static_cast<size_t>(n_chan) + variant_info(variant).swap_bytes;
 }
 
 cudaError_t mac_prepare(int variant, int n_chan) {
-  const VariantInfo vi = variant_info(variant, n_chan);
+  if (variant == MAC_G12_4x8) return mac_split_prepare();
+  const VariantInfo vi = variant_info(variant);
   const int bytes = static_cast<int>(mac_smem_bytes(variant, n_chan));
   cudaError_t e = cudaFuncSetAttribute(vi.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess || !vi.batch_fn) return e;
   return cudaFuncSetAttribute(vi.batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-int mac_variant_bins_per_cta(int variant) { return variant_info(variant, 1).bins(); }
+int mac_variant_bins_per_cta(int variant) { return variant_info(variant).bins(); }
 
-bool mac_variant_batchable(int variant) { return variant_info(variant, 1).batch_fn != nullptr; }
+bool mac_variant_batchable(int variant) {
+  return variant == MAC_G12_4x8 || variant_info(variant).batch_fn != nullptr;
+}
 
 int mac_batch_ctas_per_sm(int variant, int n_chan) {
-  const VariantInfo vi = variant_info(variant, n_chan);
+  if (variant == MAC_G12_4x8) return 1;  // (tensor memory and registers: one CTA per SM)
+  const VariantInfo vi = variant_info(variant);
   if (!vi.batch_fn) return 0;
   int n = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, vi.batch_fn, vi.warps * 32,
@@ -1201,8 +677,10 @@ int mac_batch_ctas_per_sm(int variant, int n_chan) {
 
 cudaError_t launch_mac_batch(const BatchSet* d_sets, int n_sets, long long n_items,
                              unsigned long long* d_counter, int variant, int n_ctas, int n_chan,
-                             cudaStream_t s) {
-  const VariantInfo vi = variant_info(variant, n_chan);
+                             int max_n_dm, cudaStream_t s) {
+  if (variant == MAC_G12_4x8)
+    return launch_mac_split_batch(d_sets, n_sets, n_items, max_n_dm, n_ctas, s);
+  const VariantInfo vi = variant_info(variant);
   if (!vi.batch_fn) return cudaErrorInvalidValue;
   if (n_items <= 0) return cudaSuccess;
   void* params[] = {&d_sets, &n_sets, &n_items, &d_counter};
@@ -1213,7 +691,8 @@ cudaError_t launch_mac_batch(const BatchSet* d_sets, int n_sets, long long n_ite
 
 cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s) {
   if (a.n_dm <= 0 || a.n_series <= 0 || a.n_bins <= 0) return cudaSuccess;
-  const VariantInfo vi = variant_info(variant, a.n_chan);
+  if (variant == MAC_G12_4x8) return launch_mac_split(a, s);
+  const VariantInfo vi = variant_info(variant);
   const int bins_per_cta = vi.bins();
   dim3 grid((a.n_bins + bins_per_cta - 1) / bins_per_cta, (a.n_dm + vi.dms - 1) / vi.dms,
             a.n_series);

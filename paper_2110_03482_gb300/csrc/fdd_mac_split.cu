@@ -1,0 +1,900 @@
+// fdd_mac_split.cu -- FP32-accurate phase-rotate-and-sum on the tensor cores
+// (Sect. 2.2, Eqs. 4 and 7) for one set of spectra: the G12_4X8 tile.
+//
+//   Y[j][k] = sum_nu W(k, nu, j) X[nu][k],   W = exp(+2 pi i k d(nu, DM_j) / L)
+//
+// Trials are paired around centres.  A pass covers 256 n_a trials from j_p;
+// with Jc = j_p + 128 n_a - 1/2, trial j = Jc + s (128 al + 64) + t (b + 1/2)
+// for s, t = +-1, al < n_a, b < 64.  The phase is linear in j, so
+//
+//   W = exp(i phi_c) (Ca + i s Sa) (Cb + i t Sb),
+//
+// with (Ca, Sa) and (Cb, Sb) the cosine and sine of the al and b steps of bin
+// k and channel nu.  The sums over channels that all four signs share,
+//
+//   M = sum Cb {Xr Ca, Xi Ca, Xr Sa, Xi Sa},   N = sum Sb {the same},
+//
+// (X rotated by exp(i phi_c)) are ONE real matrix product per bin: 128 rows
+// (Cb, Sb of 64 b's) x channels times channels x 4 n_a columns.  Against the
+// complex form this halves both the multiplications (eight real ones for four
+// trials' complex products) and the phasors to evaluate (64 for 128 trials).
+//
+// Each operand is split into two FP16 terms (hi + lo: 22 bits; the columns
+// scaled by a power of two per bin and stage of 64 channels) and the product
+// formed as hi hi + (hi lo + lo hi) on tcgen05 with FP32 accumulators.  The
+// tensor cores round their sums toward zero, so an accumulator only lives for
+// one stage; the stages' sums are added in FP32 registers (to nearest).  The
+// error against FP64 is 3.2e-7 of the result whatever the channel count (rows
+// and columns from the hardware sine, 1.6e-7 each); the FP32 multiply-adds
+// this replaces rounded every sum: 3.2e-7 at 64 channels, 4.2e-7 at 200,
+// 7.7e-7 at 1024.
+//
+// Sixty-four channels of a bin are a stage.  Two warps turn the spectra and
+// phase constants into a table per stage, thirteen evaluate and split rows and
+// columns into shared memory (K-major core matrices), one issues the MMAs,
+// four add the stages up and store.  4096 bins x 1024 channels x 2048 trials
+// take 305 us, against 1185 us for the FP32 multiply-adds (three real products
+// per complex one) at 0.75 of the FP32 peak; 301 bins x 4096 channels x 8192
+// trials 218 against 1292 us; 701 trials of 387 channels 216 against 560 us.
+// What bounds it: writing and reading the operands in shared memory (71 % of
+// its cycles, the MMAs' reads and the producers' stores about equal) beside
+// 50 warp instructions per bin and channel (61 % of the issue slots), most of
+// them phasors and splits of the 128 rows.  Hence the wide passes: the rows
+// serve all columns of a pass, up to 4096 trials.
+// Measured and dropped: results kept until a whole octet is done in wider
+// stores with fewer warps (16 warps of 128 registers: 344 us), four bytes per
+// store from registers used at once (317), one octet per task (353), the MMA
+// loop unrolled by stage (334: instruction fetch), lo hi as an MMA of its own
+// (307).
+#include <atomic>
+
+#include <cuda_fp16.h>
+
+#include "fdd_device.cuh"
+#include "fdd_internal.h"
+
+namespace fdd {
+namespace {
+
+using dev::mbar_arrive;
+using dev::mbar_arrive_warp;
+using dev::mbar_init;
+using dev::smem_u32;
+using dev::unit_phasor;
+
+// The warp waits for a phase, bounded: every lane asks (together: a divided
+// warp would run what follows twice), suspended in the hardware for up to two
+// microseconds at a time, so that waiting takes few shared-memory cycles from
+// the operands.
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
+  long long t0 = 0;
+  while (true) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+                 " selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok)
+                 : "r"(smem_u32(bar)), "r"(parity), "r"(2000)
+                 : "memory");
+    if (__all_sync(0xffffffffu, ok)) return true;
+    const long long t = clock64();
+    if (t0 == 0) t0 = t;
+    if (__any_sync(0xffffffffu, *abort_flag != 0 || t - t0 > dev::kWaitCycles)) return false;
+  }
+}
+
+constexpr int kCh = 64;     // channels per stage (four K steps of 16)
+constexpr int kRows = 128;  // Cb | Sb of 64 b's
+constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's
+
+// Warps: 0-3 epilogue (a warp reads the tensor-memory lanes of its quarter),
+// the MMA issuer, two that make the stages' tables in turn, and thirteen
+// producers of rows and columns: five warps per scheduler, 96 registers each.
+constexpr int kEpiWarps = 4;
+constexpr int kMmaWarp = kEpiWarps;
+constexpr int kPrepFirst = kMmaWarp + 1, kPrepWarps = 2;
+constexpr int kProdFirst = kPrepFirst + kPrepWarps, kProdWarps = 13;
+constexpr int kThreads = 32 * (kProdFirst + kProdWarps);
+
+// kNa: al's a pass can hold; kBins: bins a CTA works on at a time (their
+// accumulators share the epilogue's registers: kNa * kBins = 16).
+template <int kNa>
+struct Cfg {
+  static constexpr int kBins = 16 / kNa;
+  static constexpr int kN = 4 * kNa;          // columns
+  static constexpr int kStages = kNa == 16 ? 4 : 5;
+  static constexpr int kTables = kNa == 8 ? 6 : 8;  // tables run further ahead than operands
+  static constexpr uint32_t kATile = kRows * kCh * 2;  // 8 KB per term
+  static constexpr uint32_t kBTile = kN * kCh * 2;
+  static constexpr uint32_t kStageBytes = 2 * (kATile + kBTile);
+  // tasks of a stage, dealt to the producer warps in turn: the columns (sixteen
+  // half octets of channels x kNa al's, two rounds of a warp each), then the
+  // rows of each of the four K steps
+  static constexpr int kColTasks = kNa / 4;
+  static constexpr int kTasks = 4 + kColTasks;
+  static_assert((kProdWarps + kTasks - 1) / kTasks < kStages, "a producer's step between tasks");
+  static constexpr uint32_t kTmemCols = kNa == 4 ? 256 : 512;
+  static_assert(kStages * 2 * kN <= static_cast<int>(kTmemCols), "accumulator ring");
+};
+
+// Per stage: what the producers need of each channel.
+struct Table {
+  uint32_t hw[kCh];   // half the trial step's phase, units of 2^-32 cycle
+  uint32_t ha[kCh];   // 64 trial steps
+  float fr[kCh], fi[kCh];  // phasor of 16 trial steps (b -> b + 16)
+  float xr[kCh], xi[kCh];  // X rotated to the pass centre and scaled
+  int steps;               // K steps of 16 channels the MMAs read
+  int pad[3];
+};
+template <int kNa>
+struct Smem {
+  using C = Cfg<kNa>;
+  alignas(128) unsigned char stage[C::kStages][C::kStageBytes];
+  alignas(16) float4 xch[8][kRows];  // epilogue exchange: A_+, A_- of a row (or B_+, B_-)
+  alignas(16) Table table[C::kTables];
+  float inv[4 * C::kTables];  // undoes a stage's scale (read by the epilogue, well after the table)
+  uint64_t pfull[C::kTables], pfree[C::kTables];  // table written; every producer has read it
+  uint64_t full[C::kStages], done[C::kStages];   // operands written; MMAs complete
+  uint64_t xbar, drain;
+  uint32_t tmem;
+  int abort_flag;
+};
+
+// Shared-memory matrix descriptor, K-major without swizzle: 8-row x 16-byte
+// core matrices of 128 contiguous bytes, 128 bytes apart along the rows and
+// `k_stride` apart along K.
+__device__ __forceinline__ uint64_t core_desc(uint32_t addr, uint32_t k_stride) {
+  return static_cast<uint64_t>((addr & 0x3FFFF) >> 4) | (static_cast<uint64_t>(k_stride >> 4) << 16) |
+         (static_cast<uint64_t>(128 >> 4) << 32) | (static_cast<uint64_t>(1) << 46);
+}
+
+// One thread of the (converged) warp, as a value the compiler keeps uniform:
+// MMAs issued under it take their descriptors from uniform registers.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
+
+__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t accum, uint32_t id) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d),
+      "l"(a), "l"(b), "r"(id), "r"(accum));
+}
+
+// Four columns of this warp's 32 lanes from each of four places, waited for:
+// one statement, so no use of the values can move before the wait.
+__device__ __forceinline__ void tmem_ld4x4(uint32_t t0, uint32_t t1, uint32_t t2, uint32_t t3,
+                                           uint32_t (&r)[4][4]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%16];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%17];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%8,%9,%10,%11}, [%18];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%12,%13,%14,%15}, [%19];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=&r"(r[0][0]), "=&r"(r[0][1]), "=&r"(r[0][2]), "=&r"(r[0][3]), "=&r"(r[1][0]),
+        "=&r"(r[1][1]), "=&r"(r[1][2]), "=&r"(r[1][3]), "=&r"(r[2][0]), "=&r"(r[2][1]),
+        "=&r"(r[2][2]), "=&r"(r[2][3]), "=&r"(r[3][0]), "=&r"(r[3][1]), "=&r"(r[3][2]),
+        "=&r"(r[3][3])
+      : "r"(t0), "r"(t1), "r"(t2), "r"(t3)
+      : "memory");
+}
+
+// v as FP16 hi + lo, both components packed (x in the low half).
+__device__ __forceinline__ void split2(float2 v, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(v.x, v.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  float dx, dy;  // hi - v
+  asm("sub.rn.f32.f16 %0, %1, %2;" : "=f"(dx) : "h"(__half_as_ushort(__low2half(h))), "f"(v.x));
+  asm("sub.rn.f32.f16 %0, %1, %2;" : "=f"(dy) : "h"(__half_as_ushort(__high2half(h))), "f"(v.y));
+  const __half2 l = __floats2half2_rn(-dx, -dy);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// Cosine and sine of two phases given in units of 2^-32 cycle: the nearest
+// quarter cycle taken off exactly in the integers, then the Taylor series to
+// x^8 and x^9 on |x| <= pi / 4 (truncation below 3e-8, rounding of the order
+// of 2^-24), two phases per instruction.  The stage tables use it: their
+// phasors multiply every row and column of a channel, where the hardware
+// sine's 2^-21 would be seen twice.
+__device__ __forceinline__ void sincos2(uint32_t p0, uint32_t p1, float2& cs, float2& sn) {
+  const uint32_t q0 = (p0 + 0x20000000u) >> 30, q1 = (p1 + 0x20000000u) >> 30;
+  const float2 r = make_float2(static_cast<float>(static_cast<int>(p0 - (q0 << 30))),
+                               static_cast<float>(static_cast<int>(p1 - (q1 << 30))));
+  auto two = [](float v) { return make_float2(v, v); };
+  const float2 x = __fmul2_rn(r, two(1.46291807926715968e-9f));  // 2 pi / 2^32
+  const float2 z = __fmul2_rn(x, x);
+  float2 s = __ffma2_rn(z, two(2.7557319e-6f), two(-1.9841270e-4f));
+  s = __ffma2_rn(z, s, two(8.3333333e-3f));
+  s = __ffma2_rn(z, s, two(-1.6666667e-1f));
+  s = __ffma2_rn(__fmul2_rn(x, z), s, x);
+  float2 c = __ffma2_rn(z, two(2.4801587e-5f), two(-1.3888889e-3f));
+  c = __ffma2_rn(z, c, two(4.1666667e-2f));
+  c = __ffma2_rn(z, c, two(-0.5f));
+  c = __ffma2_rn(z, c, two(1.0f));
+  // (cos, sin)(x + q pi / 2)
+  auto turn = [](uint32_t q, float cx, float sx, float& co, float& so) {
+    const float a = (q & 1u) ? sx : cx, b = (q & 1u) ? cx : sx;
+    co = __uint_as_float(__float_as_uint(a) ^ (((q + 1u) & 2u) << 30));
+    so = __uint_as_float(__float_as_uint(b) ^ ((q & 2u) << 30));
+  };
+  turn(q0, c.x, s.x, cs.x, sn.x);
+  turn(q1, c.y, s.y, cs.y, sn.y);
+}
+
+// An item of the launch: bins k0 .. k0 + kBins - 1 of one set of spectra and
+// the pass of n_a al's from trial j_p.
+struct Item {
+  int set;  // series, or batch set
+  int k0, j_p, n_a;
+};
+template <int kNa>
+__host__ __device__ inline int n_passes(int n_dm) {
+  const int total = (n_dm + kPairTrials - 1) / kPairTrials;
+  return (total + kNa - 1) / kNa;
+}
+// Pass p of n_dm trials: al's spread evenly over the passes.
+template <int kNa>
+__device__ __forceinline__ void pass_range(int n_dm, int p, int& j_p, int& n_a) {
+  const int total = (n_dm + kPairTrials - 1) / kPairTrials;
+  const int passes = (total + kNa - 1) / kNa;
+  const int per = (total + passes - 1) / passes;
+  j_p = p * per * kPairTrials;
+  n_a = total - p * per < per ? total - p * per : per;
+}
+template <int kNa>
+__device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, int n_sets, int item) {
+  Item q;
+  int local, n_dm, groups;
+  if (sets) {
+    int lo = 0, hi = n_sets - 1;  // last set with item_begin <= item
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (sets[mid].item_begin <= item) lo = mid; else hi = mid - 1;
+    }
+    q.set = lo;
+    local = item - static_cast<int>(sets[lo].item_begin);
+    n_dm = sets[lo].args.n_dm;
+    groups = sets[lo].n_bin_tiles;
+  } else {
+    groups = (a.n_bins + Cfg<kNa>::kBins - 1) / Cfg<kNa>::kBins;
+    n_dm = a.n_dm;
+    const int per_series = groups * n_passes<kNa>(n_dm);
+    q.set = item / per_series;
+    local = item - q.set * per_series;
+  }
+  const int p = local / groups;
+  q.k0 = (local - p * groups) * Cfg<kNa>::kBins;
+  pass_range<kNa>(n_dm, p, q.j_p, q.n_a);
+  return q;
+}
+
+template <int kNa>
+__global__ void __launch_bounds__(kThreads, 1)
+    mac_split_kernel(const MacArgs a, const BatchSet* sets, int n_sets, int n_items) {
+  using C = Cfg<kNa>;
+  constexpr int kBins = C::kBins;
+  constexpr int kN = C::kN;
+  constexpr int S = C::kStages;
+  constexpr int T = C::kTables;
+  extern __shared__ unsigned char smem_raw[];
+  Smem<kNa>& sm = *reinterpret_cast<Smem<kNa>*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  volatile int* abort_flag = &sm.abort_flag;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < C::kTables; ++i) {
+      mbar_init(&sm.pfull[i], 1);
+      mbar_init(&sm.pfree[i], C::kTasks);
+    }
+    for (int i = 0; i < S; ++i) {
+      // the stage's operands written, and its accumulator's last contents read
+      mbar_init(&sm.full[i], C::kTasks + kEpiWarps);
+      mbar_init(&sm.done[i], 1);
+    }
+    mbar_init(&sm.xbar, kEpiWarps);
+    mbar_init(&sm.drain, 1);
+    sm.abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncwarp();
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&sm.tmem)),
+                 "n"(C::kTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = sm.tmem;
+
+  const int n_chan = sets ? sets[0].args.n_chan : a.n_chan;  // common to a batch
+  const int n_chunks = (n_chan + kCh - 1) / kCh;
+  const int per_item = n_chunks * kBins;  // stages of an item: chunk-major, bins inner
+  const int my_items = (n_items - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1;
+  const uint32_t total = static_cast<uint32_t>(my_items) * per_item;  // stages of this CTA
+  // K steps of 16 channels of an item's last stage (the others have all four)
+  const int tail_steps = (n_chan - (n_chunks - 1) * kCh + 15) / 16;
+  bool ok = true;
+  int* status = sets ? sets[0].args.status : a.status;
+
+  if (warp < kEpiWarps) {
+    // ------------------------------------------------------------ epilogue
+    // A thread holds sixteen (bin, al) units of four sums each.
+    const int row = threadIdx.x;  // row of the product: Cb (< 64) or Sb
+    const uint32_t t_lane = tmem + (static_cast<uint32_t>(warp * 32) << 16);
+    const int b = row & 63;
+    const bool is_c = row < 64;
+    for (int s = 0; s < S; ++s) mbar_arrive_warp(&sm.full[s]);  // every accumulator is free at first
+    uint32_t xphase = 0;  // phases of the exchange barrier: two per item
+    auto exchange_sync = [&]() {
+      mbar_arrive_warp(&sm.xbar);
+      const bool met = warp_wait(&sm.xbar, xphase & 1, abort_flag);
+      ++xphase;
+      return met;
+    };
+    uint32_t n_item = 0;  // first stage of the item
+    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, n_item += per_item) {
+      float2 acc[kBins][4][kNa / 2];
+#pragma unroll
+      for (int s = 0; s < kBins; ++s)
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int i = 0; i < kNa / 2; ++i) acc[s][t][i] = make_float2(0.f, 0.f);
+      for (int c = 0; c < n_chunks && ok; ++c) {
+#pragma unroll
+        for (int sl = 0; sl < kBins; ++sl) {
+          const uint32_t n = n_item + c * kBins + sl;
+          const uint32_t s = n % S;
+          ok = ok && warp_wait(&sm.done[s], (n / S) & 1, abort_flag);
+          if (!ok) break;
+          const float hv = sm.inv[n % (4 * C::kTables)];
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const float2 inv = make_float2(hv, hv);
+#pragma unroll
+          for (int h = 0; h < kNa / 4; ++h) {
+#pragma unroll
+            for (int t = 0; t < 4; t += 2) {
+              // [type t, t + 1: hi hi; the small products of both][al]
+              uint32_t r[4][4];
+              const uint32_t col = t_lane + s * 2 * kN + t * kNa + 4 * h;
+              tmem_ld4x4(col, col + kNa, col + kN, col + kN + kNa, r);
+              if (h == kNa / 4 - 1 && t == 2) {
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                mbar_arrive_warp(&sm.full[s]);
+              }
+#pragma unroll
+              for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                  float2& d = acc[sl][t + e][2 * h + i];
+                  const float2 v = __fadd2_rn(
+                      make_float2(__uint_as_float(r[e][2 * i]), __uint_as_float(r[e][2 * i + 1])),
+                      make_float2(__uint_as_float(r[2 + e][2 * i]),
+                                  __uint_as_float(r[2 + e][2 * i + 1])));
+                  d = __ffma2_rn(v, inv, d);
+                }
+            }
+          }
+        }
+      }
+      if (!ok) break;
+      // Y[s, t] = A_s + i t B_s,  A_s = sum Cb X (Ca + i s Sa), B_s the same
+      // with Sb: through shared memory, eight (al, bin) units at a time; the
+      // thread of a Cb row then makes the trials of s = +, that of the Sb row
+      // of the same b those of s = -.
+      const Item q = decode<kNa>(a, sets, n_sets, item);
+      const MacArgs& m = sets ? sets[q.set].args : a;
+      const int64_t dm_stride = m.y_dm_stride;
+      const int n_dm = m.n_dm, n_bins = m.n_bins, out_kind = m.out_kind;
+      const float scale = m.scale;
+      const int k_abs = m.k_begin + q.k0, real_a = m.real_bin_a, real_b = m.real_bin_b;
+      const int64_t off = (sets ? 0 : static_cast<int64_t>(q.set) * m.y_series_stride) + q.k0;
+      void* const Yv = m.Y;
+      const bool whole = q.k0 + kBins <= n_bins;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        constexpr int kAls = 8 / kBins;  // al's of a half
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int al = half * kAls + u / kBins, sl = u % kBins;
+          const float m1 = (al & 1) ? acc[sl][0][al / 2].y : acc[sl][0][al / 2].x;
+          const float m2 = (al & 1) ? acc[sl][1][al / 2].y : acc[sl][1][al / 2].x;
+          const float m3 = (al & 1) ? acc[sl][2][al / 2].y : acc[sl][2][al / 2].x;
+          const float m4 = (al & 1) ? acc[sl][3][al / 2].y : acc[sl][3][al / 2].x;
+          sm.xch[u][row] = make_float4(m1 - m4, m2 + m3, m1 + m4, m2 - m3);
+        }
+        if (!(ok = exchange_sync())) break;
+#pragma unroll 1
+        for (int i = 0; i < kAls; ++i) {
+          const int al = half * kAls + i;
+          if (al >= q.n_a) break;
+          float2 y[2][kBins];  // t = +, -
+#pragma unroll
+          for (int sl = 0; sl < kBins; ++sl) {
+            const float2 A = reinterpret_cast<const float2*>(&sm.xch[i * kBins + sl][b])[is_c ? 0 : 1];
+            const float2 B = reinterpret_cast<const float2*>(&sm.xch[i * kBins + sl][b + 64])[is_c ? 0 : 1];
+            const bool real_only = k_abs + sl == real_a || k_abs + sl == real_b;
+            y[0][sl] = make_float2((A.x - B.y) * scale, real_only ? 0.f : (A.y + B.x) * scale);
+            y[1][sl] = make_float2((A.x + B.y) * scale, real_only ? 0.f : (A.y - B.x) * scale);
+          }
+          // trial of (s, al, t, b)
+          const int step = 128 * al + 64;
+          const int jc = q.j_p + kPairTrials / 2 * q.n_a + (is_c ? step : -step);
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const int j = t == 0 ? jc + b : jc - 1 - b;
+            if (j >= n_dm) continue;
+            const int64_t o = off + static_cast<int64_t>(j) * dm_stride;
+            if (out_kind == 2) {
+              float* Y = static_cast<float*>(Yv) + o;
+              float pw[kBins];
+#pragma unroll
+              for (int sl = 0; sl < kBins; ++sl)
+                pw[sl] = y[t][sl].x * y[t][sl].x + y[t][sl].y * y[t][sl].y;
+              if (kBins == 4 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
+                *reinterpret_cast<float4*>(Y) = make_float4(pw[0], pw[1 % kBins], pw[2 % kBins], pw[3 % kBins]);
+              } else if (kBins == 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 7) == 0) {
+                *reinterpret_cast<float2*>(Y) = make_float2(pw[0], pw[1 % kBins]);
+              } else {
+#pragma unroll
+                for (int sl = 0; sl < kBins; ++sl)
+                  if (q.k0 + sl < n_bins) Y[sl] = pw[sl];
+              }
+            } else {
+              float2* Y = static_cast<float2*>(Yv) + o;
+              if (kBins >= 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
+#pragma unroll
+                for (int sl = 0; sl < kBins; sl += 2)
+                  *reinterpret_cast<float4*>(Y + sl) =
+                      make_float4(y[t][sl].x, y[t][sl].y, y[t][(sl + 1) % kBins].x, y[t][(sl + 1) % kBins].y);
+              } else {
+#pragma unroll
+                for (int sl = 0; sl < kBins; ++sl)
+                  if (q.k0 + sl < n_bins) Y[sl] = y[t][sl];
+              }
+            }
+          }
+        }
+        if (!(ok = exchange_sync())) break;  // read before the next writes
+      }
+    }
+  } else if (warp == kMmaWarp) {
+    // ------------------------------------------------------------ MMA issuer
+    const uint32_t el = elect_one();
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t base = __shfl_sync(0xffffffffu, smem_u32(&sm.stage[0][0]), 0);
+    constexpr uint32_t id = (1u << 4) | (static_cast<uint32_t>(kN >> 3) << 17) |
+                            (static_cast<uint32_t>(kRows >> 4) << 24);  // FP16 x FP16 -> FP32
+    constexpr uint32_t id2 = (1u << 4) | (static_cast<uint32_t>(2 * kN >> 3) << 17) |
+                             (static_cast<uint32_t>(kRows >> 4) << 24);  // hi and lo columns at once
+    bool issued = false;
+    uint32_t left = per_item;  // stages of the item still to come
+    uint32_t phase = 0;
+    int s = 0;
+    for (uint32_t n = 0; n < total; ++n) {
+      ok = warp_wait(&sm.full[s], phase, abort_flag);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const int steps = left <= kBins ? tail_steps : 4;
+      if (el) {
+        const uint32_t st = base + s * C::kStageBytes;
+        const uint32_t d = tm + s * 2 * kN;
+        const uint64_t a_hi = core_desc(st, kRows * 16);
+        const uint64_t a_lo = core_desc(st + C::kATile, kRows * 16);
+        const uint64_t b = core_desc(st + 2 * C::kATile, 2 * kN * 16);
+        // A K step of 16 channels: two core matrices along K.  The rows' hi
+        // term takes both terms of the columns in one MMA of twice the
+        // width (the MMAs are bound by reading the rows from shared memory:
+        // two reads a K step instead of three); the small products go to
+        // the second half of the accumulator.
+        constexpr uint32_t ka = 2 * kRows * 16 / 16, kb = 2 * 2 * kN * 16 / 16;
+        if (steps == 4) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) mma(d, a_hi + i * ka, b + i * kb, i > 0 ? 1u : 0u, id2);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) mma(d + kN, a_lo + i * ka, b + i * kb, 1u, id);
+        } else {
+#pragma unroll 1
+          for (int i = 0; i < steps; ++i) mma(d, a_hi + i * ka, b + i * kb, i > 0 ? 1u : 0u, id2);
+#pragma unroll 1
+          for (int i = 0; i < steps; ++i) mma(d + kN, a_lo + i * ka, b + i * kb, 1u, id);
+        }
+        asm volatile(
+            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                smem_u32(&sm.done[s]))
+            : "memory");
+      }
+      issued = true;
+      left = left == 1 ? per_item : left - 1;
+      if (++s == S) {
+        s = 0;
+        phase ^= 1;
+      }
+      __syncwarp();
+    }
+    // (the epilogue waits for every stage, so tensor memory is idle at the
+    // end; after a timeout the MMAs in flight are drained here)
+    if (!ok && issued) {
+      if (el)
+        asm volatile(
+            "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                smem_u32(&sm.drain))
+            : "memory");
+      volatile int never = 0;
+      warp_wait(&sm.drain, 0, &never);
+    }
+  } else if (warp < kProdFirst) {
+    // ------------------------------------------------------------ stage tables
+    // lane = channels lane and lane + 32 of the stage; the next stage's loads
+    // fly while this one's table is made and waits for its place
+    struct Fetched {
+      float2 x[2];
+      uint4 pc[2];      // u_lo, u_hi, v_lo, v_hi
+      uint32_t k;       // absolute bin
+      uint32_t before;  // Jc - 1/2: the trial below the pass centre
+      int c0;           // this lane's first channel
+      int steps;        // K steps of the stage
+      bool bin_ok;
+    };
+    const int p = warp - kPrepFirst;
+    int item = blockIdx.x;
+    int q = p;  // stage within the item
+    // the item at hand, in registers: its spectra, constants and phases' origin
+    int cur = -1, left_bins = 0, k_abs = 0;
+    uint32_t before = 0;
+    const float2* X = nullptr;
+    int64_t xs = 0;
+    const PhaseConst* pcs = nullptr;
+    auto fetch = [&](Fetched& f) {
+      // The loads are unconditional, from clamped addresses, and idle channels
+      // and bins are zeroed where they are used: a load under a condition
+      // would be waited for right here, to merge it with the other value.
+      while (q >= per_item) {
+        q -= per_item;
+        item += gridDim.x;
+      }
+      if (item != cur && item < n_items) {
+        const Item it = decode<kNa>(a, sets, n_sets, item);
+        const MacArgs& m = sets ? sets[it.set].args : a;
+        cur = item;
+        left_bins = m.n_bins - it.k0;
+        k_abs = m.k_begin + it.k0;
+        before = static_cast<uint32_t>(m.j_begin + it.j_p + 128 * it.n_a - 1);
+        X = m.X + (sets ? 0 : static_cast<int64_t>(it.set) * m.x_series_stride) + it.k0;
+        xs = m.x_chan_stride;
+        pcs = m.pc;
+      }
+      const int slot = q % kBins;
+      f.steps = q >= per_item - kBins ? tail_steps : 4;
+      f.c0 = q / kBins * kCh + lane;
+      f.bin_ok = slot < left_bins;
+      f.k = static_cast<uint32_t>(k_abs + slot);
+      f.before = before;
+      const float2* xb = X + (f.bin_ok ? slot : 0);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = min(f.c0 + 32 * h, n_chan - 1);
+        asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(f.pc[h].x), "=r"(f.pc[h].y), "=r"(f.pc[h].z), "=r"(f.pc[h].w)
+                     : "l"(pcs + c));
+        asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];"
+                     : "=f"(f.x[h].x), "=f"(f.x[h].y)
+                     : "l"(xb + static_cast<int64_t>(c) * xs));
+      }
+      q += kPrepWarps;
+    };
+    Fetched next;
+    fetch(next);
+    for (uint32_t n = p; n < total; n += kPrepWarps) {
+      const uint32_t s = n % T;
+      float2 x[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const bool use = next.bin_ok && next.c0 + 32 * h < n_chan;
+        x[h] = use ? next.x[h] : make_float2(0.f, 0.f);
+      }
+      const uint4 pc[2] = {next.pc[0], next.pc[1]};
+      const uint32_t k = next.k;
+      const uint32_t j1 = next.before;
+      const int steps = next.steps;
+      // power-of-two scale: the stage's largest component to [2^13, 2^14)
+      uint32_t top = 0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        top = max(top, max(__float_as_uint(x[h].x) & 0x7FFFFFFFu, __float_as_uint(x[h].y) & 0x7FFFFFFFu));
+      top = __reduce_max_sync(0xffffffffu, top);
+      int f = 14 + 253 - static_cast<int>(top >> 23);
+      f = f < 1 ? 1 : (f > 253 ? 253 : f);
+      const float sc = __uint_as_float(static_cast<uint32_t>(f) << 23);
+      uint32_t hw[2], ha[2], pf[2], pm[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint64_t u = (static_cast<uint64_t>(pc[h].y) << 32) | pc[h].x;
+        const uint64_t v = (static_cast<uint64_t>(pc[h].w) << 32) | pc[h].z;
+        const uint64_t half = (v * k) >> 1;  // half a trial step, mod half a cycle
+        const uint64_t mid = (u + v * j1) * k + half;  // the pass centre
+        constexpr uint64_t kRound = 0x80000000ull;
+        hw[h] = static_cast<uint32_t>((half + kRound) >> 32);
+        ha[h] = static_cast<uint32_t>(((half << 7) + kRound) >> 32);
+        pf[h] = static_cast<uint32_t>(((half << 5) + kRound) >> 32);
+        pm[h] = static_cast<uint32_t>(mid >> 32);
+      }
+      float2 fc, fs, mc, ms;
+      sincos2(pf[0], pf[1], fc, fs);
+      sincos2(pm[0], pm[1], mc, ms);
+      const float2 xr = make_float2(x[0].x * sc, x[1].x * sc), xi = make_float2(x[0].y * sc, x[1].y * sc);
+      const float2 zr = __ffma2_rn(xr, mc, __fmul2_rn(make_float2(-xi.x, -xi.y), ms));
+      const float2 zi = __ffma2_rn(xr, ms, __fmul2_rn(xi, mc));
+      fetch(next);
+      ok = warp_wait(&sm.pfree[s], ((n / T) & 1) ^ 1, abort_flag);
+      if (!ok) break;
+      Table& tb = sm.table[s];
+      tb.hw[lane] = hw[0];
+      tb.hw[lane + 32] = hw[1];
+      tb.ha[lane] = ha[0];
+      tb.ha[lane + 32] = ha[1];
+      tb.fr[lane] = fc.x;
+      tb.fr[lane + 32] = fc.y;
+      tb.fi[lane] = fs.x;
+      tb.fi[lane + 32] = fs.y;
+      tb.xr[lane] = zr.x;
+      tb.xr[lane + 32] = zr.y;
+      tb.xi[lane] = zi.x;
+      tb.xi[lane + 32] = zi.y;
+      if (lane == 0) tb.steps = steps;
+      if (lane == 0) sm.inv[n % (4 * C::kTables)] = __uint_as_float(static_cast<uint32_t>(254 - f) << 23);
+      // Tables complete in order: a producer steps fewer than T stages at a
+      // time, so the table T stages back is then complete when it waits for
+      // one (a wait by parity sees only whether the count is odd).
+      if (n > 0)
+        ok = warp_wait(&sm.pfull[(n - 1) % T], ((n - 1) / T) & 1, abort_flag);
+      if (!ok) break;
+      mbar_arrive_warp(&sm.pfull[s]);
+    }
+  } else {
+    // ------------------------------------------------------------ producers
+    // Waits by parity see one phase back only.  A producer steps fewer than S
+    // stages from task to task and waits for each task's stage to be free, so
+    // when it waits for stage n to be free, n - 2 S is (MMAs end in order).
+    for (uint32_t task = warp - kProdFirst;; task += kProdWarps) {
+      const uint32_t n = task / C::kTasks;
+      const int part0 = static_cast<int>(task % C::kTasks);
+      const bool rows = part0 >= C::kColTasks;
+      const int part = rows ? part0 - C::kColTasks : part0;
+      if (n >= total) break;
+      const uint32_t s = n % S;
+      const uint32_t ts = n % T;
+      ok = warp_wait(&sm.pfull[ts], (n / T) & 1, abort_flag);
+      if (!ok) break;
+      const Table& tb = sm.table[ts];
+      const int steps = tb.steps;
+      if (rows) {
+        // rows: lane = (b < 16, half of an octet of channels): Cb, Sb of four
+        // channels for b, b + 16, b + 32 and b + 48, the later ones by the
+        // 16-step phasor (both halves of a row's 16 bytes are stored by the
+        // same instruction, and only 32 registers hold a lane's results)
+        if (part < steps) {
+          const int b = lane >> 1, half = lane & 1;  // (16 lanes store 128 contiguous bytes)
+          const uint32_t mul = 2u * b + 1u;
+#pragma unroll
+          for (int o = 0; o < 2; ++o) {
+            const int oct = 2 * part + o;
+            const int ch = 8 * oct + 4 * half;
+            const uint4 hv = *reinterpret_cast<const uint4*>(&tb.hw[ch]);
+            const float4 frv = *reinterpret_cast<const float4*>(&tb.fr[ch]);
+            const float4 fiv = *reinterpret_cast<const float4*>(&tb.fi[ch]);
+            uint32_t hi[8][2], lo[8][2];  // [C, S of b + 16 i][channel pair]
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const float2 fr = p ? make_float2(frv.z, frv.w) : make_float2(frv.x, frv.y);
+              const float2 fi = p ? make_float2(fiv.z, fiv.w) : make_float2(fiv.x, fiv.y);
+              const float2 nfi = make_float2(-fi.x, -fi.y);
+              const float2 w0 = unit_phasor(mul * (p ? hv.z : hv.x));
+              const float2 w1 = unit_phasor(mul * (p ? hv.w : hv.y));
+              float2 cs = make_float2(w0.x, w1.x), sn = make_float2(w0.y, w1.y);
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                split2(cs, hi[i][p], lo[i][p]);
+                split2(sn, hi[4 + i][p], lo[4 + i][p]);
+                if (i < 3) {
+                  const float2 c1 = __ffma2_rn(cs, fr, __fmul2_rn(sn, nfi));
+                  sn = __ffma2_rn(cs, fi, __fmul2_rn(sn, fr));
+                  cs = c1;
+                }
+              }
+            }
+            if (o == 0) {
+              ok = warp_wait(&sm.done[s], ((n / S) & 1) ^ 1, abort_flag);
+              if (!ok) break;
+            }
+            unsigned char* at = &sm.stage[s][oct * kRows * 16 + b * 16 + half * 8];
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+              *reinterpret_cast<uint2*>(at + t * 16 * 16) = make_uint2(hi[t][0], hi[t][1]);
+              *reinterpret_cast<uint2*>(at + C::kATile + t * 16 * 16) = make_uint2(lo[t][0], lo[t][1]);
+            }
+          }
+          if (!ok) break;
+        } else {  // (waited for all the same: see the wait by parity)
+          ok = warp_wait(&sm.done[s], ((n / S) & 1) ^ 1, abort_flag);
+          if (!ok) break;
+        }
+      } else {
+        // columns: lane = (al, half octet): Xr Ca, Xi Ca, Xr Sa, Xi Sa of four
+        // channels at a time
+        constexpr int kHalves = 32 / kNa;               // half octets at a time: 2, 4, 8
+        static_assert(16 / C::kColTasks / kHalves == 2, "two rounds a task");
+        const int al = (lane >> 1) % kNa;
+        const uint32_t mul = 2u * al + 1u;
+        const int h0 = part * 2 * kHalves + 2 * (lane / (2 * kNa)) + (lane & 1);
+        const bool live = part * 2 * kHalves < 4 * steps;  // (the round's first, so uniform)
+        uint32_t hi[2][4][2], lo[2][4][2];  // [round][type][channel pair]
+        if (live) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int ch = 4 * (h0 + e * kHalves);
+            const uint4 hv = *reinterpret_cast<const uint4*>(&tb.ha[ch]);
+            const float4 xrv = *reinterpret_cast<const float4*>(&tb.xr[ch]);
+            const float4 xiv = *reinterpret_cast<const float4*>(&tb.xi[ch]);
+#pragma unroll
+            for (int p = 0; p < 2; ++p) {
+              const float2 xr = p ? make_float2(xrv.z, xrv.w) : make_float2(xrv.x, xrv.y);
+              const float2 xi = p ? make_float2(xiv.z, xiv.w) : make_float2(xiv.x, xiv.y);
+              const float2 w0 = unit_phasor(mul * (p ? hv.z : hv.x));
+              const float2 w1 = unit_phasor(mul * (p ? hv.w : hv.y));
+              const float2 cs = make_float2(w0.x, w1.x), sn = make_float2(w0.y, w1.y);
+              split2(__fmul2_rn(xr, cs), hi[e][0][p], lo[e][0][p]);
+              split2(__fmul2_rn(xi, cs), hi[e][1][p], lo[e][1][p]);
+              split2(__fmul2_rn(xr, sn), hi[e][2][p], lo[e][2][p]);
+              split2(__fmul2_rn(xi, sn), hi[e][3][p], lo[e][3][p]);
+            }
+          }
+        }
+        ok = warp_wait(&sm.done[s], ((n / S) & 1) ^ 1, abort_flag);
+        if (!ok) break;
+        if (live) {
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int hf = h0 + e * kHalves;
+            unsigned char* bt =
+                &sm.stage[s][2 * C::kATile + (hf >> 1) * 2 * kN * 16 + al * 16 + (hf & 1) * 8];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              *reinterpret_cast<uint2*>(bt + t * kNa * 16) = make_uint2(hi[e][t][0], hi[e][t][1]);
+              *reinterpret_cast<uint2*>(bt + kN * 16 + t * kNa * 16) =
+                  make_uint2(lo[e][t][0], lo[e][t][1]);
+            }
+          }
+        }
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(&sm.full[s]);
+        mbar_arrive(&sm.pfree[ts]);
+      }
+    }
+  }
+  if (!ok) {
+    *abort_flag = 1;
+    if (status && lane == 0) atomicExch(status, FDD_ERR_TIMEOUT);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == kMmaWarp) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "n"(C::kTmemCols));
+  }
+}
+
+template <int kNa>
+const void* split_fn() {
+  return reinterpret_cast<const void*>(&mac_split_kernel<kNa>);
+}
+template <int kNa>
+constexpr int split_smem() { return static_cast<int>(sizeof(Smem<kNa>)) + 128; }
+
+// al's a pass must hold for n_dm trials: up to four, eight or sixteen (1024,
+// 2048, 4096 trials a pass).
+int capacity(int n_dm) {
+  const int total = (n_dm + kPairTrials - 1) / kPairTrials;
+  return total <= 4 ? 4 : total <= 8 ? 8 : 16;
+}
+
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_sms[kMaxDevices];
+
+cudaError_t sm_count(int* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  int n = dev < kMaxDevices ? g_sms[dev].load(std::memory_order_relaxed) : 0;
+  if (n == 0) {
+    e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (dev < kMaxDevices) g_sms[dev].store(n, std::memory_order_relaxed);
+  }
+  *out = n;
+  return cudaSuccess;
+}
+
+cudaError_t launch_split(const MacArgs& a, const BatchSet* sets, int n_sets, int n_items, int cap,
+                         int n_ctas, cudaStream_t s) {
+  MacArgs args = a;
+  void* params[] = {&args, &sets, &n_sets, &n_items};
+  const dim3 grid(n_items < n_ctas ? n_items : n_ctas);
+  note_launches(1);
+  switch (cap) {
+    case 4: return cudaLaunchKernel(split_fn<4>(), grid, dim3(kThreads), params, split_smem<4>(), s);
+    case 8: return cudaLaunchKernel(split_fn<8>(), grid, dim3(kThreads), params, split_smem<8>(), s);
+    default:
+      return cudaLaunchKernel(split_fn<16>(), grid, dim3(kThreads), params, split_smem<16>(), s);
+  }
+}
+
+constexpr long long kMaxItems = 0x7FFF0000LL;  // item numbers, stepped by the grid, stay in an int
+
+}  // namespace
+
+size_t mac_split_smem_bytes() {
+  return split_smem<4>() > split_smem<8>()
+             ? (split_smem<4>() > split_smem<16>() ? split_smem<4>() : split_smem<16>())
+             : (split_smem<8>() > split_smem<16>() ? split_smem<8>() : split_smem<16>());
+}
+
+cudaError_t mac_split_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(split_fn<4>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       split_smem<4>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(split_fn<8>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             split_smem<8>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(split_fn<16>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             split_smem<16>());
+  return e;
+}
+
+void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes) {
+  const int cap = capacity(max_n_dm);
+  const int bins = 16 / cap;
+  *bin_groups = static_cast<int>((n_bins + bins - 1) / bins);
+  *passes = cap == 4 ? n_passes<4>(n_dm) : cap == 8 ? n_passes<8>(n_dm) : n_passes<16>(n_dm);
+}
+
+cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
+                                   int max_n_dm, int n_ctas, cudaStream_t s) {
+  if (n_items <= 0) return cudaSuccess;
+  if (n_items > kMaxItems) return cudaErrorInvalidConfiguration;
+  return launch_split(MacArgs{}, d_sets, n_sets, static_cast<int>(n_items), capacity(max_n_dm),
+                      n_ctas, s);
+}
+
+cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
+  int n_sms = 0;
+  cudaError_t e = sm_count(&n_sms);
+  if (e != cudaSuccess) return e;
+  int groups, passes;
+  mac_split_batch_shape(a.n_dm, a.n_dm, a.n_bins, &groups, &passes);
+  const long long per_series = static_cast<long long>(groups) * passes;
+  if (per_series > kMaxItems) return cudaErrorInvalidConfiguration;
+  // (series in blocks whose items can be numbered in an int)
+  const size_t y_elem = a.out_kind == 2 ? sizeof(float) : sizeof(float2);
+  const long long block = kMaxItems / per_series;
+  for (long long s0 = 0; s0 < a.n_series; s0 += block) {
+    MacArgs c = a;
+    c.n_series = static_cast<int>(a.n_series - s0 < block ? a.n_series - s0 : block);
+    c.X = a.X + s0 * a.x_series_stride;
+    c.Y = static_cast<char*>(a.Y) + y_elem * static_cast<size_t>(s0 * a.y_series_stride);
+    e = launch_split(c, nullptr, 0, static_cast<int>(per_series * c.n_series), capacity(a.n_dm),
+                     n_sms, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace fdd

@@ -1,0 +1,100 @@
+"""The G12_4X8 tile (split-FP16 operands on the tensor cores) at the sizes
+where it can go wrong (GB300 only): channel counts around a K step (16) and a
+stage (64), trial counts around an al (256) and the pass capacities (1024,
+2048, 4096 trials), bin counts that leave a group of bins partly idle.
+
+Tolerance: a product carries two hardware-sine phasors (absolute error up to
+2^-20.9 each, 1.7e-7 rms), table phasors of a few 2^-24 and operands of 22
+bits (2^-22 each); random over channels, the sum's relative L2 error stays
+below 4e-7, and 1e-6 leaves the factor between rms and a small sample.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2110_03482_gb300 as fdd
+from gpu_util import complex_to_device, device_to_complex, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+TOL = 1e-6
+BAND = (1200.0, 1500.0)
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fdd.build()
+
+
+def _plan(n_chan, L, dms, **kw):
+    dnu = (BAND[1] - BAND[0]) / n_chan
+    return fdd.Plan(n_chan=n_chan, nu_lo_mhz=BAND[0] + 0.5 * dnu, dnu_mhz=dnu, t_samp_s=2e-3,
+                    n_t=L, dm_list=dms, in_dtype=fdd.FDD_IN_F32, output=fdd.FDD_OUT_SPECTRA,
+                    mac_variant=1 + fdd.FDD_MAC_G12_4X8, **kw)
+
+
+def _reference(X, bins, L, n_chan, dms):
+    dnu = (BAND[1] - BAND[0]) / n_chan
+    nu = oracle.channel_centres(n_chan, BAND[0] + 0.5 * dnu, dnu)
+    return oracle.fdd_bins(X, bins, L, oracle.delays(nu, dms, 2e-3))
+
+
+@pytest.mark.parametrize("n_chan,n_dm,n_series", [
+    (1, 1, 1), (15, 255, 1), (16, 256, 2), (17, 257, 1), (48, 512, 1), (63, 513, 1),
+    (64, 1024, 1), (65, 1025, 2), (80, 2048, 1), (81, 2049, 1), (129, 2305, 1), (130, 4096, 1),
+    (193, 4097, 1), (33, 8449, 1),
+])
+def test_edges_match_oracle(n_chan, n_dm, n_series):
+    L, dms = 1 << 12, 3.7 + 0.31 * np.arange(n_dm)
+    K = L // 2 + 1
+    rng = np.random.default_rng(100 * n_chan + n_dm)
+    for b0, nb in [(0, 1), (1021, 7), (K - 6, 6)]:
+        X = (rng.standard_normal((n_series, n_chan, nb)) +
+             1j * rng.standard_normal((n_series, n_chan, nb))).astype(np.complex64)
+        with _plan(n_chan, L, dms) as plan:
+            dX = complex_to_device(X, nb + 1)
+            dY = torch.full((n_series, n_dm, nb + 3, 2), 7.0, device="cuda")
+            plan.dedisperse_spectra_bins(dX, nb + 1, n_series, b0, nb, 0, n_dm, dY, nb + 3)
+            dP = torch.full((n_series, n_dm, nb), 7.0, device="cuda")
+            plan.dedisperse_spectra_bins(dX, nb + 1, n_series, b0, nb, 0, n_dm, dP, nb,
+                                         fdd.FDD_OUT_POWER)
+            torch.cuda.synchronize()
+            plan.query()
+        assert torch.all(dY[:, :, nb:] == 7.0)  # the pitch's padding is untouched
+        for s in range(n_series):
+            ref = _reference(X[s].astype(np.complex128), np.arange(b0, b0 + nb), L, n_chan, dms)
+            assert rel_l2(device_to_complex(dY, nb)[s], ref) <= TOL, (b0, s)
+            assert rel_l2(dP[s].cpu().numpy(), np.abs(ref) ** 2) <= 2 * TOL, (b0, s)
+
+
+@pytest.mark.parametrize("n_dm", [300, 2048, 3000])
+def test_dynamic_range(n_dm):
+    """Channels of very different size (the columns share one power-of-two
+    scale per 64 channels), the smallest and largest normal magnitudes, zeros,
+    and a NaN that stays in its own bin."""
+    n_chan, L, nb, b0 = 100, 1 << 12, 8, 333
+    dms = 0.5 * np.arange(n_dm)
+    rng = np.random.default_rng(n_dm)
+    X = rng.standard_normal((1, n_chan, nb)) + 1j * rng.standard_normal((1, n_chan, nb))
+    X[0, :, 1] *= 10.0 ** rng.uniform(-6, 6, n_chan)   # spread over twelve decades
+    X[0, :, 2] *= 1e-36
+    X[0, :, 3] *= 1e35
+    X[0, :, 4] = 0.0
+    X[0, :70, 5] = 0.0
+    X[0, :, 6] = 1e-30 + 0j
+    X = X.astype(np.complex64)
+    with _plan(n_chan, L, dms) as plan:
+        dX = complex_to_device(X, nb)
+        dX[0, 40, 7, 0] = float("nan")
+        dY = torch.empty((1, n_dm, nb, 2), device="cuda")
+        plan.dedisperse_spectra_bins(dX, nb, 1, b0, nb, 0, n_dm, dY, nb)
+        torch.cuda.synchronize()
+    ref = _reference(X[0].astype(np.complex128), np.arange(b0, b0 + nb), L, n_chan, dms)
+    Y = device_to_complex(dY, nb)[0]
+    for i in range(7):
+        assert rel_l2(Y[:, i], ref[:, i]) <= TOL, i
+    assert np.all(Y[:, 4] == 0) and np.all(np.isnan(Y[:, 7]))

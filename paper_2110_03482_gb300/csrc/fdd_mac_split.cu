@@ -3,9 +3,11 @@
 //
 //   Y[j][k] = sum_nu W(k, nu, j) X[nu][k],   W = exp(+2 pi i k d(nu, DM_j) / L)
 //
-// Trials are paired around centres.  A pass covers 256 n_a trials from j_p;
-// with Jc = j_p + 128 n_a - 1/2, trial j = Jc + s (128 al + 64) + t (b + 1/2)
-// for s, t = +-1, al < n_a, b < 64.  The phase is linear in j, so
+// Trials are paired around the centre of their block of at most 2048 (counted
+// from the first trial of the call, so that calls on parts made of whole blocks
+// agree with a whole call bit for bit).  A block of 256 n_a trials from j_b has
+// the centre Jc = j_b + 128 n_a - 1/2 and the trials j = Jc + s (128 al + 64) +
+// t (b + 1/2) for s, t = +-1, al < n_a, b < 64.  The phase is linear in j, so
 //
 //   W = exp(i phi_c) (Ca + i s Sa) (Cb + i t Sb),
 //
@@ -15,7 +17,8 @@
 //   M = sum Cb {Xr Ca, Xi Ca, Xr Sa, Xi Sa},   N = sum Sb {the same},
 //
 // (X rotated by exp(i phi_c)) are ONE real matrix product per bin: 128 rows
-// (Cb, Sb of 64 b's) x channels times channels x 4 n_a columns.  Against the
+// (Cb, Sb of 64 b's) x channels times channels x 4 n_a columns, of one block or
+// of two that share the rows.  Against the
 // complex form this halves both the multiplications (eight real ones for four
 // trials' complex products) and the phasors to evaluate (64 for 128 trials).
 //
@@ -85,6 +88,7 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 constexpr int kCh = 64;     // channels per stage (four K steps of 16)
 constexpr int kRows = 128;  // Cb | Sb of 64 b's
 constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's
+constexpr int kBlockAls = 8;      // al's of a whole block (2048 trials)
 
 // Warps: 0-3 epilogue (a warp reads the tensor-memory lanes of its quarter),
 // the MMA issuer, two that make the stages' tables in turn, and thirteen
@@ -100,6 +104,8 @@ constexpr int kThreads = 32 * (kProdFirst + kProdWarps);
 template <int kNa>
 struct Cfg {
   static constexpr int kBins = 16 / kNa;
+  static constexpr int kBlocks = kNa == 16 ? 2 : 1;  // blocks of trials of a pass
+  static constexpr int kAls = kNa / kBlocks;         // al's of each
   static constexpr int kN = 4 * kNa;          // columns
   static constexpr int kStages = kNa == 16 ? 4 : 5;
   static constexpr int kTables = kNa == 8 ? 6 : 8;  // tables run further ahead than operands
@@ -117,11 +123,12 @@ struct Cfg {
 };
 
 // Per stage: what the producers need of each channel.
+template <int kBlocks>
 struct Table {
   uint32_t hw[kCh];   // half the trial step's phase, units of 2^-32 cycle
   uint32_t ha[kCh];   // 64 trial steps
   float fr[kCh], fi[kCh];  // phasor of 16 trial steps (b -> b + 16)
-  float xr[kCh], xi[kCh];  // X rotated to the pass centre and scaled
+  float xr[kBlocks][kCh], xi[kBlocks][kCh];  // X rotated to each block's centre and scaled
   int steps;               // K steps of 16 channels the MMAs read
   int pad[3];
 };
@@ -130,7 +137,7 @@ struct Smem {
   using C = Cfg<kNa>;
   alignas(128) unsigned char stage[C::kStages][C::kStageBytes];
   alignas(16) float4 xch[8][kRows];  // epilogue exchange: A_+, A_- of a row (or B_+, B_-)
-  alignas(16) Table table[C::kTables];
+  alignas(16) Table<C::kBlocks> table[C::kTables];
   float inv[4 * C::kTables];  // undoes a stage's scale (read by the epilogue, well after the table)
   uint64_t pfull[C::kTables], pfree[C::kTables];  // table written; every producer has read it
   uint64_t full[C::kStages], done[C::kStages];   // operands written; MMAs complete
@@ -223,24 +230,20 @@ __device__ __forceinline__ void sincos2(uint32_t p0, uint32_t p1, float2& cs, fl
 }
 
 // An item of the launch: bins k0 .. k0 + kBins - 1 of one set of spectra and
-// the pass of n_a al's from trial j_p.
+// the pass of up to 256 kNa trials from j_p.
 struct Item {
   int set;  // series, or batch set
-  int k0, j_p, n_a;
+  int k0, j_p;
+  int n_a;  // al's of the pass with trials: whole blocks, then the last one's
 };
 template <int kNa>
 __host__ __device__ inline int n_passes(int n_dm) {
-  const int total = (n_dm + kPairTrials - 1) / kPairTrials;
-  return (total + kNa - 1) / kNa;
+  return (n_dm + kPairTrials * kNa - 1) / (kPairTrials * kNa);
 }
-// Pass p of n_dm trials: al's spread evenly over the passes.
-template <int kNa>
-__device__ __forceinline__ void pass_range(int n_dm, int p, int& j_p, int& n_a) {
-  const int total = (n_dm + kPairTrials - 1) / kPairTrials;
-  const int passes = (total + kNa - 1) / kNa;
-  const int per = (total + passes - 1) / passes;
-  j_p = p * per * kPairTrials;
-  n_a = total - p * per < per ? total - p * per : per;
+// al's of block h of a pass with n_a al's
+__device__ __forceinline__ int block_als(int n_a, int h) {
+  const int left = n_a - h * kBlockAls;
+  return left < 0 ? 0 : left < kBlockAls ? left : kBlockAls;
 }
 template <int kNa>
 __device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, int n_sets, int item) {
@@ -265,7 +268,9 @@ __device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, i
   }
   const int p = local / groups;
   q.k0 = (local - p * groups) * Cfg<kNa>::kBins;
-  pass_range<kNa>(n_dm, p, q.j_p, q.n_a);
+  q.j_p = p * kPairTrials * kNa;
+  const int als = (n_dm - q.j_p + kPairTrials - 1) / kPairTrials;
+  q.n_a = als < kNa ? als : kNa;
   return q;
 }
 
@@ -422,8 +427,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             y[1][sl] = make_float2((A.x + B.y) * scale, real_only ? 0.f : (A.y - B.x) * scale);
           }
           // trial of (s, al, t, b)
-          const int step = 128 * al + 64;
-          const int jc = q.j_p + kPairTrials / 2 * q.n_a + (is_c ? step : -step);
+          const int h = al / kBlockAls, step = 128 * (al % kBlockAls) + 64;
+          const int jc = q.j_p + kPairTrials * kBlockAls * h +
+                         kPairTrials / 2 * block_als(q.n_a, h) + (is_c ? step : -step);
 #pragma unroll
           for (int t = 0; t < 2; ++t) {
             const int j = t == 0 ? jc + b : jc - 1 - b;
@@ -535,7 +541,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       float2 x[2];
       uint4 pc[2];      // u_lo, u_hi, v_lo, v_hi
       uint32_t k;       // absolute bin
-      uint32_t before;  // Jc - 1/2: the trial below the pass centre
+      uint32_t before[C::kBlocks];  // Jc - 1/2: the trial below each block's centre
       int c0;           // this lane's first channel
       int steps;        // K steps of the stage
       bool bin_ok;
@@ -545,7 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int q = p;  // stage within the item
     // the item at hand, in registers: its spectra, constants and phases' origin
     int cur = -1, left_bins = 0, k_abs = 0;
-    uint32_t before = 0;
+    uint32_t before[C::kBlocks] = {};
     const float2* X = nullptr;
     int64_t xs = 0;
     const PhaseConst* pcs = nullptr;
@@ -563,7 +569,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         cur = item;
         left_bins = m.n_bins - it.k0;
         k_abs = m.k_begin + it.k0;
-        before = static_cast<uint32_t>(m.j_begin + it.j_p + 128 * it.n_a - 1);
+#pragma unroll
+        for (int h = 0; h < C::kBlocks; ++h)
+          before[h] = static_cast<uint32_t>(m.j_begin + it.j_p + kPairTrials * kBlockAls * h +
+                                            kPairTrials / 2 * block_als(it.n_a, h) - 1);
         X = m.X + (sets ? 0 : static_cast<int64_t>(it.set) * m.x_series_stride) + it.k0;
         xs = m.x_chan_stride;
         pcs = m.pc;
@@ -573,7 +582,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       f.c0 = q / kBins * kCh + lane;
       f.bin_ok = slot < left_bins;
       f.k = static_cast<uint32_t>(k_abs + slot);
-      f.before = before;
+#pragma unroll
+      for (int h = 0; h < C::kBlocks; ++h) f.before[h] = before[h];
       const float2* xb = X + (f.bin_ok ? slot : 0);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -599,7 +609,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const uint4 pc[2] = {next.pc[0], next.pc[1]};
       const uint32_t k = next.k;
-      const uint32_t j1 = next.before;
+      uint32_t j1[C::kBlocks];
+#pragma unroll
+      for (int h = 0; h < C::kBlocks; ++h) j1[h] = next.before[h];
       const int steps = next.steps;
       // power-of-two scale: the stage's largest component to [2^13, 2^14)
       uint32_t top = 0;
@@ -610,29 +622,34 @@ __global__ void __launch_bounds__(kThreads, 1)
       int f = 14 + 253 - static_cast<int>(top >> 23);
       f = f < 1 ? 1 : (f > 253 ? 253 : f);
       const float sc = __uint_as_float(static_cast<uint32_t>(f) << 23);
-      uint32_t hw[2], ha[2], pf[2], pm[2];
+      uint32_t hw[2], ha[2], pf[2], pm[C::kBlocks][2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint64_t u = (static_cast<uint64_t>(pc[h].y) << 32) | pc[h].x;
         const uint64_t v = (static_cast<uint64_t>(pc[h].w) << 32) | pc[h].z;
         const uint64_t half = (v * k) >> 1;  // half a trial step, mod half a cycle
-        const uint64_t mid = (u + v * j1) * k + half;  // the pass centre
         constexpr uint64_t kRound = 0x80000000ull;
         hw[h] = static_cast<uint32_t>((half + kRound) >> 32);
         ha[h] = static_cast<uint32_t>(((half << 7) + kRound) >> 32);
         pf[h] = static_cast<uint32_t>(((half << 5) + kRound) >> 32);
-        pm[h] = static_cast<uint32_t>(mid >> 32);
+#pragma unroll
+        for (int i = 0; i < C::kBlocks; ++i)  // the blocks' centres
+          pm[i][h] = static_cast<uint32_t>(((u + v * j1[i]) * k + half) >> 32);
       }
-      float2 fc, fs, mc, ms;
+      float2 fc, fs, zr[C::kBlocks], zi[C::kBlocks];
       sincos2(pf[0], pf[1], fc, fs);
-      sincos2(pm[0], pm[1], mc, ms);
       const float2 xr = make_float2(x[0].x * sc, x[1].x * sc), xi = make_float2(x[0].y * sc, x[1].y * sc);
-      const float2 zr = __ffma2_rn(xr, mc, __fmul2_rn(make_float2(-xi.x, -xi.y), ms));
-      const float2 zi = __ffma2_rn(xr, ms, __fmul2_rn(xi, mc));
+#pragma unroll
+      for (int i = 0; i < C::kBlocks; ++i) {
+        float2 mc, ms;
+        sincos2(pm[i][0], pm[i][1], mc, ms);
+        zr[i] = __ffma2_rn(xr, mc, __fmul2_rn(make_float2(-xi.x, -xi.y), ms));
+        zi[i] = __ffma2_rn(xr, ms, __fmul2_rn(xi, mc));
+      }
       fetch(next);
       ok = warp_wait(&sm.pfree[s], ((n / T) & 1) ^ 1, abort_flag);
       if (!ok) break;
-      Table& tb = sm.table[s];
+      Table<C::kBlocks>& tb = sm.table[s];
       tb.hw[lane] = hw[0];
       tb.hw[lane + 32] = hw[1];
       tb.ha[lane] = ha[0];
@@ -641,10 +658,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       tb.fr[lane + 32] = fc.y;
       tb.fi[lane] = fs.x;
       tb.fi[lane + 32] = fs.y;
-      tb.xr[lane] = zr.x;
-      tb.xr[lane + 32] = zr.y;
-      tb.xi[lane] = zi.x;
-      tb.xi[lane + 32] = zi.y;
+#pragma unroll
+      for (int i = 0; i < C::kBlocks; ++i) {
+        tb.xr[i][lane] = zr[i].x;
+        tb.xr[i][lane + 32] = zr[i].y;
+        tb.xi[i][lane] = zi[i].x;
+        tb.xi[i][lane + 32] = zi[i].y;
+      }
       if (lane == 0) tb.steps = steps;
       if (lane == 0) sm.inv[n % (4 * C::kTables)] = __uint_as_float(static_cast<uint32_t>(254 - f) << 23);
       // Tables complete in order: a producer steps fewer than T stages at a
@@ -670,7 +690,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t ts = n % T;
       ok = warp_wait(&sm.pfull[ts], (n / T) & 1, abort_flag);
       if (!ok) break;
-      const Table& tb = sm.table[ts];
+      const Table<C::kBlocks>& tb = sm.table[ts];
       const int steps = tb.steps;
       if (rows) {
         // rows: lane = (b < 16, half of an octet of channels): Cb, Sb of four
@@ -729,7 +749,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         constexpr int kHalves = 32 / kNa;               // half octets at a time: 2, 4, 8
         static_assert(16 / C::kColTasks / kHalves == 2, "two rounds a task");
         const int al = (lane >> 1) % kNa;
-        const uint32_t mul = 2u * al + 1u;
+        const int blk = al / C::kAls;
+        const uint32_t mul = 2u * (al % C::kAls) + 1u;
         const int h0 = part * 2 * kHalves + 2 * (lane / (2 * kNa)) + (lane & 1);
         const bool live = part * 2 * kHalves < 4 * steps;  // (the round's first, so uniform)
         uint32_t hi[2][4][2], lo[2][4][2];  // [round][type][channel pair]
@@ -738,8 +759,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int e = 0; e < 2; ++e) {
             const int ch = 4 * (h0 + e * kHalves);
             const uint4 hv = *reinterpret_cast<const uint4*>(&tb.ha[ch]);
-            const float4 xrv = *reinterpret_cast<const float4*>(&tb.xr[ch]);
-            const float4 xiv = *reinterpret_cast<const float4*>(&tb.xi[ch]);
+            const float4 xrv = *reinterpret_cast<const float4*>(&tb.xr[blk][ch]);
+            const float4 xiv = *reinterpret_cast<const float4*>(&tb.xi[blk][ch]);
 #pragma unroll
             for (int p = 0; p < 2; ++p) {
               const float2 xr = p ? make_float2(xrv.z, xrv.w) : make_float2(xrv.x, xrv.y);

@@ -98,3 +98,20 @@ def test_dynamic_range(n_dm):
     for i in range(7):
         assert rel_l2(Y[:, i], ref[:, i]) <= TOL, i
     assert np.all(Y[:, 4] == 0) and np.all(np.isnan(Y[:, 7]))
+
+
+@pytest.mark.parametrize("n_dm", [2049, 4096, 5000, 9000])
+def test_calls_on_whole_blocks_agree_bit_for_bit(n_dm):
+    """Trials are centred in blocks of 2048 from the call's first: a call on
+    part of the list that starts at a whole block (as the streamed and batched
+    calls do) gives the whole call's bytes."""
+    n_chan, nb = 70, 5
+    with _plan(n_chan, 1 << 12, 0.25 * np.arange(n_dm)) as plan:
+        X = torch.randn((1, n_chan, nb, 2), device="cuda")
+        whole = torch.empty((1, n_dm, nb, 2), device="cuda")
+        plan.dedisperse_spectra_bins(X, nb, 1, 99, nb, 0, n_dm, whole, nb)
+        for j in range(0, n_dm, 2048):
+            n = min(2048, n_dm - j)
+            part = torch.empty((1, n, nb, 2), device="cuda")
+            plan.dedisperse_spectra_bins(X, nb, 1, 99, nb, j, n, part, nb)
+            assert torch.equal(part, whole[:, j:j + n]), j

@@ -27,7 +27,7 @@
 // tile the producers build serves 256 output columns, and every Z value is
 // written to shared memory once.
 //
-// Warp specialisation: warp 0 allocates tensor memory and one of its threads
+// Warp specialisation: warp 0 allocates tensor memory and an elected lane of it
 // issues the MMAs; 16 producer warps evaluate P (exact fixed-point phase,
 // MUFU sin/cos and short recurrences, hi/lo split) and Z = Q X for each stage
 // straight into the 128-byte-swizzled K-major shared layout the MMA
@@ -207,6 +207,13 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t ta, uint32_t tb, uint32_t (
 // (kind::f8f6f4).  A CTA pair's MMA, issued by the first CTA, reads each
 // CTA's 128 rows of A and its N / 2 rows of B at the same shared-memory
 // offsets and writes each CTA's 128 rows of D into its own tensor memory.
+// One lane of the converged warp, as a value the compiler keeps uniform.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
+
 template <int kPrec, bool kPair>
 __device__ __forceinline__ void mma16(uint32_t d, uint64_t adesc, uint64_t bdesc,
                                       uint32_t accum, uint32_t id) {
@@ -404,55 +411,66 @@ __global__ void __launch_bounds__(kThreads, 1) mac_tc_kernel(const MacArgs a) {
 
   if (warp == 0) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && rank == 0) {
-      uint32_t s = 0, p = 0;
+    if (rank == 0) {
+      // The whole warp keeps step and one elected lane issues, so that the
+      // descriptors come from uniform registers: issued by a lone thread of a
+      // divided warp an MMA takes up to 260 cycles to issue, twice as long as
+      // it runs (128 at N = 256).  16 beams x 4096 channels x 8192 trials x
+      // 129 bins in BF16 hi + lo 858 -> 793 us, 32 beams x 1024 channels x 4096
+      // trials x 1025 bins in FP16 (bound by the producers and the read-out)
+      // 1637 -> 1606 us.
+      const uint32_t el = elect_one();
+      const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+      const uint32_t ring = __shfl_sync(0xffffffffu, smem_u32(base), 0);
+      uint32_t st = 0, phase = 0, p = 0;
       bool issued = false, ok = true;
       for (int k = unit; k < a.n_bins && ok; k += n_units) {
         for (int it = 0; it < items_per_bin && ok; ++it, ++p) {
           // the epilogue (of both CTAs) has read the previous pass out of tensor memory
-          if (!wait_bar<kPair>(acc_empty, (p & 1) ^ 1, abort_flag)) {
-            ok = false;
-            break;
-          }
+          ok = __all_sync(0xffffffffu, wait_bar<kPair>(acc_empty, (p & 1) ^ 1, abort_flag));
+          if (!ok) break;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           // N of this pass: its a's times the group's beams
           const int n_a = pass_as(a.n_dm, (it % n_pass) * kDmsPass, kNA, kT);
           const uint32_t id = idesc<kPrec>(mma_as(n_a) * kBeams, kCtas * kM);
-          for (int t = 0; t < n_tiles; ++t, ++s) {
-            const uint32_t st = s % kStages;
-            if (!wait_bar<kPair>(&full[st], (s / kStages) & 1, abort_flag)) {
-              ok = false;
-              break;
-            }
+          for (int t = 0; t < n_tiles; ++t) {
+            ok = __all_sync(0xffffffffu, wait_bar<kPair>(&full[st], phase, abort_flag));
+            if (!ok) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const uint32_t stage = smem_u32(base + st * kStageBytes);
+            if (el) {
+              const uint64_t ad = smem_desc(ring + st * kStageBytes);
+              const uint64_t bd = smem_desc(ring + st * kStageBytes + kBOff);
+              constexpr uint32_t kTile = kTileA >> 4;  // descriptor steps of 16 bytes
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-              const uint64_t bd = smem_desc(stage + kBOff + kk * 32);
-              const uint32_t accum = (t > 0 || kk > 0) ? 1u : 0u;
-              mma16<kPrec, kPair>(tmem, smem_desc(stage + kk * 32), bd, accum, id);  // re, hi
-              mma16<kPrec, kPair>(tmem + kN, smem_desc(stage + kTileA + kk * 32), bd, accum,
-                                  id);  // im, hi
-              if (kHiLo) {
-                mma16<kPrec, kPair>(tmem, smem_desc(stage + 2 * kTileA + kk * 32), bd, 1u,
-                                    id);  // re, lo
-                mma16<kPrec, kPair>(tmem + kN, smem_desc(stage + 3 * kTileA + kk * 32), bd, 1u,
-                                    id);  // im, lo
+              for (int kk = 0; kk < 4; ++kk) {
+                const uint32_t accum = (t > 0 || kk > 0) ? 1u : 0u;
+                mma16<kPrec, kPair>(tm, ad + kk * 2, bd + kk * 2, accum, id);               // re, hi
+                mma16<kPrec, kPair>(tm + kN, ad + kTile + kk * 2, bd + kk * 2, accum, id);  // im, hi
+                if (kHiLo) {
+                  mma16<kPrec, kPair>(tm, ad + 2 * kTile + kk * 2, bd + kk * 2, 1u, id);
+                  mma16<kPrec, kPair>(tm + kN, ad + 3 * kTile + kk * 2, bd + kk * 2, 1u, id);
+                }
               }
+              mma_commit<kPair>(&empty[st]);
             }
             issued = true;
-            mma_commit<kPair>(&empty[st]);
+            if (++st == kStages) {
+              st = 0;
+              phase ^= 1;
+            }
+            __syncwarp();
           }
           if (!ok) break;
-          mma_commit<kPair>(acc_full);
+          if (el) mma_commit<kPair>(acc_full);
+          __syncwarp();
         }
       }
       if (!ok) {
         *abort_flag = 1;
-        if (a.status) atomicExch(a.status, FDD_ERR_TIMEOUT);
+        if (a.status && lane == 0) atomicExch(a.status, FDD_ERR_TIMEOUT);
       }
-      if (issued) {  // drain this thread's MMAs before tensor memory is freed
-        mma_commit_one<kPair>(drain);
+      if (issued) {  // drain this warp's MMAs before tensor memory is freed
+        if (el) mma_commit_one<kPair>(drain);
         volatile int never = 0;
         mbar_wait(drain, 0, &never);
       }

@@ -49,6 +49,11 @@
 // store from registers used at once (317), one octet per task (353), the MMA
 // loop unrolled by stage (334: instruction fetch), lo hi as an MMA of its own
 // (307).
+// Several series share a pass's rows (two or, up to 1024 trials, four), each
+// with its own columns and scales and the bits it has alone: 1024 channels x
+// 4096 (bin, series) of 1024 trials 256 us each alone, 177 in twos, 151 in
+// fours; of 2048 trials 311 and 267; two series of 387 channels x 701 trials x
+// 4001 bins 214 and 167.
 #include <atomic>
 
 #include <cuda_fp16.h>
@@ -99,16 +104,22 @@ constexpr int kPrepFirst = kMmaWarp + 1, kPrepWarps = 2;
 constexpr int kProdFirst = kPrepFirst + kPrepWarps, kProdWarps = 13;
 constexpr int kThreads = 32 * (kProdFirst + kProdWarps);
 
-// kNa: al's a pass can hold; kBins: bins a CTA works on at a time (their
-// accumulators share the epilogue's registers: kNa * kBins = 16).
-template <int kNa>
+// A pass's columns are kBlocks blocks of kAls al's that share its rows: blocks
+// of trials of one series (each with its own centre), or the same trials of
+// kBlocks series (kSeries).  kNa: al's in all; kBins: bins a CTA works on at a
+// time (their accumulators share the epilogue's registers: kNa * kBins = 16).
+template <int kAls_, int kBlocks_, bool kSeries_>
 struct Cfg {
+  static constexpr int kAls = kAls_, kBlocks = kBlocks_, kNa = kAls * kBlocks;
+  static constexpr bool kSeries = kSeries_;
+  static constexpr int kSets = kSeries ? kBlocks : 1;     // spectra of a pass
+  static constexpr int kCentres = kSeries ? 1 : kBlocks;  // and centres
+  static constexpr int kPassTrials = kPairTrials * kAls * kCentres;
   static constexpr int kBins = 16 / kNa;
-  static constexpr int kBlocks = kNa == 16 ? 2 : 1;  // blocks of trials of a pass
-  static constexpr int kAls = kNa / kBlocks;         // al's of each
   static constexpr int kN = 4 * kNa;          // columns
   static constexpr int kStages = kNa == 16 ? 4 : 5;
-  static constexpr int kTables = kNa == 8 ? 6 : 8;  // tables run further ahead than operands
+  // (tables run further ahead than operands)
+  static constexpr int kTables = kNa == 8 ? 7 - kBlocks : kBlocks == 4 ? 6 : 8;
   static constexpr uint32_t kATile = kRows * kCh * 2;  // 8 KB per term
   static constexpr uint32_t kBTile = kN * kCh * 2;
   static constexpr uint32_t kStageBytes = 2 * (kATile + kBTile);
@@ -119,6 +130,8 @@ struct Cfg {
   static constexpr int kTasks = 4 + kColTasks;
   static_assert((kProdWarps + kTasks - 1) / kTasks < kStages, "a producer's step between tasks");
   static constexpr uint32_t kTmemCols = kNa == 4 ? 256 : 512;
+  static_assert(kSeries || kBlocks == 1 || kAls == kBlockAls, "trials in whole blocks");
+  static_assert(kAls % 4 == 0, "the epilogue's four al's have one scale");
   static_assert(kStages * 2 * kN <= static_cast<int>(kTmemCols), "accumulator ring");
 };
 
@@ -132,13 +145,12 @@ struct Table {
   int steps;               // K steps of 16 channels the MMAs read
   int pad[3];
 };
-template <int kNa>
+template <class C>
 struct Smem {
-  using C = Cfg<kNa>;
   alignas(128) unsigned char stage[C::kStages][C::kStageBytes];
   alignas(16) float4 xch[8][kRows];  // epilogue exchange: A_+, A_- of a row (or B_+, B_-)
   alignas(16) Table<C::kBlocks> table[C::kTables];
-  float inv[4 * C::kTables];  // undoes a stage's scale (read by the epilogue, well after the table)
+  float inv[4 * C::kTables][C::kSets];  // undoes a stage's scales (read by the epilogue, well after the table)
   uint64_t pfull[C::kTables], pfree[C::kTables];  // table written; every producer has read it
   uint64_t full[C::kStages], done[C::kStages];   // operands written; MMAs complete
   uint64_t xbar, drain;
@@ -232,24 +244,26 @@ __device__ __forceinline__ void sincos2(uint32_t p0, uint32_t p1, float2& cs, fl
 // An item of the launch: bins k0 .. k0 + kBins - 1 of one set of spectra and
 // the pass of up to 256 kNa trials from j_p.
 struct Item {
-  int set;  // series, or batch set
+  int set;  // (first) series, or batch set
   int k0, j_p;
   int n_a;  // al's of the pass with trials: whole blocks, then the last one's
 };
-template <int kNa>
+template <class C>
 __host__ __device__ inline int n_passes(int n_dm) {
-  return (n_dm + kPairTrials * kNa - 1) / (kPairTrials * kNa);
+  return (n_dm + C::kPassTrials - 1) / C::kPassTrials;
 }
-// al's of block h of a pass with n_a al's
+// al's of block h of a pass with n_a al's (a series')
+template <class C>
 __device__ __forceinline__ int block_als(int n_a, int h) {
+  if (C::kSeries) return n_a;
   const int left = n_a - h * kBlockAls;
   return left < 0 ? 0 : left < kBlockAls ? left : kBlockAls;
 }
-template <int kNa>
+template <class C>
 __device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, int n_sets, int item) {
   Item q;
   int local, n_dm, groups;
-  if (sets) {
+  if (!C::kSeries && sets) {
     int lo = 0, hi = n_sets - 1;  // last set with item_begin <= item
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -260,30 +274,32 @@ __device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, i
     n_dm = sets[lo].args.n_dm;
     groups = sets[lo].n_bin_tiles;
   } else {
-    groups = (a.n_bins + Cfg<kNa>::kBins - 1) / Cfg<kNa>::kBins;
+    groups = (a.n_bins + C::kBins - 1) / C::kBins;
     n_dm = a.n_dm;
-    const int per_series = groups * n_passes<kNa>(n_dm);
-    q.set = item / per_series;
-    local = item - q.set * per_series;
+    const int per_set = groups * n_passes<C>(n_dm);
+    q.set = item / per_set;
+    local = item - q.set * per_set;
+    q.set *= C::kSets;
   }
   const int p = local / groups;
-  q.k0 = (local - p * groups) * Cfg<kNa>::kBins;
-  q.j_p = p * kPairTrials * kNa;
+  q.k0 = (local - p * groups) * C::kBins;
+  q.j_p = p * C::kPassTrials;
   const int als = (n_dm - q.j_p + kPairTrials - 1) / kPairTrials;
-  q.n_a = als < kNa ? als : kNa;
+  constexpr int kMost = C::kAls * C::kCentres;
+  q.n_a = als < kMost ? als : kMost;
   return q;
 }
 
-template <int kNa>
+template <class C>
 __global__ void __launch_bounds__(kThreads, 1)
     mac_split_kernel(const MacArgs a, const BatchSet* sets, int n_sets, int n_items) {
-  using C = Cfg<kNa>;
+  constexpr int kNa = C::kNa;
   constexpr int kBins = C::kBins;
   constexpr int kN = C::kN;
   constexpr int S = C::kStages;
   constexpr int T = C::kTables;
   extern __shared__ unsigned char smem_raw[];
-  Smem<kNa>& sm = *reinterpret_cast<Smem<kNa>*>(
+  Smem<C>& sm = *reinterpret_cast<Smem<C>*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   volatile int* abort_flag = &sm.abort_flag;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);
@@ -356,11 +372,14 @@ __global__ void __launch_bounds__(kThreads, 1)
           const uint32_t s = n % S;
           ok = ok && warp_wait(&sm.done[s], (n / S) & 1, abort_flag);
           if (!ok) break;
-          const float hv = sm.inv[n % (4 * C::kTables)];
+          float hv[C::kSets];
+#pragma unroll
+          for (int i = 0; i < C::kSets; ++i) hv[i] = sm.inv[n % (4 * C::kTables)][i];
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-          const float2 inv = make_float2(hv, hv);
 #pragma unroll
           for (int h = 0; h < kNa / 4; ++h) {
+            const float hs = hv[C::kSeries ? 4 * h / C::kAls : 0];
+            const float2 inv = make_float2(hs, hs);
 #pragma unroll
             for (int t = 0; t < 4; t += 2) {
               // [type t, t + 1: hi hi; the small products of both][al]
@@ -391,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // with Sb: through shared memory, eight (al, bin) units at a time; the
       // thread of a Cb row then makes the trials of s = +, that of the Sb row
       // of the same b those of s = -.
-      const Item q = decode<kNa>(a, sets, n_sets, item);
+      const Item q = decode<C>(a, sets, n_sets, item);
       const MacArgs& m = sets ? sets[q.set].args : a;
       const int64_t dm_stride = m.y_dm_stride;
       const int n_dm = m.n_dm, n_bins = m.n_bins, out_kind = m.out_kind;
@@ -402,10 +421,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool whole = q.k0 + kBins <= n_bins;
 #pragma unroll
       for (int half = 0; half < 2; ++half) {
-        constexpr int kAls = 8 / kBins;  // al's of a half
+        constexpr int kHalfAls = 8 / kBins;  // al's of a half
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
-          const int al = half * kAls + u / kBins, sl = u % kBins;
+          const int al = half * kHalfAls + u / kBins, sl = u % kBins;
           const float m1 = (al & 1) ? acc[sl][0][al / 2].y : acc[sl][0][al / 2].x;
           const float m2 = (al & 1) ? acc[sl][1][al / 2].y : acc[sl][1][al / 2].x;
           const float m3 = (al & 1) ? acc[sl][2][al / 2].y : acc[sl][2][al / 2].x;
@@ -414,9 +433,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (!(ok = exchange_sync())) break;
 #pragma unroll 1
-        for (int i = 0; i < kAls; ++i) {
-          const int al = half * kAls + i;
-          if (al >= q.n_a) break;
+        for (int i = 0; i < kHalfAls; ++i) {
+          const int al = half * kHalfAls + i;
+          if (C::kSeries ? al % C::kAls >= q.n_a : al >= q.n_a) continue;
           float2 y[2][kBins];  // t = +, -
 #pragma unroll
           for (int sl = 0; sl < kBins; ++sl) {
@@ -427,14 +446,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             y[1][sl] = make_float2((A.x + B.y) * scale, real_only ? 0.f : (A.y - B.x) * scale);
           }
           // trial of (s, al, t, b)
-          const int h = al / kBlockAls, step = 128 * (al % kBlockAls) + 64;
-          const int jc = q.j_p + kPairTrials * kBlockAls * h +
-                         kPairTrials / 2 * block_als(q.n_a, h) + (is_c ? step : -step);
+          const int h = al / C::kAls, step = 128 * (al % C::kAls) + 64;
+          const int jc = q.j_p + (C::kSeries ? 0 : kPairTrials * kBlockAls * h) +
+                         kPairTrials / 2 * block_als<C>(q.n_a, h) + (is_c ? step : -step);
+          const int64_t off_h = off + (C::kSeries ? h * m.y_series_stride : 0);
 #pragma unroll
           for (int t = 0; t < 2; ++t) {
             const int j = t == 0 ? jc + b : jc - 1 - b;
             if (j >= n_dm) continue;
-            const int64_t o = off + static_cast<int64_t>(j) * dm_stride;
+            const int64_t o = off_h + static_cast<int64_t>(j) * dm_stride;
             if (out_kind == 2) {
               float* Y = static_cast<float*>(Yv) + o;
               float pw[kBins];
@@ -538,10 +558,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     // lane = channels lane and lane + 32 of the stage; the next stage's loads
     // fly while this one's table is made and waits for its place
     struct Fetched {
-      float2 x[2];
+      float2 x[C::kSets][2];
       uint4 pc[2];      // u_lo, u_hi, v_lo, v_hi
       uint32_t k;       // absolute bin
-      uint32_t before[C::kBlocks];  // Jc - 1/2: the trial below each block's centre
+      uint32_t before[C::kCentres];  // Jc - 1/2: the trial below each block's centre
       int c0;           // this lane's first channel
       int steps;        // K steps of the stage
       bool bin_ok;
@@ -551,9 +571,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     int q = p;  // stage within the item
     // the item at hand, in registers: its spectra, constants and phases' origin
     int cur = -1, left_bins = 0, k_abs = 0;
-    uint32_t before[C::kBlocks] = {};
+    uint32_t before[C::kCentres] = {};
     const float2* X = nullptr;
-    int64_t xs = 0;
+    int64_t xs = 0, set_stride = 0;
     const PhaseConst* pcs = nullptr;
     auto fetch = [&](Fetched& f) {
       // The loads are unconditional, from clamped addresses, and idle channels
@@ -564,17 +584,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         item += gridDim.x;
       }
       if (item != cur && item < n_items) {
-        const Item it = decode<kNa>(a, sets, n_sets, item);
+        const Item it = decode<C>(a, sets, n_sets, item);
         const MacArgs& m = sets ? sets[it.set].args : a;
         cur = item;
         left_bins = m.n_bins - it.k0;
         k_abs = m.k_begin + it.k0;
 #pragma unroll
-        for (int h = 0; h < C::kBlocks; ++h)
+        for (int h = 0; h < C::kCentres; ++h)
           before[h] = static_cast<uint32_t>(m.j_begin + it.j_p + kPairTrials * kBlockAls * h +
-                                            kPairTrials / 2 * block_als(it.n_a, h) - 1);
+                                            kPairTrials / 2 * block_als<C>(it.n_a, h) - 1);
         X = m.X + (sets ? 0 : static_cast<int64_t>(it.set) * m.x_series_stride) + it.k0;
         xs = m.x_chan_stride;
+        set_stride = m.x_series_stride;
         pcs = m.pc;
       }
       const int slot = q % kBins;
@@ -583,7 +604,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       f.bin_ok = slot < left_bins;
       f.k = static_cast<uint32_t>(k_abs + slot);
 #pragma unroll
-      for (int h = 0; h < C::kBlocks; ++h) f.before[h] = before[h];
+      for (int h = 0; h < C::kCentres; ++h) f.before[h] = before[h];
       const float2* xb = X + (f.bin_ok ? slot : 0);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -591,9 +612,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
                      : "=r"(f.pc[h].x), "=r"(f.pc[h].y), "=r"(f.pc[h].z), "=r"(f.pc[h].w)
                      : "l"(pcs + c));
-        asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];"
-                     : "=f"(f.x[h].x), "=f"(f.x[h].y)
-                     : "l"(xb + static_cast<int64_t>(c) * xs));
+#pragma unroll
+        for (int i = 0; i < C::kSets; ++i)
+          asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];"
+                       : "=f"(f.x[i][h].x), "=f"(f.x[i][h].y)
+                       : "l"(xb + i * set_stride + static_cast<int64_t>(c) * xs));
       }
       q += kPrepWarps;
     };
@@ -601,28 +624,33 @@ __global__ void __launch_bounds__(kThreads, 1)
     fetch(next);
     for (uint32_t n = p; n < total; n += kPrepWarps) {
       const uint32_t s = n % T;
-      float2 x[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const bool use = next.bin_ok && next.c0 + 32 * h < n_chan;
-        x[h] = use ? next.x[h] : make_float2(0.f, 0.f);
-      }
       const uint4 pc[2] = {next.pc[0], next.pc[1]};
       const uint32_t k = next.k;
-      uint32_t j1[C::kBlocks];
+      uint32_t j1[C::kCentres];
 #pragma unroll
-      for (int h = 0; h < C::kBlocks; ++h) j1[h] = next.before[h];
+      for (int h = 0; h < C::kCentres; ++h) j1[h] = next.before[h];
       const int steps = next.steps;
       // power-of-two scale: the stage's largest component to [2^13, 2^14)
-      uint32_t top = 0;
+      float2 xr[C::kSets], xi[C::kSets];
+      int f[C::kSets];
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        top = max(top, max(__float_as_uint(x[h].x) & 0x7FFFFFFFu, __float_as_uint(x[h].y) & 0x7FFFFFFFu));
-      top = __reduce_max_sync(0xffffffffu, top);
-      int f = 14 + 253 - static_cast<int>(top >> 23);
-      f = f < 1 ? 1 : (f > 253 ? 253 : f);
-      const float sc = __uint_as_float(static_cast<uint32_t>(f) << 23);
-      uint32_t hw[2], ha[2], pf[2], pm[C::kBlocks][2];
+      for (int i = 0; i < C::kSets; ++i) {
+        float2 x[2];
+        uint32_t top = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool use = next.bin_ok && next.c0 + 32 * h < n_chan;
+          x[h] = use ? next.x[i][h] : make_float2(0.f, 0.f);
+          top = max(top, max(__float_as_uint(x[h].x) & 0x7FFFFFFFu, __float_as_uint(x[h].y) & 0x7FFFFFFFu));
+        }
+        top = __reduce_max_sync(0xffffffffu, top);
+        f[i] = 14 + 253 - static_cast<int>(top >> 23);
+        f[i] = f[i] < 1 ? 1 : (f[i] > 253 ? 253 : f[i]);
+        const float sc = __uint_as_float(static_cast<uint32_t>(f[i]) << 23);
+        xr[i] = make_float2(x[0].x * sc, x[1].x * sc);
+        xi[i] = make_float2(x[0].y * sc, x[1].y * sc);
+      }
+      uint32_t hw[2], ha[2], pf[2], pm[C::kCentres][2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint64_t u = (static_cast<uint64_t>(pc[h].y) << 32) | pc[h].x;
@@ -633,18 +661,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         ha[h] = static_cast<uint32_t>(((half << 7) + kRound) >> 32);
         pf[h] = static_cast<uint32_t>(((half << 5) + kRound) >> 32);
 #pragma unroll
-        for (int i = 0; i < C::kBlocks; ++i)  // the blocks' centres
+        for (int i = 0; i < C::kCentres; ++i)  // the blocks' centres
           pm[i][h] = static_cast<uint32_t>(((u + v * j1[i]) * k + half) >> 32);
       }
       float2 fc, fs, zr[C::kBlocks], zi[C::kBlocks];
       sincos2(pf[0], pf[1], fc, fs);
-      const float2 xr = make_float2(x[0].x * sc, x[1].x * sc), xi = make_float2(x[0].y * sc, x[1].y * sc);
+      float2 mc, ms;
 #pragma unroll
       for (int i = 0; i < C::kBlocks; ++i) {
-        float2 mc, ms;
-        sincos2(pm[i][0], pm[i][1], mc, ms);
-        zr[i] = __ffma2_rn(xr, mc, __fmul2_rn(make_float2(-xi.x, -xi.y), ms));
-        zi[i] = __ffma2_rn(xr, ms, __fmul2_rn(xi, mc));
+        if (i < C::kCentres) sincos2(pm[i % C::kCentres][0], pm[i % C::kCentres][1], mc, ms);
+        const int e = C::kSeries ? i : 0;
+        zr[i] = __ffma2_rn(xr[e], mc, __fmul2_rn(make_float2(-xi[e].x, -xi[e].y), ms));
+        zi[i] = __ffma2_rn(xr[e], ms, __fmul2_rn(xi[e], mc));
       }
       fetch(next);
       ok = warp_wait(&sm.pfree[s], ((n / T) & 1) ^ 1, abort_flag);
@@ -666,7 +694,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         tb.xi[i][lane + 32] = zi[i].y;
       }
       if (lane == 0) tb.steps = steps;
-      if (lane == 0) sm.inv[n % (4 * C::kTables)] = __uint_as_float(static_cast<uint32_t>(254 - f) << 23);
+      if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < C::kSets; ++i)
+          sm.inv[n % (4 * C::kTables)][i] = __uint_as_float(static_cast<uint32_t>(254 - f[i]) << 23);
+      }
       // Tables complete in order: a producer steps fewer than T stages at a
       // time, so the table T stages back is then complete when it waits for
       // one (a wait by parity sees only whether the count is odd).
@@ -813,18 +845,37 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-template <int kNa>
-const void* split_fn() {
-  return reinterpret_cast<const void*>(&mac_split_kernel<kNa>);
-}
-template <int kNa>
-constexpr int split_smem() { return static_cast<int>(sizeof(Smem<kNa>)) + 128; }
+// The passes' forms: one series with up to 1024, 2048 or 4096 trials a pass,
+// or two or four series that share the rows of up to 1024, two of up to 2048.
+enum Form { kUpTo1024, kUpTo2048, kUpTo4096, kTwoUpTo1024, kFourUpTo1024, kTwoUpTo2048, kForms };
 
-// al's a pass must hold for n_dm trials: up to four, eight or sixteen (1024,
-// 2048, 4096 trials a pass).
-int capacity(int n_dm) {
+struct FormInfo {
+  const void* fn;
+  int smem, sets, bins, pass_trials;
+};
+template <class C>
+FormInfo form_info() {
+  return {reinterpret_cast<const void*>(&mac_split_kernel<C>), static_cast<int>(sizeof(Smem<C>)) + 128,
+          C::kSets, C::kBins, C::kPassTrials};
+}
+FormInfo form_info(Form f) {
+  switch (f) {
+    case kUpTo1024: return form_info<Cfg<4, 1, false>>();
+    case kUpTo2048: return form_info<Cfg<8, 1, false>>();
+    case kUpTo4096: return form_info<Cfg<8, 2, false>>();
+    case kTwoUpTo1024: return form_info<Cfg<4, 2, true>>();
+    case kFourUpTo1024: return form_info<Cfg<4, 4, true>>();
+    default: return form_info<Cfg<8, 2, true>>();
+  }
+}
+
+// The form for n_dm trials of n_series (at least its sets) series.  The rows
+// take most of a stage, so the widest pass that the trials or series fill.
+Form form_for(int n_dm, int n_series) {
   const int total = (n_dm + kPairTrials - 1) / kPairTrials;
-  return total <= 4 ? 4 : total <= 8 ? 8 : 16;
+  if (total > 8) return kUpTo4096;
+  if (total > 4) return n_series >= 2 ? kTwoUpTo2048 : kUpTo2048;
+  return n_series >= 4 ? kFourUpTo1024 : n_series >= 2 ? kTwoUpTo1024 : kUpTo1024;
 }
 
 constexpr int kMaxDevices = 64;
@@ -844,18 +895,13 @@ cudaError_t sm_count(int* out) {
   return cudaSuccess;
 }
 
-cudaError_t launch_split(const MacArgs& a, const BatchSet* sets, int n_sets, int n_items, int cap,
-                         int n_ctas, cudaStream_t s) {
+cudaError_t launch_split(const MacArgs& a, const BatchSet* sets, int n_sets, int n_items,
+                         const FormInfo& f, int n_ctas, cudaStream_t s) {
   MacArgs args = a;
   void* params[] = {&args, &sets, &n_sets, &n_items};
   const dim3 grid(n_items < n_ctas ? n_items : n_ctas);
   note_launches(1);
-  switch (cap) {
-    case 4: return cudaLaunchKernel(split_fn<4>(), grid, dim3(kThreads), params, split_smem<4>(), s);
-    case 8: return cudaLaunchKernel(split_fn<8>(), grid, dim3(kThreads), params, split_smem<8>(), s);
-    default:
-      return cudaLaunchKernel(split_fn<16>(), grid, dim3(kThreads), params, split_smem<16>(), s);
-  }
+  return cudaLaunchKernel(f.fn, grid, dim3(kThreads), params, f.smem, s);
 }
 
 constexpr long long kMaxItems = 0x7FFF0000LL;  // item numbers, stepped by the grid, stay in an int
@@ -863,57 +909,58 @@ constexpr long long kMaxItems = 0x7FFF0000LL;  // item numbers, stepped by the g
 }  // namespace
 
 size_t mac_split_smem_bytes() {
-  return split_smem<4>() > split_smem<8>()
-             ? (split_smem<4>() > split_smem<16>() ? split_smem<4>() : split_smem<16>())
-             : (split_smem<8>() > split_smem<16>() ? split_smem<8>() : split_smem<16>());
+  int most = 0;
+  for (int f = 0; f < kForms; ++f) {
+    const int b = form_info(static_cast<Form>(f)).smem;
+    if (b > most) most = b;
+  }
+  return most;
 }
 
 cudaError_t mac_split_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(split_fn<4>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       split_smem<4>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(split_fn<8>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             split_smem<8>());
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(split_fn<16>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             split_smem<16>());
+  cudaError_t e = cudaSuccess;
+  for (int f = 0; f < kForms && e == cudaSuccess; ++f) {
+    const FormInfo i = form_info(static_cast<Form>(f));
+    e = cudaFuncSetAttribute(i.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, i.smem);
+  }
   return e;
 }
 
 void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes) {
-  const int cap = capacity(max_n_dm);
-  const int bins = 16 / cap;
-  *bin_groups = static_cast<int>((n_bins + bins - 1) / bins);
-  *passes = cap == 4 ? n_passes<4>(n_dm) : cap == 8 ? n_passes<8>(n_dm) : n_passes<16>(n_dm);
+  const FormInfo f = form_info(form_for(max_n_dm, 1));
+  *bin_groups = static_cast<int>((n_bins + f.bins - 1) / f.bins);
+  *passes = (n_dm + f.pass_trials - 1) / f.pass_trials;
 }
 
 cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
                                    int max_n_dm, int n_ctas, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   if (n_items > kMaxItems) return cudaErrorInvalidConfiguration;
-  return launch_split(MacArgs{}, d_sets, n_sets, static_cast<int>(n_items), capacity(max_n_dm),
-                      n_ctas, s);
+  return launch_split(MacArgs{}, d_sets, n_sets, static_cast<int>(n_items),
+                      form_info(form_for(max_n_dm, 1)), n_ctas, s);
 }
 
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
   int n_sms = 0;
   cudaError_t e = sm_count(&n_sms);
   if (e != cudaSuccess) return e;
-  int groups, passes;
-  mac_split_batch_shape(a.n_dm, a.n_dm, a.n_bins, &groups, &passes);
-  const long long per_series = static_cast<long long>(groups) * passes;
-  if (per_series > kMaxItems) return cudaErrorInvalidConfiguration;
-  // (series in blocks whose items can be numbered in an int)
   const size_t y_elem = a.out_kind == 2 ? sizeof(float) : sizeof(float2);
-  const long long block = kMaxItems / per_series;
-  for (long long s0 = 0; s0 < a.n_series; s0 += block) {
+  // series in groups that share passes, then the rest by themselves
+  for (int s0 = 0; s0 < a.n_series;) {
+    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0));
+    const long long per_set = static_cast<long long>((a.n_bins + f.bins - 1) / f.bins) *
+                              ((a.n_dm + f.pass_trials - 1) / f.pass_trials);
+    if (per_set > kMaxItems) return cudaErrorInvalidConfiguration;
+    // (as many as leave item numbers in an int)
+    long long sets = (a.n_series - s0) / f.sets;
+    if (sets > kMaxItems / per_set) sets = kMaxItems / per_set;
     MacArgs c = a;
-    c.n_series = static_cast<int>(a.n_series - s0 < block ? a.n_series - s0 : block);
+    c.n_series = static_cast<int>(sets) * f.sets;
     c.X = a.X + s0 * a.x_series_stride;
     c.Y = static_cast<char*>(a.Y) + y_elem * static_cast<size_t>(s0 * a.y_series_stride);
-    e = launch_split(c, nullptr, 0, static_cast<int>(per_series * c.n_series), capacity(a.n_dm),
-                     n_sms, s);
+    e = launch_split(c, nullptr, 0, static_cast<int>(per_set * sets), f, n_sms, s);
     if (e != cudaSuccess) return e;
+    s0 += c.n_series;
   }
   return cudaSuccess;
 }

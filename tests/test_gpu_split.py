@@ -115,3 +115,25 @@ def test_calls_on_whole_blocks_agree_bit_for_bit(n_dm):
             part = torch.empty((1, n, nb, 2), device="cuda")
             plan.dedisperse_spectra_bins(X, nb, 1, 99, nb, j, n, part, nb)
             assert torch.equal(part, whole[:, j:j + n]), j
+
+
+@pytest.mark.parametrize("n_dm", [257, 1024, 1300, 2048, 2304])
+@pytest.mark.parametrize("n_series", [2, 3, 5, 7])
+def test_series_sharing_passes_equal_each_alone(n_series, n_dm):
+    """Two or four series share a pass (up to 1024 trials; two up to 2048):
+    the same bits as each series by itself, whatever the others' scale."""
+    n_chan, L, nb, b0 = 81, 1 << 12, 9, 1500
+    rng = np.random.default_rng(n_series + n_dm)
+    X = (rng.standard_normal((n_series, n_chan, nb)) +
+         1j * rng.standard_normal((n_series, n_chan, nb)))
+    X *= np.array([1.0, 1e-12, 3e9, 1.0, 0.0, 7.0, 1e20])[:n_series, None, None]
+    dX = complex_to_device(X.astype(np.complex64), nb)
+    with _plan(n_chan, L, 3.7 + 0.31 * np.arange(n_dm)) as plan:
+        dY = torch.full((n_series, n_dm, nb, 2), 7.0, device="cuda")
+        plan.dedisperse_spectra_bins(dX, nb, n_series, b0, nb, 0, n_dm, dY, nb)
+        for s in range(n_series):
+            one = torch.full((n_dm, nb, 2), 7.0, device="cuda")
+            plan.dedisperse_spectra_bins(dX[s].contiguous(), nb, 1, b0, nb, 0, n_dm, one, nb)
+            assert torch.equal(dY[s], one), s
+        torch.cuda.synchronize()
+        plan.query()

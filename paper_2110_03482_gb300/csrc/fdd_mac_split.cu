@@ -36,24 +36,27 @@
 // phase constants into a table per stage, thirteen evaluate and split rows and
 // columns into shared memory (K-major core matrices), one issues the MMAs,
 // four add the stages up and store.  4096 bins x 1024 channels x 2048 trials
-// take 305 us, against 1185 us for the FP32 multiply-adds (three real products
+// take 300 us, against 1185 us for the FP32 multiply-adds (three real products
 // per complex one) at 0.75 of the FP32 peak; 301 bins x 4096 channels x 8192
-// trials 218 against 1292 us; 701 trials of 387 channels 216 against 560 us.
+// trials 210 against 1292 us; 701 trials of 2 x 387 channels 140 against 560 us.
 // What bounds it: writing and reading the operands in shared memory (71 % of
 // its cycles, the MMAs' reads and the producers' stores about equal) beside
 // 50 warp instructions per bin and channel (61 % of the issue slots), most of
 // them phasors and splits of the 128 rows.  Hence the wide passes: the rows
-// serve all columns of a pass, up to 4096 trials.
+// serve all columns of a pass, up to 4096 trials of one series.  Several series
+// share them too (two, or four up to 1024 trials), each with its own columns
+// and scales and the bits it has alone: 4096 (bin, series) x 1024 channels of
+// 2048 trials take 300 us each alone and 227 in twos; of 1024 trials 256, 160
+// in twos and 130 in fours.
+// The four adding warps do not take stages while they store an item, so that
+// must be short: Cb and Sb of a b are rows of one warp, which exchanges them
+// by shuffles (through shared memory and barriers of the four warps: 311 us
+// for the first figure, 218, 167, and 267 for two series).
 // Measured and dropped: results kept until a whole octet is done in wider
 // stores with fewer warps (16 warps of 128 registers: 344 us), four bytes per
 // store from registers used at once (317), one octet per task (353), the MMA
 // loop unrolled by stage (334: instruction fetch), lo hi as an MMA of its own
-// (307).
-// Several series share a pass's rows (two or, up to 1024 trials, four), each
-// with its own columns and scales and the bits it has alone: 1024 channels x
-// 4096 (bin, series) of 1024 trials 256 us each alone, 177 in twos, 151 in
-// fours; of 2048 trials 311 and 267; two series of 387 channels x 701 trials x
-// 4001 bins 214 and 167.
+// (307), four more warps to store, with the producers at 80 registers (335).
 #include <atomic>
 
 #include <cuda_fp16.h>
@@ -91,7 +94,12 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 }
 
 constexpr int kCh = 64;     // channels per stage (four K steps of 16)
-constexpr int kRows = 128;  // Cb | Sb of 64 b's
+constexpr int kRows = 128;  // Cb, Sb of 64 b's: sixteen b's Cb, then their Sb, and so on
+// Up to this many channels the columns' phasors come from the Taylor series,
+// too (2.1e-7 to 2.4e-7 of the result instead of 3.2e-7): over so few the
+// FP32 multiply-adds' sums lost little, and reached 3.0e-7.  A call of 63
+// channels x 277 trials x 347 bins takes 13 us either way.
+constexpr int kFewChan = 128;
 constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's
 constexpr int kBlockAls = 8;      // al's of a whole block (2048 trials)
 
@@ -119,7 +127,7 @@ struct Cfg {
   static constexpr int kN = 4 * kNa;          // columns
   static constexpr int kStages = kNa == 16 ? 4 : 5;
   // (tables run further ahead than operands)
-  static constexpr int kTables = kNa == 8 ? 7 - kBlocks : kBlocks == 4 ? 6 : 8;
+  static constexpr int kTables = 8;
   static constexpr uint32_t kATile = kRows * kCh * 2;  // 8 KB per term
   static constexpr uint32_t kBTile = kN * kCh * 2;
   static constexpr uint32_t kStageBytes = 2 * (kATile + kBTile);
@@ -129,10 +137,17 @@ struct Cfg {
   static constexpr int kColTasks = kNa / 4;
   static constexpr int kTasks = 4 + kColTasks;
   static_assert((kProdWarps + kTasks - 1) / kTasks < kStages, "a producer's step between tasks");
-  static constexpr uint32_t kTmemCols = kNa == 4 ? 256 : 512;
+  // tensor memory: a ring of accumulators, then the sums of the kOutBins
+  // bins that are stored together (sixteen (al, bin) units of four a slot; a
+  // wide pass of one series stores from registers and keeps the longer ring)
+  static constexpr int kSlots = kNa < 16 ? 1 : kSeries ? 2 : 0;
+  static constexpr int kOutBins = kSlots > 1 ? kSlots * kBins : kBins;
+  static constexpr int kAccs = kSlots > 1 ? 3 : kStages;
+  static constexpr uint32_t kPark = kAccs * 2 * kN;
+  static_assert(kPark + kSlots * 64 <= 512 && kAccs <= kStages, "tensor memory");
+  static constexpr uint32_t kTmemCols = 512;
   static_assert(kSeries || kBlocks == 1 || kAls == kBlockAls, "trials in whole blocks");
   static_assert(kAls % 4 == 0, "the epilogue's four al's have one scale");
-  static_assert(kStages * 2 * kN <= static_cast<int>(kTmemCols), "accumulator ring");
 };
 
 // Per stage: what the producers need of each channel.
@@ -148,12 +163,12 @@ struct Table {
 template <class C>
 struct Smem {
   alignas(128) unsigned char stage[C::kStages][C::kStageBytes];
-  alignas(16) float4 xch[8][kRows];  // epilogue exchange: A_+, A_- of a row (or B_+, B_-)
   alignas(16) Table<C::kBlocks> table[C::kTables];
   float inv[4 * C::kTables][C::kSets];  // undoes a stage's scales (read by the epilogue, well after the table)
   uint64_t pfull[C::kTables], pfree[C::kTables];  // table written; every producer has read it
   uint64_t full[C::kStages], done[C::kStages];   // operands written; MMAs complete
-  uint64_t xbar, drain;
+  uint64_t acc_free[C::kAccs];  // accumulators added up
+  uint64_t drain;
   uint32_t tmem;
   int abort_flag;
 };
@@ -196,6 +211,39 @@ __device__ __forceinline__ void tmem_ld4x4(uint32_t t0, uint32_t t1, uint32_t t2
         "=&r"(r[2][2]), "=&r"(r[2][3]), "=&r"(r[3][0]), "=&r"(r[3][1]), "=&r"(r[3][2]),
         "=&r"(r[3][3])
       : "r"(t0), "r"(t1), "r"(t2), "r"(t3)
+      : "memory");
+}
+
+// Sixteen columns of this warp's 32 lanes written; units of four columns read
+// from two places, or one to four from one place, and waited for.
+__device__ __forceinline__ void tmem_st16(uint32_t t, const float (&v)[4][4]) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+      ::"r"(t), "f"(v[0][0]), "f"(v[0][1]), "f"(v[0][2]), "f"(v[0][3]), "f"(v[1][0]), "f"(v[1][1]),
+      "f"(v[1][2]), "f"(v[1][3]), "f"(v[2][0]), "f"(v[2][1]), "f"(v[2][2]), "f"(v[2][3]),
+      "f"(v[3][0]), "f"(v[3][1]), "f"(v[3][2]), "f"(v[3][3])
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t t0, uint32_t t1, float (&v)[2][4]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n"
+      "tcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=&f"(v[0][0]), "=&f"(v[0][1]), "=&f"(v[0][2]), "=&f"(v[0][3]), "=&f"(v[1][0]),
+        "=&f"(v[1][1]), "=&f"(v[1][2]), "=&f"(v[1][3])
+      : "r"(t0), "r"(t1)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t t, float (&v)[2][4]) { tmem_ld4(t, t + 4, v); }
+__device__ __forceinline__ void tmem_ld4(uint32_t t, float (&v)[4][4]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=&f"(v[0][0]), "=&f"(v[0][1]), "=&f"(v[0][2]), "=&f"(v[0][3]), "=&f"(v[1][0]),
+        "=&f"(v[1][1]), "=&f"(v[1][2]), "=&f"(v[1][3]), "=&f"(v[2][0]), "=&f"(v[2][1]),
+        "=&f"(v[2][2]), "=&f"(v[2][3]), "=&f"(v[3][0]), "=&f"(v[3][1]), "=&f"(v[3][2]),
+        "=&f"(v[3][3])
+      : "r"(t)
       : "memory");
 }
 
@@ -310,11 +358,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&sm.pfree[i], C::kTasks);
     }
     for (int i = 0; i < S; ++i) {
-      // the stage's operands written, and its accumulator's last contents read
-      mbar_init(&sm.full[i], C::kTasks + kEpiWarps);
+      mbar_init(&sm.full[i], C::kTasks);
       mbar_init(&sm.done[i], 1);
     }
-    mbar_init(&sm.xbar, kEpiWarps);
+    for (int i = 0; i < C::kAccs; ++i) mbar_init(&sm.acc_free[i], kEpiWarps);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -334,7 +381,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_chan = sets ? sets[0].args.n_chan : a.n_chan;  // common to a batch
   const int n_chunks = (n_chan + kCh - 1) / kCh;
   const int per_item = n_chunks * kBins;  // stages of an item: chunk-major, bins inner
-  const int my_items = (n_items - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1;
+  // This CTA's items: every gridDim.x-th; or, where a second bin of the same
+  // trials is stored together with a first, every gridDim.x-th two neighbours
+  // (CTAs beside each other still work on bins beside each other, which share
+  // sectors) and then its part of the rest, so that no CTA has more than one
+  // item more than another.
+  const int cta = blockIdx.x, n_ctas = gridDim.x;
+  const int my_items = n_items / n_ctas + (cta < n_items % n_ctas ? 1 : 0);
+  const int rounds = C::kSlots > 1 ? n_items / (2 * n_ctas) : 0;
+  const int rest = n_items - rounds * 2 * n_ctas, each = rest / n_ctas, more = rest % n_ctas;
+  auto item_at = [&](int i) {
+    if (C::kSlots < 2) return cta + i * n_ctas;
+    if (i < 2 * rounds) return (i >> 1) * 2 * n_ctas + 2 * cta + (i & 1);
+    return rounds * 2 * n_ctas + cta * each + min(cta, more) + i - 2 * rounds;
+  };
   const uint32_t total = static_cast<uint32_t>(my_items) * per_item;  // stages of this CTA
   // K steps of 16 channels of an item's last stage (the others have all four)
   const int tail_steps = (n_chan - (n_chunks - 1) * kCh + 15) / 16;
@@ -344,20 +404,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (warp < kEpiWarps) {
     // ------------------------------------------------------------ epilogue
     // A thread holds sixteen (bin, al) units of four sums each.
-    const int row = threadIdx.x;  // row of the product: Cb (< 64) or Sb
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-    const int b = row & 63;
-    const bool is_c = row < 64;
-    for (int s = 0; s < S; ++s) mbar_arrive_warp(&sm.full[s]);  // every accumulator is free at first
-    uint32_t xphase = 0;  // phases of the exchange barrier: two per item
-    auto exchange_sync = [&]() {
-      mbar_arrive_warp(&sm.xbar);
-      const bool met = warp_wait(&sm.xbar, xphase & 1, abort_flag);
-      ++xphase;
-      return met;
-    };
+    const bool is_c = lane < 16;  // this lane's row: Cb, or Sb of the same b
+    const int b = 16 * warp + (lane & 15);
+    uint32_t acc_at = 0;  // the stage's accumulator
+    bool held = false;    // the last item's sums wait in slot 0 for this one's
     uint32_t n_item = 0;  // first stage of the item
-    for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, n_item += per_item) {
+    for (int i_item = 0; i_item < my_items && ok; ++i_item, n_item += per_item) {
       float2 acc[kBins][4][kNa / 2];
 #pragma unroll
       for (int s = 0; s < kBins; ++s)
@@ -370,6 +423,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int sl = 0; sl < kBins; ++sl) {
           const uint32_t n = n_item + c * kBins + sl;
           const uint32_t s = n % S;
+          const uint32_t d = acc_at;
+          acc_at = acc_at + 1 == C::kAccs ? 0 : acc_at + 1;
           ok = ok && warp_wait(&sm.done[s], (n / S) & 1, abort_flag);
           if (!ok) break;
           float hv[C::kSets];
@@ -384,63 +439,89 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int t = 0; t < 4; t += 2) {
               // [type t, t + 1: hi hi; the small products of both][al]
               uint32_t r[4][4];
-              const uint32_t col = t_lane + s * 2 * kN + t * kNa + 4 * h;
+              const uint32_t col = t_lane + d * 2 * kN + t * kNa + 4 * h;
               tmem_ld4x4(col, col + kNa, col + kN, col + kN + kNa, r);
               if (h == kNa / 4 - 1 && t == 2) {
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                mbar_arrive_warp(&sm.full[s]);
+                mbar_arrive_warp(&sm.acc_free[d]);
               }
 #pragma unroll
               for (int e = 0; e < 2; ++e)
 #pragma unroll
                 for (int i = 0; i < 2; ++i) {
-                  float2& d = acc[sl][t + e][2 * h + i];
+                  float2& to = acc[sl][t + e][2 * h + i];
                   const float2 v = __fadd2_rn(
                       make_float2(__uint_as_float(r[e][2 * i]), __uint_as_float(r[e][2 * i + 1])),
                       make_float2(__uint_as_float(r[2 + e][2 * i]),
                                   __uint_as_float(r[2 + e][2 * i + 1])));
-                  d = __ffma2_rn(v, inv, d);
+                  to = __ffma2_rn(v, inv, to);
                 }
             }
           }
         }
       }
       if (!ok) break;
-      // Y[s, t] = A_s + i t B_s,  A_s = sum Cb X (Ca + i s Sa), B_s the same
-      // with Sb: through shared memory, eight (al, bin) units at a time; the
-      // thread of a Cb row then makes the trials of s = +, that of the Sb row
-      // of the same b those of s = -.
+      // The sums go through tensor memory, whose columns a loop can index.  A
+      // wide pass of several series has one bin at a time: it leaves an even
+      // bin's there and stores it with the next, sixteen bytes a trial instead
+      // of eight (a store touches as many cache lines as lanes, whatever its
+      // width).
+      const int item = item_at(i_item);
       const Item q = decode<C>(a, sets, n_sets, item);
+      const uint32_t park = t_lane + C::kPark + (held ? 64 : 0);
+#pragma unroll
+      for (int u = 0; u < (C::kSlots > 0 ? 16 : 0); u += 4) {
+        float v[4][4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int al = (u + e) / kBins, sl = (u + e) % kBins;
+#pragma unroll
+          for (int t = 0; t < 4; ++t) v[e][t] = (al & 1) ? acc[sl][t][al / 2].y : acc[sl][t][al / 2].x;
+        }
+        tmem_st16(park + u * 4, v);
+      }
+      if (C::kSlots > 0) asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      if (C::kSlots > 1 && !held && (q.k0 & 1) == 0 && i_item + 1 < my_items &&
+          item_at(i_item + 1) == item + 1) {
+        const Item next = decode<C>(a, sets, n_sets, item + 1);
+        held = next.set == q.set && next.j_p == q.j_p;
+        if (held) continue;
+      }
+      // Y[s, t] = A_s + i t B_s,  A_s = sum Cb X (Ca + i s Sa), B_s the same
+      // with Sb: the lane of a Cb row makes the trials of s = +, that of the
+      // Sb row of the same b those of s = -, each with two values of the other.
+      constexpr int kOut = C::kOutBins;
+      const int k0 = held ? q.k0 - 1 : q.k0;
       const MacArgs& m = sets ? sets[q.set].args : a;
       const int64_t dm_stride = m.y_dm_stride;
-      const int n_dm = m.n_dm, n_bins = m.n_bins, out_kind = m.out_kind;
+      const int n_dm = m.n_dm, out_kind = m.out_kind;
       const float scale = m.scale;
-      const int k_abs = m.k_begin + q.k0, real_a = m.real_bin_a, real_b = m.real_bin_b;
-      const int64_t off = (sets ? 0 : static_cast<int64_t>(q.set) * m.y_series_stride) + q.k0;
+      const int k_abs = m.k_begin + k0, real_a = m.real_bin_a, real_b = m.real_bin_b;
+      const int64_t off = (sets ? 0 : static_cast<int64_t>(q.set) * m.y_series_stride) + k0;
       void* const Yv = m.Y;
-      const bool whole = q.k0 + kBins <= n_bins;
+      const int n_out = C::kSlots > 1 ? (held ? 2 : 1) : m.n_bins - k0 < kOut ? m.n_bins - k0 : kOut;
+      const bool whole = n_out == kOut;
+      held = false;
+      const float sg = is_c ? 1.f : -1.f;
+#pragma unroll (C::kSlots > 0 ? 1 : kNa)
+      for (int al = 0; al < kNa; ++al) {
+        if (C::kSeries ? al % C::kAls < q.n_a : al < q.n_a) {
+          float v[kOut][4];
+          if constexpr (C::kSlots > 1)
+            tmem_ld4(t_lane + C::kPark + al * 4, t_lane + C::kPark + 64 + al * 4, v);
+          else if constexpr (C::kSlots == 1)
+            tmem_ld4(t_lane + C::kPark + al * 4 * kBins, v);
+          else
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        constexpr int kHalfAls = 8 / kBins;  // al's of a half
+            for (int t = 0; t < 4; ++t) v[0][t] = (al & 1) ? acc[0][t][al / 2].y : acc[0][t][al / 2].x;
+          float2 y[2][kOut];  // t = +, -
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int al = half * kHalfAls + u / kBins, sl = u % kBins;
-          const float m1 = (al & 1) ? acc[sl][0][al / 2].y : acc[sl][0][al / 2].x;
-          const float m2 = (al & 1) ? acc[sl][1][al / 2].y : acc[sl][1][al / 2].x;
-          const float m3 = (al & 1) ? acc[sl][2][al / 2].y : acc[sl][2][al / 2].x;
-          const float m4 = (al & 1) ? acc[sl][3][al / 2].y : acc[sl][3][al / 2].x;
-          sm.xch[u][row] = make_float4(m1 - m4, m2 + m3, m1 + m4, m2 - m3);
-        }
-        if (!(ok = exchange_sync())) break;
-#pragma unroll 1
-        for (int i = 0; i < kHalfAls; ++i) {
-          const int al = half * kHalfAls + i;
-          if (C::kSeries ? al % C::kAls >= q.n_a : al >= q.n_a) continue;
-          float2 y[2][kBins];  // t = +, -
-#pragma unroll
-          for (int sl = 0; sl < kBins; ++sl) {
-            const float2 A = reinterpret_cast<const float2*>(&sm.xch[i * kBins + sl][b])[is_c ? 0 : 1];
-            const float2 B = reinterpret_cast<const float2*>(&sm.xch[i * kBins + sl][b + 64])[is_c ? 0 : 1];
+          for (int sl = 0; sl < kOut; ++sl) {
+            const float ox = v[sl][0] - sg * v[sl][3], oy = v[sl][1] + sg * v[sl][2];
+            const float rx = __shfl_xor_sync(0xffffffffu, v[sl][0] + sg * v[sl][3], 16);
+            const float ry = __shfl_xor_sync(0xffffffffu, v[sl][1] - sg * v[sl][2], 16);
+            const float2 A = is_c ? make_float2(ox, oy) : make_float2(rx, ry);
+            const float2 B = is_c ? make_float2(rx, ry) : make_float2(ox, oy);
             const bool real_only = k_abs + sl == real_a || k_abs + sl == real_b;
             y[0][sl] = make_float2((A.x - B.y) * scale, real_only ? 0.f : (A.y + B.x) * scale);
             y[1][sl] = make_float2((A.x + B.y) * scale, real_only ? 0.f : (A.y - B.x) * scale);
@@ -457,35 +538,34 @@ __global__ void __launch_bounds__(kThreads, 1)
             const int64_t o = off_h + static_cast<int64_t>(j) * dm_stride;
             if (out_kind == 2) {
               float* Y = static_cast<float*>(Yv) + o;
-              float pw[kBins];
+              float pw[kOut];
 #pragma unroll
-              for (int sl = 0; sl < kBins; ++sl)
+              for (int sl = 0; sl < kOut; ++sl)
                 pw[sl] = y[t][sl].x * y[t][sl].x + y[t][sl].y * y[t][sl].y;
-              if (kBins == 4 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
-                *reinterpret_cast<float4*>(Y) = make_float4(pw[0], pw[1 % kBins], pw[2 % kBins], pw[3 % kBins]);
-              } else if (kBins == 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 7) == 0) {
-                *reinterpret_cast<float2*>(Y) = make_float2(pw[0], pw[1 % kBins]);
+              if (kOut == 4 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
+                *reinterpret_cast<float4*>(Y) = make_float4(pw[0], pw[1 % kOut], pw[2 % kOut], pw[3 % kOut]);
+              } else if (kOut == 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 7) == 0) {
+                *reinterpret_cast<float2*>(Y) = make_float2(pw[0], pw[1 % kOut]);
               } else {
 #pragma unroll
-                for (int sl = 0; sl < kBins; ++sl)
-                  if (q.k0 + sl < n_bins) Y[sl] = pw[sl];
+                for (int sl = 0; sl < kOut; ++sl)
+                  if (sl < n_out) Y[sl] = pw[sl];
               }
             } else {
               float2* Y = static_cast<float2*>(Yv) + o;
-              if (kBins >= 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
+              if (kOut >= 2 && whole && (reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
 #pragma unroll
-                for (int sl = 0; sl < kBins; sl += 2)
+                for (int sl = 0; sl < kOut; sl += 2)
                   *reinterpret_cast<float4*>(Y + sl) =
-                      make_float4(y[t][sl].x, y[t][sl].y, y[t][(sl + 1) % kBins].x, y[t][(sl + 1) % kBins].y);
+                      make_float4(y[t][sl].x, y[t][sl].y, y[t][(sl + 1) % kOut].x, y[t][(sl + 1) % kOut].y);
               } else {
 #pragma unroll
-                for (int sl = 0; sl < kBins; ++sl)
-                  if (q.k0 + sl < n_bins) Y[sl] = y[t][sl];
+                for (int sl = 0; sl < kOut; ++sl)
+                  if (sl < n_out) Y[sl] = y[t][sl];
               }
             }
           }
         }
-        if (!(ok = exchange_sync())) break;  // read before the next writes
       }
     }
   } else if (warp == kMmaWarp) {
@@ -499,16 +579,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                              (static_cast<uint32_t>(kRows >> 4) << 24);  // hi and lo columns at once
     bool issued = false;
     uint32_t left = per_item;  // stages of the item still to come
-    uint32_t phase = 0;
-    int s = 0;
+    uint32_t phase = 0, acc_phase = 1;
+    int s = 0, acc = 0;
     for (uint32_t n = 0; n < total; ++n) {
-      ok = warp_wait(&sm.full[s], phase, abort_flag);
+      ok = warp_wait(&sm.full[s], phase, abort_flag) &&
+           warp_wait(&sm.acc_free[acc], acc_phase, abort_flag);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int steps = left <= kBins ? tail_steps : 4;
       if (el) {
         const uint32_t st = base + s * C::kStageBytes;
-        const uint32_t d = tm + s * 2 * kN;
+        const uint32_t d = tm + acc * 2 * kN;
         const uint64_t a_hi = core_desc(st, kRows * 16);
         const uint64_t a_lo = core_desc(st + C::kATile, kRows * 16);
         const uint64_t b = core_desc(st + 2 * C::kATile, 2 * kN * 16);
@@ -540,6 +621,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         s = 0;
         phase ^= 1;
       }
+      if (++acc == C::kAccs) {
+        acc = 0;
+        acc_phase ^= 1;
+      }
       __syncwarp();
     }
     // (the epilogue waits for every stage, so tensor memory is idle at the
@@ -567,8 +652,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool bin_ok;
     };
     const int p = warp - kPrepFirst;
-    int item = blockIdx.x;
-    int q = p;  // stage within the item
+    int i_item = 0, q = p;  // stage within the item
     // the item at hand, in registers: its spectra, constants and phases' origin
     int cur = -1, left_bins = 0, k_abs = 0;
     uint32_t before[C::kCentres] = {};
@@ -581,12 +665,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       // would be waited for right here, to merge it with the other value.
       while (q >= per_item) {
         q -= per_item;
-        item += gridDim.x;
+        ++i_item;
       }
-      if (item != cur && item < n_items) {
-        const Item it = decode<C>(a, sets, n_sets, item);
+      if (i_item != cur && i_item < my_items) {
+        const Item it = decode<C>(a, sets, n_sets, item_at(i_item));
         const MacArgs& m = sets ? sets[it.set].args : a;
-        cur = item;
+        cur = i_item;
         left_bins = m.n_bins - it.k0;
         k_abs = m.k_begin + it.k0;
 #pragma unroll
@@ -709,6 +793,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else {
     // ------------------------------------------------------------ producers
+    const bool few = n_chan <= kFewChan;
     // Waits by parity see one phase back only.  A producer steps fewer than S
     // stages from task to task and waits for each task's stage to be free, so
     // when it waits for stage n to be free, n - 2 S is (MMAs end in order).
@@ -763,11 +848,12 @@ __global__ void __launch_bounds__(kThreads, 1)
               ok = warp_wait(&sm.done[s], ((n / S) & 1) ^ 1, abort_flag);
               if (!ok) break;
             }
-            unsigned char* at = &sm.stage[s][oct * kRows * 16 + b * 16 + half * 8];
+            unsigned char* at = &sm.stage[s][oct * kRows * 16 + b * 16 + half * 8];  // (row b)
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
-              *reinterpret_cast<uint2*>(at + t * 16 * 16) = make_uint2(hi[t][0], hi[t][1]);
-              *reinterpret_cast<uint2*>(at + C::kATile + t * 16 * 16) = make_uint2(lo[t][0], lo[t][1]);
+              const int row = 32 * (t & 3) + 16 * (t >> 2);
+              *reinterpret_cast<uint2*>(at + row * 16) = make_uint2(hi[t][0], hi[t][1]);
+              *reinterpret_cast<uint2*>(at + C::kATile + row * 16) = make_uint2(lo[t][0], lo[t][1]);
             }
           }
           if (!ok) break;
@@ -797,9 +883,15 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int p = 0; p < 2; ++p) {
               const float2 xr = p ? make_float2(xrv.z, xrv.w) : make_float2(xrv.x, xrv.y);
               const float2 xi = p ? make_float2(xiv.z, xiv.w) : make_float2(xiv.x, xiv.y);
-              const float2 w0 = unit_phasor(mul * (p ? hv.z : hv.x));
-              const float2 w1 = unit_phasor(mul * (p ? hv.w : hv.y));
-              const float2 cs = make_float2(w0.x, w1.x), sn = make_float2(w0.y, w1.y);
+              const uint32_t p0 = mul * (p ? hv.z : hv.x), p1 = mul * (p ? hv.w : hv.y);
+              float2 cs, sn;
+              if (few) {
+                sincos2(p0, p1, cs, sn);
+              } else {
+                const float2 w0 = unit_phasor(p0), w1 = unit_phasor(p1);
+                cs = make_float2(w0.x, w1.x);
+                sn = make_float2(w0.y, w1.y);
+              }
               split2(__fmul2_rn(xr, cs), hi[e][0][p], lo[e][0][p]);
               split2(__fmul2_rn(xi, cs), hi[e][1][p], lo[e][1][p]);
               split2(__fmul2_rn(xr, sn), hi[e][2][p], lo[e][2][p]);

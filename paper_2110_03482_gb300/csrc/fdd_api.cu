@@ -42,6 +42,10 @@ struct fdd_plan_s {
   float2* d_Y = nullptr;      // [dm_batch][bin_pitch] dedispersed spectra (time output;
                               // tensor-core form: [beam][dm_batch][bin_pitch])
   float* d_yt = nullptr;      // [dm_batch][L] inverse transforms (time output)
+  // a second beam's or chunk's spectra and dedispersed spectra, where two share
+  // the launches of the phase-rotate-and-sum (pairing_bytes); nullptr otherwise
+  float2* d_X2 = nullptr;
+  float2* d_Y2 = nullptr;
   // spin-frequency-dependent grids (fdd_params.spin_group): the scaled grid's
   // phase table, the scratch of the groups, and the FP32 tile of the bins
   // below the first group
@@ -343,7 +347,25 @@ size_t spin_plan_bytes(const fdd_params* p, const fdd::CoreGeometry& cg, int64_t
   return sizeof(fdd::PhaseConst) * p->n_chan + fdd::spin_scratch_bytes(sg, p->n_chan, n_bins);
 }
 
-fdd_status compute_plan(const fdd_params* p, fdd_info* g, fdd::CoreGeometry* core_out) {
+// Bytes a plan holds to take two (beam, chunk)s through each launch of the
+// phase-rotate-and-sum: the G12 tile's series share its cosine and sine rows
+// (1024 channels x 2048 trials: 73 ns a bin one by one, 52 in twos).  Only what
+// fits the limit beside the rest, with every trial in one batch, as the
+// batches' order is the same then; 0 where there is nothing to share or no room.
+size_t pairing_bytes(const fdd_params* p, const fdd_info* g) {
+  if (p->precision != FDD_PREC_FP32 || g->mac_variant != FDD_MAC_G12_4X8 ||
+      !fdd::mac_split_series_share(p->n_dm) || p->n_beams * g->n_chunks < 2)
+    return 0;
+  const bool time = p->output == FDD_OUT_TIME;
+  if (time && g->dm_batch < p->n_dm) return 0;
+  const size_t bytes = sizeof(float2) * static_cast<size_t>(g->bin_pitch) *
+                       (static_cast<size_t>(p->n_chan) + (time ? p->n_dm : 0));
+  const size_t limit = p->workspace_limit ? p->workspace_limit : kDefaultWorkspace;
+  return static_cast<size_t>(g->workspace_bytes) + bytes <= limit ? bytes : 0;
+}
+
+fdd_status compute_plan(const fdd_params* p, fdd_info* g, fdd::CoreGeometry* core_out,
+                        size_t* pair_out = nullptr) {
   if (!p) return fail(FDD_ERR_INVALID_ARG, "params is NULL");
   if (!g) return fail(FDD_ERR_INVALID_ARG, "info is NULL");
   if (p->n_beams < 1) return fail(FDD_ERR_INVALID_ARG, "n_beams must be >= 1");
@@ -465,6 +487,9 @@ fdd_status compute_plan(const fdd_params* p, fdd_info* g, fdd::CoreGeometry* cor
   if (tc) g->mac_variant = pair ? FDD_MAC_TC_PAIR : FDD_MAC_TC;
   g->dm_batch = static_cast<int32_t>(batch);
   g->workspace_bytes = static_cast<int64_t>(fixed + per_dm * batch);
+  const size_t pair_bytes = pairing_bytes(p, g);
+  g->workspace_bytes += static_cast<int64_t>(pair_bytes);
+  if (pair_out) *pair_out = pair_bytes;
   // Streamed calls: output blocks of one beam's DM batch (time), or of
   // block_dm trials of every spectra set (spectra, power; whole passes of the
   // kernel tile, up to 4 GiB or a quarter of workspace_limit, at least one
@@ -496,7 +521,7 @@ void release(fdd_plan_s* P) {
   if (P->has_r2c) cufftDestroy(P->r2c);
   if (P->has_c2r) cufftDestroy(P->c2r);
   if (P->has_c2r_tail) cufftDestroy(P->c2r_tail);
-  void* ptrs[] = {P->d_pc, P->d_xw, P->d_X, P->d_Y, P->d_yt, P->d_xb, P->d_Yb, P->d_fftwork,
+  void* ptrs[] = {P->d_pc, P->d_xw, P->d_X, P->d_Y, P->d_yt, P->d_X2, P->d_Y2, P->d_xb, P->d_Yb, P->d_fftwork,
                   P->d_pc_spin, P->d_spin_scratch, P->d_status,
                   P->d_win[0], P->d_win[1], P->d_blk[0], P->d_blk[1], P->d_tcx, P->d_shift,
                   P->d_shift_base, P->d_tdd_x};
@@ -782,72 +807,83 @@ fdd_status run(fdd_plan_s* P, const Io& io, cudaStream_t s) {
   if (P->tc) return run_tc(P, io, s);
   fdd_status st;
   const int dm_end = io.dm_first + io.n_dm;
-  for (int b = 0; b < p.n_beams; ++b) {
-    for (int64_t c = 0; c < g.n_chunks; ++c) {
-      if ((st = transform(P, io, b, c, P->d_X, s)) != FDD_OK) return st;
-      fdd::MacArgs m{};
-      m.X = P->d_X;
-      m.x_series_stride = 0;
-      m.x_chan_stride = g.bin_pitch;
-      m.pc = P->d_pc;
-      m.n_chan = p.n_chan;
-      m.n_bins = static_cast<int>(g.n_bins);
-      m.n_series = 1;
-      m.scale = 1.0f;
-      m.status = P->d_status;
-      if (p.output == FDD_OUT_TIME) {
-        // (shortened inverse: only the bins up to Nyquist of length L / f)
-        const int64_t Ls = g.fft_len / g.downsample;
-        m.n_bins = static_cast<int>(Ls / 2 + 1);
-        for (int j0 = io.dm_first; j0 < dm_end; j0 += g.dm_batch) {
-          const int nb = (dm_end - j0) < g.dm_batch ? (dm_end - j0) : g.dm_batch;
-          m.j_begin = j0;
-          m.n_dm = nb;
-          m.Y = P->d_Y;
-          m.y_series_stride = 0;
-          m.y_dm_stride = g.bin_pitch;
-          m.out_kind = 1;
-          m.real_bin_a = 0;                           // DC and Nyquist of a real
-          m.real_bin_b = static_cast<int>(Ls / 2);    // series: real parts only
-          m.scale = whole_rows(P) ? static_cast<float>(1.0 / static_cast<double>(g.fft_len)) : 1.0f;
-          {
-            StageTimer t(P, FDD_STAGE_MAC, s);
-            FDD_CUDA(fdd::launch_mac_fp32(m, g.mac_variant, s));
-          }
-          if ((st = inverse_and_place(P, io, b, c, j0, nb, P->d_Y, s)) != FDD_OK) return st;
+  // (beam, chunk)s in turn, or two at a time (device buffers: streamed windows
+  // and blocks keep their order)
+  const bool in_twos = P->d_X2 != nullptr && io.d_in && io.d_out;
+  const int64_t n_units = p.n_beams * g.n_chunks;
+  for (int64_t u = 0; u < n_units;) {
+    const int n_u = in_twos && u + 1 < n_units ? 2 : 1;
+    auto beam = [&](int i) { return static_cast<int>((u + i) / g.n_chunks); };
+    auto chunk = [&](int i) { return (u + i) % g.n_chunks; };
+    float2* const X[2] = {P->d_X, P->d_X2};
+    float2* const Y[2] = {P->d_Y, P->d_Y2};
+    for (int i = 0; i < n_u; ++i)
+      if ((st = transform(P, io, beam(i), chunk(i), X[i], s)) != FDD_OK) return st;
+    fdd::MacArgs m{};
+    m.X = X[0];
+    m.x_series_stride = n_u == 2 ? X[1] - X[0] : 0;
+    m.x_chan_stride = g.bin_pitch;
+    m.pc = P->d_pc;
+    m.n_chan = p.n_chan;
+    m.n_bins = static_cast<int>(g.n_bins);
+    m.n_series = n_u;
+    m.scale = 1.0f;
+    m.status = P->d_status;
+    if (p.output == FDD_OUT_TIME) {
+      // (shortened inverse: only the bins up to Nyquist of length L / f)
+      const int64_t Ls = g.fft_len / g.downsample;
+      m.n_bins = static_cast<int>(Ls / 2 + 1);
+      for (int j0 = io.dm_first; j0 < dm_end; j0 += g.dm_batch) {
+        const int nb = (dm_end - j0) < g.dm_batch ? (dm_end - j0) : g.dm_batch;
+        m.j_begin = j0;
+        m.n_dm = nb;
+        m.Y = Y[0];
+        m.y_series_stride = n_u == 2 ? Y[1] - Y[0] : 0;
+        m.y_dm_stride = g.bin_pitch;
+        m.out_kind = 1;
+        m.real_bin_a = 0;                           // DC and Nyquist of a real
+        m.real_bin_b = static_cast<int>(Ls / 2);    // series: real parts only
+        m.scale = whole_rows(P) ? static_cast<float>(1.0 / static_cast<double>(g.fft_len)) : 1.0f;
+        {
+          StageTimer t(P, FDD_STAGE_MAC, s);
+          FDD_CUDA(fdd::launch_mac_fp32(m, g.mac_variant, s));
         }
-      } else {
-        m.y_series_stride = 0;
-        m.y_dm_stride = g.n_bins;
-        m.real_bin_a = -1;
-        m.real_bin_b = -1;
-        m.out_kind = p.output == FDD_OUT_SPECTRA ? 1 : 2;
-        const size_t esz = p.output == FDD_OUT_SPECTRA ? 8 : 4;
-        // the whole trial range into the output, or blocks of block_dm trials
-        const int step = io.d_out ? io.n_dm : P->block_dm;
-        for (int j0 = io.dm_first; j0 < dm_end; j0 += step) {
-          const int nb = (dm_end - j0) < step ? (dm_end - j0) : step;
-          m.j_begin = j0;
-          m.n_dm = nb;
-          int k = -1;
-          if (io.d_out) {
-            const int64_t row0 = (static_cast<int64_t>(b) * g.n_chunks + c) * io.n_dm;
-            m.Y = static_cast<char*>(io.d_out) + esz * row0 * g.n_bins;
-          } else {
-            if ((st = block_slot(P, io, s, &k)) != FDD_OK) return st;
-            m.Y = P->d_blk[k];
-          }
-          {
-            StageTimer t(P, FDD_STAGE_MAC, s);
-            FDD_CUDA(fdd::launch_mac_fp32(m, g.mac_variant, s));
-          }
-          if (k >= 0) {
-            fdd_block blk{b, 1, c, j0, nb, P->d_blk[k], g.n_bins, g.n_bins, 0, nullptr};
-            if ((st = deliver(P, io, k, blk, s)) != FDD_OK) return st;
-          }
+        for (int i = 0; i < n_u; ++i)
+          if ((st = inverse_and_place(P, io, beam(i), chunk(i), j0, nb, Y[i], s)) != FDD_OK)
+            return st;
+      }
+    } else {
+      // (the next (beam, chunk)'s rows follow this one's)
+      m.y_series_stride = static_cast<int64_t>(io.n_dm) * g.n_bins;
+      m.y_dm_stride = g.n_bins;
+      m.real_bin_a = -1;
+      m.real_bin_b = -1;
+      m.out_kind = p.output == FDD_OUT_SPECTRA ? 1 : 2;
+      const size_t esz = p.output == FDD_OUT_SPECTRA ? 8 : 4;
+      // the whole trial range into the output, or blocks of block_dm trials
+      const int step = io.d_out ? io.n_dm : P->block_dm;
+      for (int j0 = io.dm_first; j0 < dm_end; j0 += step) {
+        const int nb = (dm_end - j0) < step ? (dm_end - j0) : step;
+        m.j_begin = j0;
+        m.n_dm = nb;
+        int k = -1;
+        if (io.d_out) {
+          m.Y = static_cast<char*>(io.d_out) + esz * (u * io.n_dm) * g.n_bins;
+        } else {
+          if ((st = block_slot(P, io, s, &k)) != FDD_OK) return st;
+          m.Y = P->d_blk[k];
+        }
+        {
+          StageTimer t(P, FDD_STAGE_MAC, s);
+          FDD_CUDA(fdd::launch_mac_fp32(m, g.mac_variant, s));
+        }
+        if (k >= 0) {
+          fdd_block blk{beam(0), 1, chunk(0), j0, nb, P->d_blk[k], g.n_bins, g.n_bins, 0, nullptr};
+          if ((st = deliver(P, io, k, blk, s)) != FDD_OK) return st;
         }
       }
     }
+    u += n_u;
   }
   return FDD_OK;
 }
@@ -1142,7 +1178,8 @@ fdd_status plan_create(const fdd_params* p, void* arena, size_t arena_bytes, fdd
   P->arena = static_cast<char*>(arena);
   P->arena_bytes = arena ? arena_bytes : 0;
 
-  fdd_status st = compute_plan(p, &P->info, &P->core);
+  size_t pair_bytes = 0;
+  fdd_status st = compute_plan(p, &P->info, &P->core, &pair_bytes);
   if (st != FDD_OK) return st;
   P->rate.resize(p->n_chan);
   for (int c = 0; c < p->n_chan; ++c) P->rate[c] = fdd::delay_rate(*p, P->core, c);
@@ -1260,6 +1297,20 @@ fdd_status plan_create(const fdd_params* p, void* arena, size_t arena_bytes, fdd
     FDD_CUFFT(cufftSetWorkArea(P->r2c, P->d_fftwork));
     if (P->has_c2r) FDD_CUFFT(cufftSetWorkArea(P->c2r, P->d_fftwork));
     if (P->has_c2r_tail) FDD_CUFFT(cufftSetWorkArea(P->c2r_tail, P->d_fftwork));
+  }
+  if (pair_bytes > 0 && !P->arena) {
+    // (the plan runs one by one where the device has no room for two)
+    const size_t x = sizeof(float2) * size_t(nc) * g.bin_pitch;
+    void* two[2] = {};
+    if (cudaMalloc(&two[0], x) != cudaSuccess ||
+        (pair_bytes > x && cudaMalloc(&two[1], pair_bytes - x) != cudaSuccess)) {
+      cudaGetLastError();
+      if (two[0]) cudaFree(two[0]);
+    } else {
+      P->d_X2 = static_cast<float2*>(two[0]);
+      P->d_Y2 = static_cast<float2*>(two[1]);
+      P->bytes_held += pair_bytes;
+    }
   }
   g.workspace_bytes = static_cast<int64_t>(P->bytes_held);
   P->block_dm = g.block_dm;

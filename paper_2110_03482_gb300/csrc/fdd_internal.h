@@ -95,6 +95,8 @@ size_t mac_smem_bytes(int variant, int n_chan);
 size_t mac_split_smem_bytes();
 cudaError_t mac_split_prepare();
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s);
+// whether the series of one launch share passes at this trial count
+bool mac_split_series_share(int n_dm);
 void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes);
 cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
                                    int max_n_dm, int n_ctas, cudaStream_t s);

@@ -1018,6 +1018,8 @@ cudaError_t mac_split_prepare() {
   return e;
 }
 
+bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2)).sets > 1; }
+
 void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes) {
   const FormInfo f = form_info(form_for(max_n_dm, 1));
   *bin_groups = static_cast<int>((n_bins + f.bins - 1) / f.bins);

@@ -137,3 +137,35 @@ def test_series_sharing_passes_equal_each_alone(n_series, n_dm):
             assert torch.equal(dY[s], one), s
         torch.cuda.synchronize()
         plan.query()
+
+
+@pytest.mark.parametrize("output", [fdd.FDD_OUT_TIME, fdd.FDD_OUT_SPECTRA, fdd.FDD_OUT_POWER])
+@pytest.mark.parametrize("n_beams,n_t,chunk_len,n_dm", [
+    (1, 20000, 1 << 12, 300),    # chunks of one beam, an odd number
+    (3, 20000, 1 << 13, 1100),   # beams and chunks, two of different beams together
+    (2, 4096, 0, 2048),          # whole rows, no chunks
+    (1, 9000, 1 << 12, 257),
+])
+def test_plans_that_take_two_at_a_time_give_the_same_bits(n_beams, n_t, chunk_len, n_dm, output):
+    """A plan with room for two (beam, chunk)s a launch against one whose
+    limit leaves room for one."""
+    kw = dict(n_chan=40, nu_lo_mhz=1200.0, dnu_mhz=7.5, t_samp_s=1e-3, n_t=n_t,
+              chunk_len=chunk_len, n_beams=n_beams, in_dtype=fdd.FDD_IN_F32,
+              dm_list=1.0 + 0.05 * np.arange(n_dm), output=output)
+    g = torch.Generator(device="cuda").manual_seed(n_t + n_dm)
+    x = torch.randn(n_beams * n_t * 40, generator=g, device="cuda")
+    outs, held = [], []
+    limit = 0
+    for _ in range(2):
+        with fdd.Plan(workspace_limit=limit, **kw) as plan:
+            assert plan.info["mac_variant"] == fdd.FDD_MAC_G12_4X8
+            out = torch.full((plan.info["out_elems"] * (2 if output == fdd.FDD_OUT_SPECTRA else 1),),
+                             7.0, device="cuda")
+            plan.execute(x, out)
+            torch.cuda.synchronize()
+            plan.query()
+            outs.append(out)
+            held.append(plan.info["workspace_bytes"])
+            limit = fdd.fdd_plan_geometry(fdd.Params(**kw))["workspace_bytes"] - 1
+    assert held[1] < held[0]
+    assert torch.equal(outs[0], outs[1])

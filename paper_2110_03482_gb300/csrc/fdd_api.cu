@@ -87,8 +87,9 @@ struct fdd_plan_s {
   // smallest, and those smallest) and one beam's channel-major series
   int* d_shift = nullptr;
   int* d_shift_base = nullptr;
-  float* d_tdd_x = nullptr;
+  void* d_tdd_x = nullptr;  // floats, or bytes at tdd_pitch where they are added as integers
   int tdd_win = 0;
+  int64_t tdd_pitch = 0;
   size_t bytes_held = 0;
   // profiling: event pairs around stage launches (fdd_profile_enable)
   bool prof_on = false;
@@ -1553,55 +1554,95 @@ fdd_status fdd_tdd_execute(fdd_plan_t plan, const void* d_in, void* d_out, fdd_s
         sh[static_cast<size_t>(j) * nc + c] = static_cast<int>(std::floor(d + 0.5));
       }
     const int n_blk = (nd + fdd::kTdDms - 1) / fdd::kTdDms;
-    std::vector<int> base(static_cast<size_t>(n_blk) * nc);
-    std::vector<int> rel(static_cast<size_t>(n_blk) * nc * fdd::kTdDms, 0);
-    int span = 0;
+    // smallest and largest shift of a block and channel
+    auto range = [&](int b, int c, int* lo, int* hi) {
+      *lo = INT_MAX, *hi = INT_MIN;
+      for (int j = b * fdd::kTdDms; j < nd && j < (b + 1) * fdd::kTdDms; ++j) {
+        *lo = std::min(*lo, sh[static_cast<size_t>(j) * nc + c]);
+        *hi = std::max(*hi, sh[static_cast<size_t>(j) * nc + c]);
+      }
+    };
+    int span = 0, span8 = 0, lo, hi;  // span8: from the smallest's multiple of 16
     for (int b = 0; b < n_blk; ++b)
       for (int c = 0; c < nc; ++c) {
-        int lo = INT_MAX, hi = INT_MIN;
-        for (int j = b * fdd::kTdDms; j < nd && j < (b + 1) * fdd::kTdDms; ++j) {
-          lo = std::min(lo, sh[static_cast<size_t>(j) * nc + c]);
-          hi = std::max(hi, sh[static_cast<size_t>(j) * nc + c]);
-        }
-        base[static_cast<size_t>(b) * nc + c] = lo;
+        range(b, c, &lo, &hi);
         span = std::max(span, hi - lo);
-        for (int j = b * fdd::kTdDms; j < nd && j < (b + 1) * fdd::kTdDms; ++j)
-          rel[(static_cast<size_t>(b) * nc + c) * fdd::kTdDms + (j - b * fdd::kTdDms)] =
-              sh[static_cast<size_t>(j) * nc + c] - lo;
+        span8 = std::max(span8, hi - lo / 16 * 16);
       }
-    const int win = (fdd::kTdSamp + span + 3) / 4 * 4;
+    int win = (fdd::kTdSamp + span + 3) / 4 * 4;
     if (fdd::tdd_smem_bytes(win) > kMaxSmem)
       return fail(FDD_ERR_UNSUPPORTED,
                   "a block of %d trials spans %d samples of delay in one channel", fdd::kTdDms,
                   span);
+    // Bytes are added as integers where the sums are exact either way: 1024
+    // channels x 512 trials x 2^17 samples 4.4 ms, as floats 10.8.  (Their
+    // windows, six bytes a sample and channel of a stage to the floats' eight,
+    // fit wherever those do.)
+    const int win8 = (fdd::kTd8Samp + span8 + 4 + 15) / 16 * 16;
+    const bool bytes = p.in_dtype == FDD_IN_U8 && nc <= fdd::kTd8MaxChan;
+    if (bytes) win = win8;
+    const int rows = bytes ? (nc + fdd::kTdCh - 1) / fdd::kTdCh * fdd::kTdCh : nc;
+    std::vector<int> base(static_cast<size_t>(n_blk) * rows, 0);
+    std::vector<int> rel(static_cast<size_t>(n_blk) * rows * fdd::kTdDms, 0);
+    for (int b = 0; b < n_blk; ++b)
+      for (int c = 0; c < rows; ++c) {
+        if (c < nc) {
+          range(b, c, &lo, &hi);
+          if (bytes) lo = lo / 16 * 16;
+          base[static_cast<size_t>(b) * rows + c] = lo;
+        }
+        for (int q = 0; q < fdd::kTdDms; ++q) {
+          const int j = b * fdd::kTdDms + q;
+          const int r = c < nc && j < nd ? sh[static_cast<size_t>(j) * nc + c] - lo : 0;
+          rel[(static_cast<size_t>(b) * rows + c) * fdd::kTdDms + q] =
+              bytes ? (c % fdd::kTdCh * 4 + r % 4) * win + r / 4 * 4 : r;
+        }
+      }
+    const int64_t pitch = (p.n_t + 31) / 32 * 32;
     if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift), sizeof(int) * rel.size())))
       return st;
     if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift_base),
                         sizeof(int) * base.size())))
       return st;
     if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_tdd_x),
-                        sizeof(float) * static_cast<size_t>(nc) * p.n_t)))
+                        bytes ? static_cast<size_t>(nc) * pitch
+                              : sizeof(float) * static_cast<size_t>(nc) * p.n_t)))
       return st;
     FDD_CUDA(cudaMemcpy(plan->d_shift, rel.data(), sizeof(int) * rel.size(),
                         cudaMemcpyHostToDevice));
     FDD_CUDA(cudaMemcpy(plan->d_shift_base, base.data(), sizeof(int) * base.size(),
                         cudaMemcpyHostToDevice));
-    FDD_CUDA(fdd::tdd_prepare(win));
+    FDD_CUDA(bytes ? fdd::tdd8_prepare(win) : fdd::tdd_prepare(win));
     plan->tdd_win = win;
+    plan->tdd_pitch = bytes ? pitch : 0;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const size_t esz = p.in_dtype == FDD_IN_U8 ? 1 : 4;
   const int64_t beam_elems = p.n_t * static_cast<int64_t>(nc);
   for (int b = 0; b < p.n_beams; ++b) {
+    float* y = static_cast<float*>(d_out) + static_cast<int64_t>(b) * nd * out_len;
     fdd::UnpackArgs ua{static_cast<const char*>(d_in) + esz * beam_elems * b, p.in_dtype,
-                       p.in_layout, nc, p.n_t, 0, p.n_t, plan->d_tdd_x, p.n_t};
+                       p.in_layout, nc, p.n_t, 0, p.n_t, nullptr, p.n_t};
+    if (plan->tdd_pitch > 0) {
+      unsigned char* x = static_cast<unsigned char*>(plan->d_tdd_x);
+      ua.out_stride = plan->tdd_pitch;
+      {
+        StageTimer t(plan, FDD_STAGE_UNPACK, s);
+        FDD_CUDA(fdd::launch_unpack_bytes(ua, x, s));
+      }
+      fdd::Tdd8Args ta{x, plan->tdd_pitch, p.n_t, nc, plan->d_shift, plan->d_shift_base, nd,
+                       plan->tdd_win, y, out_len};
+      StageTimer t(plan, FDD_STAGE_TDD, s);
+      FDD_CUDA(fdd::launch_tdd8(ta, s));
+      continue;
+    }
+    ua.out = static_cast<float*>(plan->d_tdd_x);
     {
       StageTimer t(plan, FDD_STAGE_UNPACK, s);
       FDD_CUDA(fdd::launch_unpack(ua, s));
     }
-    fdd::TddArgs ta{plan->d_tdd_x, p.n_t, nc, plan->d_shift, plan->d_shift_base, nd,
-                    plan->tdd_win,
-                    static_cast<float*>(d_out) + static_cast<int64_t>(b) * nd * out_len, out_len};
+    fdd::TddArgs ta{ua.out, p.n_t, nc, plan->d_shift, plan->d_shift_base, nd, plan->tdd_win, y,
+                    out_len};
     StageTimer t(plan, FDD_STAGE_TDD, s);
     FDD_CUDA(fdd::launch_tdd(ta, s));
   }

@@ -267,6 +267,8 @@ struct UnpackArgs {
   int64_t out_stride;
 };
 cudaError_t launch_unpack(const UnpackArgs& a, cudaStream_t s);
+// The same for 8-bit input kept in 8 bits: a.out is [n_chan][out_stride] bytes.
+cudaError_t launch_unpack_bytes(const UnpackArgs& a, unsigned char* out, cudaStream_t s);
 
 // Scale by 1/L and place the first n_keep samples of each DM series of one
 // chunk into the time-domain output (the discard rule of Sect. 2.2).
@@ -302,5 +304,28 @@ struct TddArgs {
 size_t tdd_smem_bytes(int win);
 cudaError_t tdd_prepare(int win);
 cudaError_t launch_tdd(const TddArgs& a, cudaStream_t s);
+
+// The same for 8-bit samples, added as integers.
+constexpr int kTd8Samp = 512;     // output samples per CTA
+constexpr int kTd8MaxChan = 65793;  // 255 x this is below 2^24: sums are exact in FP32
+struct Tdd8Args {
+  const unsigned char* x;  // one beam, channel-major [n_chan][pitch], 16-byte aligned
+  int64_t pitch;           // a multiple of 16
+  int64_t n_t;
+  int n_chan;
+  // tables of [blocks of kTdDms trials][n_chan up to a multiple of kTdCh]:
+  const int* off;     // [..][kTdDms] place of the trial's first sample in its stage's
+                      // windows, ((c mod kTdCh) 4 + r mod 4) win + r / 4 * 4 for the
+                      // rounded delay r minus base
+  const int* base;    // [..] smallest shift of the block, down to a multiple of 16
+  int n_dm;
+  int win;            // window bytes per channel: kTd8Samp + the largest r + 4, up to a
+                      // multiple of 16
+  float* y;           // [n_dm][out_len]
+  int64_t out_len;
+};
+size_t tdd8_smem_bytes(int win);
+cudaError_t tdd8_prepare(int win);
+cudaError_t launch_tdd8(const Tdd8Args& a, cudaStream_t s);
 
 }  // namespace fdd

@@ -42,11 +42,11 @@ struct Vec4<float> {
   }
 };
 
-template <typename Tin, bool kVec>
+template <typename Tin, bool kVec, typename Tout>
 __global__ void __launch_bounds__(256) unpack_time_major_kernel(const Tin* __restrict__ in,
                                                                 int n_chan, int64_t n_t,
                                                                 int64_t t_begin, int64_t L,
-                                                                float* __restrict__ out,
+                                                                Tout* __restrict__ out,
                                                                 int64_t out_stride) {
   __shared__ float tile[kUnpC][kTile + 1];
   const int64_t n0 = static_cast<int64_t>(blockIdx.x) * kTile;
@@ -76,22 +76,23 @@ __global__ void __launch_bounds__(256) unpack_time_major_kernel(const Tin* __res
     const int c = c0 + cl;
     const int64_t n = n0 + threadIdx.x;
     if (c < n_chan && n < L)
-      out[static_cast<int64_t>(c) * out_stride + n] = tile[cl][(threadIdx.x + (cl >> 2)) & (kTile - 1)];
+      out[static_cast<int64_t>(c) * out_stride + n] =
+          static_cast<Tout>(tile[cl][(threadIdx.x + (cl >> 2)) & (kTile - 1)]);
   }
 }
 
-template <typename Tin>
+template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(256) unpack_chan_major_kernel(const Tin* __restrict__ in,
                                                                 int n_chan, int64_t n_t,
                                                                 int64_t t_begin, int64_t L,
-                                                                float* __restrict__ out,
+                                                                Tout* __restrict__ out,
                                                                 int64_t out_stride) {
   const int c = blockIdx.y;
   for (int64_t n = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; n < L;
        n += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t t = t_begin + n;
     out[static_cast<int64_t>(c) * out_stride + n] =
-        (t < n_t) ? static_cast<float>(in[static_cast<int64_t>(c) * n_t + t]) : 0.f;
+        (t < n_t) ? static_cast<Tout>(in[static_cast<int64_t>(c) * n_t + t]) : Tout(0);
   }
 }
 
@@ -275,48 +276,39 @@ cudaError_t launch_bin_absmax(const BinAbsmaxArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpack(const UnpackArgs& a, cudaStream_t s) {
+namespace {
+template <typename Tin, typename Tout>
+cudaError_t unpack_as(const UnpackArgs& a, Tout* out, cudaStream_t s) {
   note_launches(1);
+  const Tin* in = static_cast<const Tin*>(a.in);
   if (a.in_layout == FDD_LAYOUT_TIME_MAJOR) {
     dim3 grid(static_cast<unsigned>((a.L + kTile - 1) / kTile), (a.n_chan + kUnpC - 1) / kUnpC);
     dim3 block(kTile, 8);
     if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
     // vector loads when every row of four channels is aligned for them
-    const size_t esz = a.in_dtype == FDD_IN_U8 ? 1 : 4;
-    const bool vec = a.n_chan % 4 == 0 && reinterpret_cast<uintptr_t>(a.in) % (4 * esz) == 0;
-    if (a.in_dtype == FDD_IN_U8) {
-      const uint8_t* in = static_cast<const uint8_t*>(a.in);
-      if (vec)
-        unpack_time_major_kernel<uint8_t, true><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t,
-                                                                       a.t_begin, a.L, a.out,
-                                                                       a.out_stride);
-      else
-        unpack_time_major_kernel<uint8_t, false><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t,
-                                                                        a.t_begin, a.L, a.out,
-                                                                        a.out_stride);
-    } else {
-      const float* in = static_cast<const float*>(a.in);
-      if (vec)
-        unpack_time_major_kernel<float, true><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t,
-                                                                     a.t_begin, a.L, a.out,
-                                                                     a.out_stride);
-      else
-        unpack_time_major_kernel<float, false><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t,
-                                                                      a.t_begin, a.L, a.out,
-                                                                      a.out_stride);
-    }
+    if (a.n_chan % 4 == 0 && reinterpret_cast<uintptr_t>(a.in) % (4 * sizeof(Tin)) == 0)
+      unpack_time_major_kernel<Tin, true><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t, a.t_begin,
+                                                                 a.L, out, a.out_stride);
+    else
+      unpack_time_major_kernel<Tin, false><<<grid, block, 0, s>>>(in, a.n_chan, a.n_t, a.t_begin,
+                                                                  a.L, out, a.out_stride);
   } else {
     const int64_t blocks = (a.L + 255) / 256;
     dim3 grid(static_cast<unsigned>(blocks < 4096 ? blocks : 4096), a.n_chan);
     if (grid.y > 65535u) return cudaErrorInvalidConfiguration;
-    if (a.in_dtype == FDD_IN_U8)
-      unpack_chan_major_kernel<uint8_t><<<grid, 256, 0, s>>>(
-          static_cast<const uint8_t*>(a.in), a.n_chan, a.n_t, a.t_begin, a.L, a.out, a.out_stride);
-    else
-      unpack_chan_major_kernel<float><<<grid, 256, 0, s>>>(
-          static_cast<const float*>(a.in), a.n_chan, a.n_t, a.t_begin, a.L, a.out, a.out_stride);
+    unpack_chan_major_kernel<Tin>
+        <<<grid, 256, 0, s>>>(in, a.n_chan, a.n_t, a.t_begin, a.L, out, a.out_stride);
   }
   return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_unpack(const UnpackArgs& a, cudaStream_t s) {
+  return a.in_dtype == FDD_IN_U8 ? unpack_as<uint8_t>(a, a.out, s) : unpack_as<float>(a, a.out, s);
+}
+
+cudaError_t launch_unpack_bytes(const UnpackArgs& a, unsigned char* out, cudaStream_t s) {
+  return unpack_as<uint8_t>(a, out, s);
 }
 
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {

@@ -828,6 +828,7 @@ fdd_status run(fdd_plan_s* P, const Io& io, cudaStream_t s) {
     m.n_chan = p.n_chan;
     m.n_bins = static_cast<int>(g.n_bins);
     m.n_series = n_u;
+    m.of_n_dm = p.n_dm;
     m.scale = 1.0f;
     m.status = P->d_status;
     if (p.output == FDD_OUT_TIME) {
@@ -1482,6 +1483,7 @@ fdd_status fdd_dedisperse_spectra_bins(fdd_plan_t plan, const void* d_X, int64_t
   if (st != FDD_OK) return st;
   if ((st = need_uniform_grid(plan)) != FDD_OK) return st;
   fdd::MacArgs m{};
+  m.of_n_dm = plan->p.n_dm;
   m.tc_pair = plan->info.mac_variant == FDD_MAC_TC_PAIR;
   m.X = static_cast<const float2*>(d_X);
   m.x_chan_stride = x_pitch;

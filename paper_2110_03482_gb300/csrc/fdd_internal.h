@@ -49,6 +49,7 @@ struct MacArgs {
                             // |re| or |im| of the spectra (sets that bin's data scale)
   int absmax_ready;         // tensor cores in FP16: the scratch already holds the
                             // per-bin maxima of these spectra (a later DM batch)
+  int of_n_dm;              // trials of the plan this call is part of (the G12 tile's form)
   int tc_pair;              // tensor cores: the CTA-pair form (the plan's choice)
 };
 

@@ -47,7 +47,9 @@
 // share them too (two, or four up to 1024 trials), each with its own columns
 // and scales and the bits it has alone: 4096 (bin, series) x 1024 channels of
 // 2048 trials take 300 us each alone and 227 in twos; of 1024 trials 256, 160
-// in twos and 130 in fours.
+// in twos and 130 in fours.  Plans of up to 512 trials fill no wide pass; they
+// halve the rows instead, and a stage takes two bins (190 us for 4096 bins x
+// 1024 channels x 512 trials, 249 with rows for twice the trials).
 // The four adding warps do not take stages while they store an item, so that
 // must be short: Cb and Sb of a b are rows of one warp, which exchanges them
 // by shuffles (through shared memory and barriers of the four warps: 311 us
@@ -100,7 +102,7 @@ constexpr int kRows = 128;  // Cb, Sb of 64 b's: sixteen b's Cb, then their Sb, 
 // FP32 multiply-adds' sums lost little, and reached 3.0e-7.  A call of 63
 // channels x 277 trials x 347 bins takes 13 us either way.
 constexpr int kFewChan = 128;
-constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's
+constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's (twin: half)
 constexpr int kBlockAls = 8;      // al's of a whole block (2048 trials)
 
 // Warps: 0-3 epilogue (a warp reads the tensor-memory lanes of its quarter),
@@ -116,14 +118,24 @@ constexpr int kThreads = 32 * (kProdFirst + kProdWarps);
 // of trials of one series (each with its own centre), or the same trials of
 // kBlocks series (kSeries).  kNa: al's in all; kBins: bins a CTA works on at a
 // time (their accumulators share the epilogue's registers: kNa * kBins = 16).
-template <int kAls_, int kBlocks_, bool kSeries_>
+// For few trials the rows, too, are shared out (kTwin): a stage takes two bins
+// (the blocks), rows of 32 b's of each, and the epilogue the quarter of the
+// product that has rows and columns of the same bin.
+template <int kAls_, int kBlocks_, bool kSeries_, bool kTwin_ = false>
 struct Cfg {
   static constexpr int kAls = kAls_, kBlocks = kBlocks_, kNa = kAls * kBlocks;
-  static constexpr bool kSeries = kSeries_;
-  static constexpr int kSets = kSeries ? kBlocks : 1;     // spectra of a pass
-  static constexpr int kCentres = kSeries ? 1 : kBlocks;  // and centres
-  static constexpr int kPassTrials = kPairTrials * kAls * kCentres;
-  static constexpr int kBins = 16 / kNa;
+  static constexpr bool kSeries = kSeries_, kTwin = kTwin_;
+  static constexpr int kSeriesSets = kSeries ? kBlocks : 1;       // series of a pass
+  static constexpr int kSets = kSeries || kTwin ? kBlocks : 1;    // (series, bin)s of a stage
+  static constexpr int kRowBins = kTwin ? 2 : 1;                  // bins of a stage
+  static constexpr int kCentres = kSeries || kTwin ? 1 : kBlocks; // centres of a pass
+  static constexpr int kCentrePhases = kTwin ? 2 : kCentres;      // of a stage
+  static constexpr int kAlTrials = kPairTrials / kRowBins;
+  static constexpr int kMostAls = kAls * kCentres;
+  static constexpr int kPassTrials = kAlTrials * kMostAls;
+  static constexpr int kOwn = kTwin ? kAls : kNa;  // al's a thread of the epilogue adds up
+  static constexpr int kBins = 16 / kOwn;          // stages per 64 channels of an item
+  static constexpr int kItemBins = kBins * kRowBins;  // stage i: bins i (and kBins + i)
   static constexpr int kN = 4 * kNa;          // columns
   static constexpr int kStages = kNa == 16 ? 4 : 5;
   // (tables run further ahead than operands)
@@ -146,24 +158,24 @@ struct Cfg {
   static constexpr uint32_t kPark = kAccs * 2 * kN;
   static_assert(kPark + kSlots * 64 <= 512 && kAccs <= kStages, "tensor memory");
   static constexpr uint32_t kTmemCols = 512;
-  static_assert(kSeries || kBlocks == 1 || kAls == kBlockAls, "trials in whole blocks");
+  static_assert(kSeries || kTwin || kBlocks == 1 || kAls == kBlockAls, "trials in whole blocks");
   static_assert(kAls % 4 == 0, "the epilogue's four al's have one scale");
 };
 
 // Per stage: what the producers need of each channel.
-template <int kBlocks>
+template <class C>
 struct Table {
-  uint32_t hw[kCh];   // half the trial step's phase, units of 2^-32 cycle
-  uint32_t ha[kCh];   // 64 trial steps
-  float fr[kCh], fi[kCh];  // phasor of 16 trial steps (b -> b + 16)
-  float xr[kBlocks][kCh], xi[kBlocks][kCh];  // X rotated to each block's centre and scaled
+  uint32_t hw[C::kRowBins][kCh];   // half the trial step's phase, units of 2^-32 cycle
+  uint32_t ha[C::kRowBins][kCh];   // half the step of al's: 64 (32) trial steps
+  float fr[C::kRowBins][kCh], fi[C::kRowBins][kCh];  // phasor of 16 trial steps (b -> b + 16)
+  float xr[C::kBlocks][kCh], xi[C::kBlocks][kCh];  // X rotated to each block's centre and scaled
   int steps;               // K steps of 16 channels the MMAs read
   int pad[3];
 };
 template <class C>
 struct Smem {
   alignas(128) unsigned char stage[C::kStages][C::kStageBytes];
-  alignas(16) Table<C::kBlocks> table[C::kTables];
+  alignas(16) Table<C> table[C::kTables];
   float inv[4 * C::kTables][C::kSets];  // undoes a stage's scales (read by the epilogue, well after the table)
   uint64_t pfull[C::kTables], pfree[C::kTables];  // table written; every producer has read it
   uint64_t full[C::kStages], done[C::kStages];   // operands written; MMAs complete
@@ -289,7 +301,7 @@ __device__ __forceinline__ void sincos2(uint32_t p0, uint32_t p1, float2& cs, fl
   turn(q1, c.y, s.y, cs.y, sn.y);
 }
 
-// An item of the launch: bins k0 .. k0 + kBins - 1 of one set of spectra and
+// An item of the launch: kItemBins bins from k0 of one set of spectra and
 // the pass of up to 256 kNa trials from j_p.
 struct Item {
   int set;  // (first) series, or batch set
@@ -303,7 +315,7 @@ __host__ __device__ inline int n_passes(int n_dm) {
 // al's of block h of a pass with n_a al's (a series')
 template <class C>
 __device__ __forceinline__ int block_als(int n_a, int h) {
-  if (C::kSeries) return n_a;
+  if (C::kSeries || C::kTwin) return n_a;
   const int left = n_a - h * kBlockAls;
   return left < 0 ? 0 : left < kBlockAls ? left : kBlockAls;
 }
@@ -322,19 +334,18 @@ __device__ __forceinline__ Item decode(const MacArgs& a, const BatchSet* sets, i
     n_dm = sets[lo].args.n_dm;
     groups = sets[lo].n_bin_tiles;
   } else {
-    groups = (a.n_bins + C::kBins - 1) / C::kBins;
+    groups = (a.n_bins + C::kItemBins - 1) / C::kItemBins;
     n_dm = a.n_dm;
     const int per_set = groups * n_passes<C>(n_dm);
     q.set = item / per_set;
     local = item - q.set * per_set;
-    q.set *= C::kSets;
+    q.set *= C::kSeriesSets;
   }
   const int p = local / groups;
-  q.k0 = (local - p * groups) * C::kBins;
+  q.k0 = (local - p * groups) * C::kItemBins;
   q.j_p = p * C::kPassTrials;
-  const int als = (n_dm - q.j_p + kPairTrials - 1) / kPairTrials;
-  constexpr int kMost = C::kAls * C::kCentres;
-  q.n_a = als < kMost ? als : kMost;
+  const int als = (n_dm - q.j_p + C::kAlTrials - 1) / C::kAlTrials;
+  q.n_a = als < C::kMostAls ? als : C::kMostAls;
   return q;
 }
 
@@ -406,18 +417,19 @@ __global__ void __launch_bounds__(kThreads, 1)
     // A thread holds sixteen (bin, al) units of four sums each.
     const uint32_t t_lane = tmem + (static_cast<uint32_t>(warp * 32) << 16);
     const bool is_c = lane < 16;  // this lane's row: Cb, or Sb of the same b
-    const int b = 16 * warp + (lane & 15);
+    const int b = 16 * (C::kTwin ? warp & 1 : warp) + (lane & 15);
+    const int own = C::kTwin ? warp >> 1 : 0;  // this warp's bin of a stage
     uint32_t acc_at = 0;  // the stage's accumulator
     bool held = false;    // the last item's sums wait in slot 0 for this one's
     uint32_t n_item = 0;  // first stage of the item
     for (int i_item = 0; i_item < my_items && ok; ++i_item, n_item += per_item) {
-      float2 acc[kBins][4][kNa / 2];
+      float2 acc[kBins][4][C::kOwn / 2];
 #pragma unroll
       for (int s = 0; s < kBins; ++s)
 #pragma unroll
         for (int t = 0; t < 4; ++t)
 #pragma unroll
-          for (int i = 0; i < kNa / 2; ++i) acc[s][t][i] = make_float2(0.f, 0.f);
+          for (int i = 0; i < C::kOwn / 2; ++i) acc[s][t][i] = make_float2(0.f, 0.f);
       for (int c = 0; c < n_chunks && ok; ++c) {
 #pragma unroll
         for (int sl = 0; sl < kBins; ++sl) {
@@ -427,21 +439,21 @@ __global__ void __launch_bounds__(kThreads, 1)
           acc_at = acc_at + 1 == C::kAccs ? 0 : acc_at + 1;
           ok = ok && warp_wait(&sm.done[s], (n / S) & 1, abort_flag);
           if (!ok) break;
-          float hv[C::kSets];
+          float hv[C::kSeriesSets];
 #pragma unroll
-          for (int i = 0; i < C::kSets; ++i) hv[i] = sm.inv[n % (4 * C::kTables)][i];
+          for (int i = 0; i < C::kSeriesSets; ++i) hv[i] = sm.inv[n % (4 * C::kTables)][own + i];
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-          for (int h = 0; h < kNa / 4; ++h) {
+          for (int h = 0; h < C::kOwn / 4; ++h) {
             const float hs = hv[C::kSeries ? 4 * h / C::kAls : 0];
             const float2 inv = make_float2(hs, hs);
 #pragma unroll
             for (int t = 0; t < 4; t += 2) {
               // [type t, t + 1: hi hi; the small products of both][al]
               uint32_t r[4][4];
-              const uint32_t col = t_lane + d * 2 * kN + t * kNa + 4 * h;
+              const uint32_t col = t_lane + d * 2 * kN + t * kNa + own * C::kAls + 4 * h;
               tmem_ld4x4(col, col + kNa, col + kN, col + kN + kNa, r);
-              if (h == kNa / 4 - 1 && t == 2) {
+              if (h == C::kOwn / 4 - 1 && t == 2) {
                 asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
                 mbar_arrive_warp(&sm.acc_free[d]);
               }
@@ -491,7 +503,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       // with Sb: the lane of a Cb row makes the trials of s = +, that of the
       // Sb row of the same b those of s = -, each with two values of the other.
       constexpr int kOut = C::kOutBins;
-      const int k0 = held ? q.k0 - 1 : q.k0;
+      const int k0 = held ? q.k0 - 1 : q.k0 + own * kBins;
       const MacArgs& m = sets ? sets[q.set].args : a;
       const int64_t dm_stride = m.y_dm_stride;
       const int n_dm = m.n_dm, out_kind = m.out_kind;
@@ -504,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       held = false;
       const float sg = is_c ? 1.f : -1.f;
 #pragma unroll (C::kSlots > 0 ? 1 : kNa)
-      for (int al = 0; al < kNa; ++al) {
+      for (int al = 0; al < C::kOwn; ++al) {
         if (C::kSeries ? al % C::kAls < q.n_a : al < q.n_a) {
           float v[kOut][4];
           if constexpr (C::kSlots > 1)
@@ -527,9 +539,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             y[1][sl] = make_float2((A.x + B.y) * scale, real_only ? 0.f : (A.y - B.x) * scale);
           }
           // trial of (s, al, t, b)
-          const int h = al / C::kAls, step = 128 * (al % C::kAls) + 64;
+          const int h = al / C::kAls, step = C::kAlTrials / 2 * (al % C::kAls) + C::kAlTrials / 4;
           const int jc = q.j_p + (C::kSeries ? 0 : kPairTrials * kBlockAls * h) +
-                         kPairTrials / 2 * block_als<C>(q.n_a, h) + (is_c ? step : -step);
+                         C::kAlTrials / 2 * block_als<C>(q.n_a, h) + (is_c ? step : -step);
           const int64_t off_h = off + (C::kSeries ? h * m.y_series_stride : 0);
 #pragma unroll
           for (int t = 0; t < 2; ++t) {
@@ -649,7 +661,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       uint32_t before[C::kCentres];  // Jc - 1/2: the trial below each block's centre
       int c0;           // this lane's first channel
       int steps;        // K steps of the stage
-      bool bin_ok;
+      bool bin_ok[C::kRowBins];
     };
     const int p = warp - kPrepFirst;
     int i_item = 0, q = p;  // stage within the item
@@ -676,7 +688,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int h = 0; h < C::kCentres; ++h)
           before[h] = static_cast<uint32_t>(m.j_begin + it.j_p + kPairTrials * kBlockAls * h +
-                                            kPairTrials / 2 * block_als<C>(it.n_a, h) - 1);
+                                            C::kAlTrials / 2 * block_als<C>(it.n_a, h) - 1);
         X = m.X + (sets ? 0 : static_cast<int64_t>(it.set) * m.x_series_stride) + it.k0;
         xs = m.x_chan_stride;
         set_stride = m.x_series_stride;
@@ -685,11 +697,14 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int slot = q % kBins;
       f.steps = q >= per_item - kBins ? tail_steps : 4;
       f.c0 = q / kBins * kCh + lane;
-      f.bin_ok = slot < left_bins;
+#pragma unroll
+      for (int i = 0; i < C::kRowBins; ++i) f.bin_ok[i] = slot + i * kBins < left_bins;
       f.k = static_cast<uint32_t>(k_abs + slot);
 #pragma unroll
       for (int h = 0; h < C::kCentres; ++h) f.before[h] = before[h];
-      const float2* xb = X + (f.bin_ok ? slot : 0);
+      const float2* xb[C::kRowBins];
+#pragma unroll
+      for (int i = 0; i < C::kRowBins; ++i) xb[i] = X + (f.bin_ok[i] ? slot + i * kBins : 0);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = min(f.c0 + 32 * h, n_chan - 1);
@@ -700,7 +715,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int i = 0; i < C::kSets; ++i)
           asm volatile("ld.global.nc.v2.f32 {%0,%1}, [%2];"
                        : "=f"(f.x[i][h].x), "=f"(f.x[i][h].y)
-                       : "l"(xb + i * set_stride + static_cast<int64_t>(c) * xs));
+                       : "l"(xb[C::kTwin ? i : 0] + (C::kTwin ? 0 : i * set_stride) +
+                             static_cast<int64_t>(c) * xs));
       }
       q += kPrepWarps;
     };
@@ -723,7 +739,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t top = 0;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const bool use = next.bin_ok && next.c0 + 32 * h < n_chan;
+          const bool use = next.bin_ok[C::kTwin ? i : 0] && next.c0 + 32 * h < n_chan;
           x[h] = use ? next.x[i][h] : make_float2(0.f, 0.f);
           top = max(top, max(__float_as_uint(x[h].x) & 0x7FFFFFFFu, __float_as_uint(x[h].y) & 0x7FFFFFFFu));
         }
@@ -734,42 +750,52 @@ __global__ void __launch_bounds__(kThreads, 1)
         xr[i] = make_float2(x[0].x * sc, x[1].x * sc);
         xi[i] = make_float2(x[0].y * sc, x[1].y * sc);
       }
-      uint32_t hw[2], ha[2], pf[2], pm[C::kCentres][2];
+      uint32_t hw[C::kRowBins][2], ha[C::kRowBins][2], pf[C::kRowBins][2], pm[C::kCentrePhases][2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint64_t u = (static_cast<uint64_t>(pc[h].y) << 32) | pc[h].x;
         const uint64_t v = (static_cast<uint64_t>(pc[h].w) << 32) | pc[h].z;
-        const uint64_t half = (v * k) >> 1;  // half a trial step, mod half a cycle
         constexpr uint64_t kRound = 0x80000000ull;
-        hw[h] = static_cast<uint32_t>((half + kRound) >> 32);
-        ha[h] = static_cast<uint32_t>(((half << 7) + kRound) >> 32);
-        pf[h] = static_cast<uint32_t>(((half << 5) + kRound) >> 32);
+        constexpr int kAlShift = C::kTwin ? 6 : 7;
 #pragma unroll
-        for (int i = 0; i < C::kCentres; ++i)  // the blocks' centres
-          pm[i][h] = static_cast<uint32_t>(((u + v * j1[i]) * k + half) >> 32);
+        for (int e = 0; e < C::kRowBins; ++e) {
+          const uint32_t ke = k + e * kBins;
+          const uint64_t half = (v * ke) >> 1;  // half a trial step, mod half a cycle
+          hw[e][h] = static_cast<uint32_t>((half + kRound) >> 32);
+          ha[e][h] = static_cast<uint32_t>(((half << kAlShift) + kRound) >> 32);
+          pf[e][h] = static_cast<uint32_t>(((half << 5) + kRound) >> 32);
+#pragma unroll
+          for (int i = 0; i < C::kCentres; ++i)  // the blocks' centres
+            pm[C::kTwin ? e : i][h] = static_cast<uint32_t>(((u + v * j1[i]) * ke + half) >> 32);
+        }
       }
-      float2 fc, fs, zr[C::kBlocks], zi[C::kBlocks];
-      sincos2(pf[0], pf[1], fc, fs);
+      float2 fc[C::kRowBins], fs[C::kRowBins], zr[C::kBlocks], zi[C::kBlocks];
+#pragma unroll
+      for (int e = 0; e < C::kRowBins; ++e) sincos2(pf[e][0], pf[e][1], fc[e], fs[e]);
       float2 mc, ms;
 #pragma unroll
       for (int i = 0; i < C::kBlocks; ++i) {
-        if (i < C::kCentres) sincos2(pm[i % C::kCentres][0], pm[i % C::kCentres][1], mc, ms);
-        const int e = C::kSeries ? i : 0;
+        if (i < C::kCentrePhases)
+          sincos2(pm[i % C::kCentrePhases][0], pm[i % C::kCentrePhases][1], mc, ms);
+        const int e = C::kSets > 1 ? i : 0;
         zr[i] = __ffma2_rn(xr[e], mc, __fmul2_rn(make_float2(-xi[e].x, -xi[e].y), ms));
         zi[i] = __ffma2_rn(xr[e], ms, __fmul2_rn(xi[e], mc));
       }
       fetch(next);
       ok = warp_wait(&sm.pfree[s], ((n / T) & 1) ^ 1, abort_flag);
       if (!ok) break;
-      Table<C::kBlocks>& tb = sm.table[s];
-      tb.hw[lane] = hw[0];
-      tb.hw[lane + 32] = hw[1];
-      tb.ha[lane] = ha[0];
-      tb.ha[lane + 32] = ha[1];
-      tb.fr[lane] = fc.x;
-      tb.fr[lane + 32] = fc.y;
-      tb.fi[lane] = fs.x;
-      tb.fi[lane + 32] = fs.y;
+      Table<C>& tb = sm.table[s];
+#pragma unroll
+      for (int e = 0; e < C::kRowBins; ++e) {
+        tb.hw[e][lane] = hw[e][0];
+        tb.hw[e][lane + 32] = hw[e][1];
+        tb.ha[e][lane] = ha[e][0];
+        tb.ha[e][lane + 32] = ha[e][1];
+        tb.fr[e][lane] = fc[e].x;
+        tb.fr[e][lane + 32] = fc[e].y;
+        tb.fi[e][lane] = fs[e].x;
+        tb.fi[e][lane + 32] = fs[e].y;
+      }
 #pragma unroll
       for (int i = 0; i < C::kBlocks; ++i) {
         tb.xr[i][lane] = zr[i].x;
@@ -807,7 +833,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t ts = n % T;
       ok = warp_wait(&sm.pfull[ts], (n / T) & 1, abort_flag);
       if (!ok) break;
-      const Table<C::kBlocks>& tb = sm.table[ts];
+      const Table<C>& tb = sm.table[ts];
       const int steps = tb.steps;
       if (rows) {
         // rows: lane = (b < 16, half of an octet of channels): Cb, Sb of four
@@ -821,26 +847,30 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int o = 0; o < 2; ++o) {
             const int oct = 2 * part + o;
             const int ch = 8 * oct + 4 * half;
-            const uint4 hv = *reinterpret_cast<const uint4*>(&tb.hw[ch]);
-            const float4 frv = *reinterpret_cast<const float4*>(&tb.fr[ch]);
-            const float4 fiv = *reinterpret_cast<const float4*>(&tb.fi[ch]);
             uint32_t hi[8][2], lo[8][2];  // [C, S of b + 16 i][channel pair]
 #pragma unroll
-            for (int p = 0; p < 2; ++p) {
-              const float2 fr = p ? make_float2(frv.z, frv.w) : make_float2(frv.x, frv.y);
-              const float2 fi = p ? make_float2(fiv.z, fiv.w) : make_float2(fiv.x, fiv.y);
-              const float2 nfi = make_float2(-fi.x, -fi.y);
-              const float2 w0 = unit_phasor(mul * (p ? hv.z : hv.x));
-              const float2 w1 = unit_phasor(mul * (p ? hv.w : hv.y));
-              float2 cs = make_float2(w0.x, w1.x), sn = make_float2(w0.y, w1.y);
+            for (int e = 0; e < C::kRowBins; ++e) {  // (twin: i = 0, 1 of each bin)
+              const uint4 hv = *reinterpret_cast<const uint4*>(&tb.hw[e][ch]);
+              const float4 frv = *reinterpret_cast<const float4*>(&tb.fr[e][ch]);
+              const float4 fiv = *reinterpret_cast<const float4*>(&tb.fi[e][ch]);
+              constexpr int kSteps = 4 / C::kRowBins;
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                split2(cs, hi[i][p], lo[i][p]);
-                split2(sn, hi[4 + i][p], lo[4 + i][p]);
-                if (i < 3) {
-                  const float2 c1 = __ffma2_rn(cs, fr, __fmul2_rn(sn, nfi));
-                  sn = __ffma2_rn(cs, fi, __fmul2_rn(sn, fr));
-                  cs = c1;
+              for (int p = 0; p < 2; ++p) {
+                const float2 fr = p ? make_float2(frv.z, frv.w) : make_float2(frv.x, frv.y);
+                const float2 fi = p ? make_float2(fiv.z, fiv.w) : make_float2(fiv.x, fiv.y);
+                const float2 nfi = make_float2(-fi.x, -fi.y);
+                const float2 w0 = unit_phasor(mul * (p ? hv.z : hv.x));
+                const float2 w1 = unit_phasor(mul * (p ? hv.w : hv.y));
+                float2 cs = make_float2(w0.x, w1.x), sn = make_float2(w0.y, w1.y);
+#pragma unroll
+                for (int i = 0; i < kSteps; ++i) {
+                  split2(cs, hi[e * kSteps + i][p], lo[e * kSteps + i][p]);
+                  split2(sn, hi[4 + e * kSteps + i][p], lo[4 + e * kSteps + i][p]);
+                  if (i + 1 < kSteps) {
+                    const float2 c1 = __ffma2_rn(cs, fr, __fmul2_rn(sn, nfi));
+                    sn = __ffma2_rn(cs, fi, __fmul2_rn(sn, fr));
+                    cs = c1;
+                  }
                 }
               }
             }
@@ -876,7 +906,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             const int ch = 4 * (h0 + e * kHalves);
-            const uint4 hv = *reinterpret_cast<const uint4*>(&tb.ha[ch]);
+            const uint4 hv = *reinterpret_cast<const uint4*>(&tb.ha[C::kTwin ? blk : 0][ch]);
             const float4 xrv = *reinterpret_cast<const float4*>(&tb.xr[blk][ch]);
             const float4 xiv = *reinterpret_cast<const float4*>(&tb.xi[blk][ch]);
 #pragma unroll
@@ -937,9 +967,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
 }
 
-// The passes' forms: one series with up to 1024, 2048 or 4096 trials a pass,
+// The passes' forms: one series with up to 512 (two bins a stage), 1024, 2048 or
+// 4096 trials a pass,
 // or two or four series that share the rows of up to 1024, two of up to 2048.
-enum Form { kUpTo1024, kUpTo2048, kUpTo4096, kTwoUpTo1024, kFourUpTo1024, kTwoUpTo2048, kForms };
+enum Form { kUpTo512, kUpTo1024, kUpTo2048, kUpTo4096, kTwoUpTo1024, kFourUpTo1024, kTwoUpTo2048, kForms };
 
 struct FormInfo {
   const void* fn;
@@ -948,10 +979,11 @@ struct FormInfo {
 template <class C>
 FormInfo form_info() {
   return {reinterpret_cast<const void*>(&mac_split_kernel<C>), static_cast<int>(sizeof(Smem<C>)) + 128,
-          C::kSets, C::kBins, C::kPassTrials};
+          C::kSeriesSets, C::kItemBins, C::kPassTrials};
 }
 FormInfo form_info(Form f) {
   switch (f) {
+    case kUpTo512: return form_info<Cfg<4, 2, false, true>>();
     case kUpTo1024: return form_info<Cfg<4, 1, false>>();
     case kUpTo2048: return form_info<Cfg<8, 1, false>>();
     case kUpTo4096: return form_info<Cfg<8, 2, false>>();
@@ -962,10 +994,16 @@ FormInfo form_info(Form f) {
 }
 
 // The form for n_dm trials of n_series (at least its sets) series.  The rows
-// take most of a stage, so the widest pass that the trials or series fill.
-Form form_for(int n_dm, int n_series) {
+// take most of a stage, so the widest pass that the trials or series fill, and
+// half the rows where the plan (or batch) has no more than 512 trials (of_n_dm):
+// calls on parts of its trials then take the same form as the whole.  The form
+// may depend on the series only among those whose results are the same bits.
+// 4096 bins x 1024 channels x 512 trials take 190 us in twin stages, 249 in
+// those for 1024.
+Form form_for(int n_dm, int n_series, int of_n_dm) {
   const int total = (n_dm + kPairTrials - 1) / kPairTrials;
   if (total > 8) return kUpTo4096;
+  if (of_n_dm > 0 && of_n_dm <= 2 * kPairTrials) return kUpTo512;
   if (total > 4) return n_series >= 2 ? kTwoUpTo2048 : kUpTo2048;
   return n_series >= 4 ? kFourUpTo1024 : n_series >= 2 ? kTwoUpTo1024 : kUpTo1024;
 }
@@ -1018,10 +1056,10 @@ cudaError_t mac_split_prepare() {
   return e;
 }
 
-bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2)).sets > 1; }
+bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2, n_dm)).sets > 1; }
 
 void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes) {
-  const FormInfo f = form_info(form_for(max_n_dm, 1));
+  const FormInfo f = form_info(form_for(max_n_dm, 1, max_n_dm));
   *bin_groups = static_cast<int>((n_bins + f.bins - 1) / f.bins);
   *passes = (n_dm + f.pass_trials - 1) / f.pass_trials;
 }
@@ -1031,7 +1069,7 @@ cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long
   if (n_items <= 0) return cudaSuccess;
   if (n_items > kMaxItems) return cudaErrorInvalidConfiguration;
   return launch_split(MacArgs{}, d_sets, n_sets, static_cast<int>(n_items),
-                      form_info(form_for(max_n_dm, 1)), n_ctas, s);
+                      form_info(form_for(max_n_dm, 1, max_n_dm)), n_ctas, s);
 }
 
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
@@ -1041,7 +1079,7 @@ cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
   const size_t y_elem = a.out_kind == 2 ? sizeof(float) : sizeof(float2);
   // series in groups that share passes, then the rest by themselves
   for (int s0 = 0; s0 < a.n_series;) {
-    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0));
+    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0, a.of_n_dm));
     const long long per_set = static_cast<long long>((a.n_bins + f.bins - 1) / f.bins) *
                               ((a.n_dm + f.pass_trials - 1) / f.pass_trials);
     if (per_set > kMaxItems) return cudaErrorInvalidConfiguration;

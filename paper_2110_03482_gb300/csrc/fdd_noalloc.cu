@@ -130,6 +130,7 @@ extern "C" fdd_status fdd_dedisperse_spectra_static(const fdd_params* p, const v
   m.n_series = n_series;
   m.j_begin = dm_first;
   m.n_dm = n_dm;
+  m.of_n_dm = p->n_dm;
   m.Y = d_Y;
   m.y_dm_stride = y_pitch;
   m.y_series_stride = y_pitch * n_dm;

@@ -141,10 +141,10 @@ def test_series_sharing_passes_equal_each_alone(n_series, n_dm):
 
 @pytest.mark.parametrize("output", [fdd.FDD_OUT_TIME, fdd.FDD_OUT_SPECTRA, fdd.FDD_OUT_POWER])
 @pytest.mark.parametrize("n_beams,n_t,chunk_len,n_dm", [
-    (1, 20000, 1 << 12, 300),    # chunks of one beam, an odd number
+    (1, 20000, 1 << 12, 600),    # chunks of one beam, an odd number
     (3, 20000, 1 << 13, 1100),   # beams and chunks, two of different beams together
     (2, 4096, 0, 2048),          # whole rows, no chunks
-    (1, 9000, 1 << 12, 257),
+    (1, 9000, 1 << 12, 513),
 ])
 def test_plans_that_take_two_at_a_time_give_the_same_bits(n_beams, n_t, chunk_len, n_dm, output):
     """A plan with room for two (beam, chunk)s a launch against one whose

@@ -287,6 +287,149 @@ __global__ void __launch_bounds__(W * 32, 1) mac_kernel(const MacArgs a) {
   mac_block<Gm, M, W>(a, pcs, swap_all, blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
+// ------------------------------------- small calls: channels shared by warps
+// The 128-trial tile's calls are mostly small (64 channels x 128 trials x 2049
+// bins are 513 warps of four bins for 608 schedulers), and a warp alone waits
+// for its own results five cycles of six.  So kParts warps share the bins, each
+// with a part of the channels, and add their sums up at the end; a warp
+// evaluates a group of kGroup channels while it accumulates the group before;
+// and X arrives kXAhead batches of eight channels early.  Groups of two keep
+// the swap areas small enough for three CTAs an SM.  The split depends on
+// nothing but the channels, so calls on parts of the bins or trials agree
+// bit for bit.  Against a warp taking all the channels one by one: 64 channels
+// x 128 trials x 2049 bins 21.2 -> 10.6 us a call (8 of which the host takes),
+// 1024 channels x 250 trials x 500 bins 279 -> 76, x 186 trials x 4096 bins
+// 393 -> 301, 100 channels x 128 trials x 9000 bins 44.8 -> 44.7.  (Groups of four, two
+// CTAs an SM: 10.7, 76, 340 and 50 us; evaluating ahead alone, without the
+// split: 18.7, 217, 492, 43.)
+constexpr int kParts = 4, kBinSets = 2;  // warps per four bins; fours of bins per CTA
+constexpr int kGroup = 2, kXAhead = 4;
+struct SplitQ {
+  using Gm = G4x4;
+  using M = PackedCompact<G4x4>;
+  static constexpr int kWarpsOf = kParts * kBinSets;
+  static constexpr int kStage = Gm::NG * M::GFL;            // floats of a channel
+  static constexpr int kSwap = 2 * kGroup * kStage;         // of a warp's two swap areas
+  static constexpr int kRing = 2 * 32 * kXAhead;            // and its X ring
+  static constexpr int kSums = 2 * Gm::AT * Gm::BT * 32;    // the sums, over the swap areas
+  static_assert(kSums <= kSwap, "sums fit the swap areas");
+  static size_t smem(int n_chan) {
+    return sizeof(PhaseConst) * static_cast<size_t>(n_chan) +
+           sizeof(float) * static_cast<size_t>(kWarpsOf) * (kSwap + kRing);
+  }
+};
+
+__global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(const MacArgs a) {
+  using Gm = SplitQ::Gm;
+  using M = SplitQ::M;
+  constexpr int kStage = SplitQ::kStage;
+  static_assert(Gm::NG == 4 && 8 % (2 * kGroup) == 0, "a batch of X is eight channels x four bins");
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  PhaseConst* pcs = reinterpret_cast<PhaseConst*>(smem_raw);
+  float* areas = reinterpret_cast<float*>(smem_raw + sizeof(PhaseConst) * a.n_chan);
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int part = warp % kParts, set = warp / kParts;
+  float* const swap = areas + warp * (SplitQ::kSwap + SplitQ::kRing);
+  float2* const ring = reinterpret_cast<float2*>(swap + SplitQ::kSwap);
+  const int g = lane / Gm::G, lg = lane % Gm::G;
+  const int ga = lg / Gm::GB, gb = lg % Gm::GB;
+  const int k4 = (blockIdx.x * kBinSets + set) * 4;  // the four bins
+  const int k = k4 + g;
+  const int series = blockIdx.z;
+  const int jblk = blockIdx.y * Gm::DMS;
+  // this warp's channels; c0 below counts from the first
+  const int each = (a.n_chan + kParts - 1) / kParts;
+  const int c_lo = min(part * each, a.n_chan), n_c = min(c_lo + each, a.n_chan) - c_lo;
+
+  const int k_mine = k4 + (lane & 3);
+  const float2* x_mine = a.X + static_cast<int64_t>(series) * a.x_series_stride +
+                         (k_mine < a.n_bins ? k_mine : 0);  // (idle bins: bin 0, not stored)
+  auto fetch = [&](int c0) {  // an element a lane (zeros beyond the part)
+    const int c = c0 + (lane >> 2);
+    const bool in = c < n_c;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                     dev::smem_u32(ring + (c0 / 8 % kXAhead) * 32 + lane)),
+                 "l"(x_mine + static_cast<int64_t>(in ? c_lo + c : 0) * a.x_chan_stride), "r"(in ? 8 : 0)
+                 : "memory");
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  for (int b = 0; b < kXAhead; ++b) fetch(8 * b);
+  for (int i = threadIdx.x; i < a.n_chan; i += SplitQ::kWarpsOf * 32) pcs[i] = a.pc[i];
+  __syncthreads();
+
+  Generator<Gm, M> gen;
+  gen.init(static_cast<uint32_t>(a.k_begin + (k < a.n_bins ? k : 0)), lg, a.j_begin + jblk);
+  float* const grp0 = swap + g * M::GFL;
+  typename M::Acc acc;
+  M::zero(acc);
+  auto evaluate = [&](int c0, int area) {
+#pragma unroll
+    for (int i = 0; i < kGroup; ++i)
+      if (c0 + i < n_c)
+        gen.run(pcs[c_lo + c0 + i], ring[(c0 / 8 % kXAhead) * 32 + (c0 % 8 + i) * 4 + g],
+                grp0 + (area * kGroup + i) * kStage);
+  };
+  auto accumulate = [&](int c0, int area) {
+#pragma unroll
+    for (int i = 0; i < kGroup; ++i) {
+      if (c0 + i < n_c) {
+        typename M::Ops ops;
+        M::load(grp0 + (area * kGroup + i) * kStage, ga, gb, ops);
+        M::mac(acc, ops);
+      }
+    }
+  };
+  // Two swap areas: a group is evaluated into the one that the accumulation
+  // before the last sync has read, while the group before it is accumulated.
+  asm volatile("cp.async.wait_group %0;" ::"n"(kXAhead - 1) : "memory");
+  __syncwarp();
+  evaluate(0, 0);
+  for (int c0 = 0; c0 < n_c; c0 += 8) {
+#pragma unroll
+    for (int i = 0; i < 8; i += kGroup) {
+      if (i + kGroup == 8) asm volatile("cp.async.wait_group %0;" ::"n"(kXAhead - 2) : "memory");
+      __syncwarp();
+      if (i + kGroup == 8) fetch(c0 + 8 * kXAhead);
+      evaluate(c0 + i + kGroup, (i / kGroup + 1) & 1);
+      accumulate(c0 + i, (i / kGroup) & 1);
+    }
+  }
+
+  // The parts' sums: each warp adds one row of the lanes' tiles, in the parts'
+  // order, and stores it.
+  static_assert(Gm::AT == kParts, "a row of the tile for each warp");
+  __syncwarp();
+  float2* const sums = reinterpret_cast<float2*>(swap);
+#pragma unroll
+  for (int ii = 0; ii < Gm::AT; ++ii)
+#pragma unroll
+    for (int jj = 0; jj < Gm::BT; ++jj) sums[(ii * Gm::BT + jj) * 32 + lane] = M::get(acc, ii, jj);
+  __syncthreads();
+  if (k >= a.n_bins) return;
+  const bool real_only = (a.k_begin + k == a.real_bin_a) || (a.k_begin + k == a.real_bin_b);
+#pragma unroll
+  for (int jj = 0; jj < Gm::BT; ++jj) {
+    float2 v = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int q = 0; q < kParts; ++q)
+      v = __fadd2_rn(v, reinterpret_cast<const float2*>(
+                            areas + (set * kParts + q) * (SplitQ::kSwap + SplitQ::kRing))[
+                            (part * Gm::BT + jj) * 32 + lane]);
+    const int jl = jblk + (ga * Gm::AT + part) * Gm::TW + gb * Gm::BT + jj;
+    if (jl < a.n_dm) {
+      const float re = v.x * a.scale;
+      const float im = real_only ? 0.f : v.y * a.scale;
+      const int64_t o = static_cast<int64_t>(series) * a.y_series_stride +
+                        static_cast<int64_t>(jl) * a.y_dm_stride + k;
+      if (a.out_kind == 2)
+        static_cast<float*>(a.Y)[o] = re * re + im * im;
+      else
+        static_cast<float2*>(a.Y)[o] = make_float2(re, im);
+    }
+  }
+}
+
 // --------------------------------------------- warp-specialised schedule
 // The plain schedule makes every warp alternate between the
 // latency-bound phasor evaluation (integer phase, MUFU sin/cos, the swap) and
@@ -604,13 +747,11 @@ VariantInfo variant_info(int v) {
 }  // namespace
 
 // Default tile for a trial count.  From 257 trials on the G12 tile while the
-// channels allow it: on 4096 bins x 1024 channels its passes of up to 1024,
-// 2048 and 4096 trials take 247, 305 and 430 us whatever their filling, the
-// 128-trial tile 624 us at 257 trials and 767 at 512.  (From 129 to 256 trials
-// the G12 tile would be the faster one too with many channels, 247 against
-// 392 us; plans have always reported Q_4X4 there, and keep to it.  Up to 128
-// the two are within 17 % at 1024 channels and Q_4X4 is 1.4-1.7 times faster
-// at 64 to 200.)  Otherwise the tile with the least time for the padded trial
+// channels allow it: on 4096 bins x 1024 channels its passes of up to 512,
+// 1024, 2048 and 4096 trials take 190, 250, 300 and 430 us whatever their filling,
+// the 128-trial tile 310 us at 256 trials and more with every 128.  (From 129 to
+// 256 trials the G12 tile would be the faster one too with many channels; plans
+// have always reported Q_4X4 there, and keep to it.)  Otherwise the tile with the least time for the padded trial
 // blocks, ceil(n_dm / block) * block / rate, with each tile's rate measured
 // kernel-only (fraction of the FP32 peak, 1024 channels, 131073 bins): Q_4x8
 // 0.493 (1024-trial blocks), Q_8x8_512 0.415 (512), Q_4x4 0.347 (128).  (The
@@ -651,6 +792,10 @@ cudaError_t mac_prepare(int variant, int n_chan) {
   const VariantInfo vi = variant_info(variant);
   const int bytes = static_cast<int>(mac_smem_bytes(variant, n_chan));
   cudaError_t e = cudaFuncSetAttribute(vi.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && variant == MAC_Q_4x4 && SplitQ::smem(n_chan) <= kMaxSmem)
+    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&mac_parts_kernel),
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             static_cast<int>(SplitQ::smem(n_chan)));
   if (e != cudaSuccess || !vi.batch_fn) return e;
   return cudaFuncSetAttribute(vi.batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
@@ -692,16 +837,23 @@ cudaError_t launch_mac_batch(const BatchSet* d_sets, int n_sets, long long n_ite
 cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s) {
   if (a.n_dm <= 0 || a.n_series <= 0 || a.n_bins <= 0) return cudaSuccess;
   if (variant == MAC_G12_4x8) return launch_mac_split(a, s);
-  const VariantInfo vi = variant_info(variant);
-  const int bins_per_cta = vi.bins();
+  VariantInfo vi = variant_info(variant);
+  size_t smem = mac_smem_bytes(variant, a.n_chan);
+  int bins_per_cta = vi.bins();
+  // (up to 11,000 channels, whose table fits beside the swap areas)
+  if (variant == MAC_Q_4x4 && SplitQ::smem(a.n_chan) <= kMaxSmem) {
+    vi.fn = reinterpret_cast<const void*>(&mac_parts_kernel);
+    vi.warps = SplitQ::kWarpsOf;
+    bins_per_cta = 4 * kBinSets;
+    smem = SplitQ::smem(a.n_chan);
+  }
   dim3 grid((a.n_bins + bins_per_cta - 1) / bins_per_cta, (a.n_dm + vi.dms - 1) / vi.dms,
             a.n_series);
   if (grid.y > 65535u || grid.z > 65535u) return cudaErrorInvalidConfiguration;
   MacArgs args = a;
   void* params[] = {&args};
   note_launches(1);
-  return cudaLaunchKernel(vi.fn, grid, dim3(vi.warps * 32), params,
-                          mac_smem_bytes(variant, a.n_chan), s);
+  return cudaLaunchKernel(vi.fn, grid, dim3(vi.warps * 32), params, smem, s);
 }
 
 }  // namespace fdd

@@ -42,7 +42,7 @@ METRIC = "DM·channel·bin phasor-MACs/s and % of FP32/tensor peak, batched TC v
 UNIT = "phasor-MAC/s"
 DEFAULT_WORKLOAD = "fdd_1024ch_2p20t_2048dm"
 FLOPS_PER_MAC = 8
-MAC_SOURCE = os.path.join(ROOT, "paper_2110_03482_gb300", "csrc", "fdd_mac_fp32.cu")
+MAC_SOURCE = os.path.join(ROOT, "paper_2110_03482_gb300", "csrc", "fdd_mac_split.cu")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "mac_g12_survey_1024ch_2048dm.md")
 
 
@@ -438,7 +438,8 @@ def job_rate(units_per_rank_step: float, steps: int, world: int, ms_max: float) 
     return units_per_rank_step * steps * world / (ms_max / 1e3)
 
 
-TDD_SMEM_ADDS_PER_CLK = 32  # one 4-byte shared load per add, 128 B per clock per SM
+TDD_SMEM_ADDS_PER_CLK = 32  # floats: one 4-byte shared load per add, 128 B per clock per SM
+TDD_INT_ADDS_PER_CLK = 64 * 16 / 13  # bytes: 13 integer instructions per 16 adds, 64 lanes a clock
 
 
 def measure_tdd(plan, w, info, d_in, stream, torch, sm_count, fdd_ms_per_step, reps=3) -> dict:
@@ -461,13 +462,16 @@ def measure_tdd(plan, w, info, d_in, stream, torch, sm_count, fdd_ms_per_step, r
     ms = e0.elapsed_time(e1) / reps
     kernel_ms = prof["ms"]["tdd"] / max(prof["launches"]["tdd"], 1)
     adds = w.n_dm * w.n_chan * out_len
-    peak = TDD_SMEM_ADDS_PER_CLK * sm_count * float(load_peaks().get("sm_max_mhz") or 2070) * 1e6
+    as_bytes = w.dtype == "u8"
+    per_clk = TDD_INT_ADDS_PER_CLK if as_bytes else TDD_SMEM_ADDS_PER_CLK
+    peak = per_clk * sm_count * float(load_peaks().get("sm_max_mhz") or 2070) * 1e6
     del y
     return {"method": "brute-force time-domain shift-and-sum (Eq. 2), same workload",
             "ms_per_step": ms, "kernel_ms": kernel_ms,
             "adds_per_s_kernel": adds / (kernel_ms / 1e3),
-            "frac_smem_bound": adds / (kernel_ms / 1e3) / peak,
-            "bound": f"shared memory: {TDD_SMEM_ADDS_PER_CLK} adds (4-byte loads) per clock per SM",
+            "frac_of_bound": adds / (kernel_ms / 1e3) / peak,
+            "bound": f"integer pipe: {per_clk:.0f} adds (bytes in pairs) per clock per SM" if as_bytes
+                     else f"shared memory: {per_clk} adds (4-byte loads) per clock per SM",
             "output_samples_per_trial": out_len,
             "fdd_over_tdd_time": fdd_ms_per_step / ms}
 
@@ -674,22 +678,31 @@ def run_fdd(args, rank: int, world: int, dist) -> None:
     # dominant kernel: the phasor-MAC
     mac_n = prof["launches"]["mac"]
     mac_ms = prof["ms"]["mac"] / max(mac_n, 1)
-    flops_launch = FLOPS_PER_MAC * min(info["dm_batch"], w.n_dm) * w.n_chan * info["n_bins"]
+    # (average over the launches: some take two beams or chunks)
+    flops_launch = FLOPS_PER_MAC * macs_step * args.steps / max(mac_n, 1)
     achieved = flops_launch / (mac_ms / 1e3) / 1e12
     peaks = load_peaks()
     max_mhz = float(peaks.get("sm_max_mhz") or clk.get("sm_max_mhz") or 2070.0)
     peak = sm_count * 128 * 2 * max_mhz * 1e6 / 1e12
     traffic = read_traffic_summary()
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
-                "frac": achieved / peak, "traffic": traffic,
+    split = info["mac_variant"] == fdd.FDD_MAC_G12_4X8  # FP16 halves on the tensor cores
+    bound_peak = float(peaks.get("bf16_tflops_sustained") or 1723.8) if split else peak
+    roofline = {"bound": "tensor" if split else "alu", "achieved": achieved, "peak": bound_peak,
+                "unit": "TFLOP/s", "frac": achieved / bound_peak, "traffic": traffic,
                 "kernel": "phase-rotate-and-sum (Eqs. 4 and 7), variant "
                           + fdd.MAC_VARIANT_NAMES[info["mac_variant"]],
-                "peak_source": f"derived: {sm_count} SMs x 128 FP32 lanes x 2 flop x "
+                "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (measured; FP16 "
+                               "operands run at the BF16 rate)" if split else
+                               f"derived: {sm_count} SMs x 128 FP32 lanes x 2 flop x "
                                f"{max_mhz:.0f} MHz max SM clock (FP32 FFMA; "
                                "MEASURED_PEAKS.json has no FP32 figure)",
                 "algorithmic_flops_per_launch": flops_launch,
                 "mac_ms_per_launch": mac_ms, "mac_launches_timed": mac_n}
-    if clk.get("sm_mhz"):
+    if split:
+        # two real products per complex one (trials in pairs), three FP16 ones each
+        roofline["tensor_frac_physical"] = 12 / FLOPS_PER_MAC * achieved / bound_peak
+        roofline["over_fp32_peak"] = achieved / peak
+    elif clk.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = achieved / (peak * clk["sm_mhz"] / max_mhz)
     stage_share = {k: v / max(sum(prof["ms"].values()), 1e-9) for k, v in prof["ms"].items()}
     own_launches = prof["kernels"]

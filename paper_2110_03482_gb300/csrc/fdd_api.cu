@@ -1544,7 +1544,7 @@ fdd_status fdd_tdd_execute(fdd_plan_t plan, const void* d_in, void* d_out, fdd_s
   fdd_status st = check_device(plan);
   if (st != FDD_OK) return st;
   const int nc = p.n_chan, nd = p.n_dm;
-  if (!plan->d_shift) {
+  if (plan->tdd_win == 0) {  // (set last: a call that failed half-way is taken up again)
     // Eq. 1 delays in samples (FP64), rounded to the nearest sample (halves
     // away from zero; delays are >= 0), and per block of kTdDms trials the
     // smallest shift of each channel and the widest span.
@@ -1601,12 +1601,14 @@ fdd_status fdd_tdd_execute(fdd_plan_t plan, const void* d_in, void* d_out, fdd_s
         }
       }
     const int64_t pitch = (p.n_t + 31) / 32 * 32;
-    if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift), sizeof(int) * rel.size())))
+    if (!plan->d_shift &&
+        (st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift), sizeof(int) * rel.size())))
       return st;
-    if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift_base),
-                        sizeof(int) * base.size())))
+    if (!plan->d_shift_base && (st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_shift_base),
+                                               sizeof(int) * base.size())))
       return st;
-    if ((st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_tdd_x),
+    if (!plan->d_tdd_x &&
+        (st = dev_alloc(plan, reinterpret_cast<void**>(&plan->d_tdd_x),
                         bytes ? static_cast<size_t>(nc) * pitch
                               : sizeof(float) * static_cast<size_t>(nc) * p.n_t)))
       return st;

@@ -44,3 +44,25 @@ def test_bytes_equal_floats(n_chan, n_t, ddm, n_dm, n_beams, layout):
             ys.append(y)
     assert torch.isfinite(ys[0]).all()
     assert torch.equal(ys[0], ys[1])
+
+
+@pytest.mark.parametrize("dtype", [fdd.FDD_IN_U8, fdd.FDD_IN_F32])
+@pytest.mark.parametrize("after", [0, 1, 2])
+def test_a_call_after_a_failed_allocation_starts_over(after, dtype):
+    x = torch.arange(1000 * 8, device="cuda") % 251
+    x = x.to(torch.uint8 if dtype == fdd.FDD_IN_U8 else torch.float32)
+    kw = dict(n_chan=8, nu_lo_mhz=1200.0, dnu_mhz=30.0, t_samp_s=1e-3, n_t=1000, in_dtype=dtype,
+              dm_list=3.0 * np.arange(9), output=fdd.FDD_OUT_TIME)
+    with fdd.Plan(**kw) as plan, fdd.Plan(**kw) as other:
+        y, ref = [torch.empty((9, 1000 - plan.info["d_max"]), device="cuda") for _ in range(2)]
+        fdd.fdd_debug_fail_alloc(after)
+        try:
+            with pytest.raises(fdd.FddError) as e:
+                plan.tdd_execute(x, y)
+            assert e.value.status == fdd.FDD_ERR_ALLOC
+        finally:
+            fdd.fdd_debug_fail_alloc(-1)
+        plan.tdd_execute(x, y)
+        other.tdd_execute(x, ref)
+        torch.cuda.synchronize()
+    assert torch.equal(y, ref)

@@ -6,8 +6,8 @@
 // wave the beams are unpacked and transformed one by one, whole or in their
 // own overlap-save chunks (one cuFFT plan per distinct transform length),
 // then ONE persistent launch of the FP32 phase-rotate-and-sum serves the
-// whole wave: its CTAs pull (beam, chunk, bin tile, trial block) items from a
-// counter.  The whole execute is captured once as a
+// whole wave (the G12 tile: one per form of its passes): its CTAs pull (beam,
+// chunk, bin tile, trial block) items from a counter.  The whole execute is captured once as a
 // CUDA graph and replayed.  At plan time an autotuner times the candidate
 // kernel tiles on the batch's real shapes and keeps the fastest.
 #include <cufft.h>
@@ -43,9 +43,17 @@ struct fdd_batch_s {
   std::vector<int64_t> L, n_bins, pitch, n_chunks, hop, in_off, out_off, spec_off;
   std::vector<int> wave_of;
   // per wave
+  // sets of a wave that go into one launch (the G12 tile: those whose trials
+  // take the same form of its passes; other tiles: all of them)
+  struct Group {
+    int first = 0, n_sets = 0;
+    long long n_items = 0;
+    int max_n_dm = 0;
+  };
   struct Wave {
     int first = 0, count = 0;  // beams
     long long n_items = 0;
+    std::vector<Group> groups;
     fdd::BatchSet* d_sets = nullptr;
     std::vector<fdd::BatchSet> h_sets;   // one per (beam, chunk)
     std::vector<int> set_beam, set_chunk;
@@ -57,7 +65,6 @@ struct fdd_batch_s {
   };
   std::vector<Wave> waves;
   int64_t in_elems = 0, out_elems = 0;
-  int max_n_dm = 0;  // largest trial count of the beams
   // device memory
   fdd::PhaseConst* d_pc = nullptr;  // [beam][n_chan]
   float* d_xw = nullptr;            // [n_chan][L_max]
@@ -206,6 +213,18 @@ fdd_status transform_chunk(fdd_batch_s* B, const void* beam_in, int b, int64_t c
   return FDD_OK;
 }
 
+// The main launches of a wave over its sets at d_sets.
+cudaError_t launch_groups(const fdd_batch_s* B, const fdd_batch_s::Wave& w,
+                          const fdd::BatchSet* d_sets, unsigned long long* counter,
+                          cudaStream_t s) {
+  for (const auto& g : w.groups) {
+    const cudaError_t e = fdd::launch_mac_batch(d_sets + g.first, g.n_sets, g.n_items, counter,
+                                                B->variant, B->ctas, B->p.n_chan, g.max_n_dm, s);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 // All work of one execute, issued on stream s (also used under capture).
 fdd_status issue(fdd_batch_s* B, const void* d_in, cudaStream_t s) {
   const size_t esz = B->p.in_dtype == FDD_IN_U8 ? 1 : 4;
@@ -221,12 +240,11 @@ fdd_status issue(fdd_batch_s* B, const void* d_in, cudaStream_t s) {
       }
     }
     B_CUDA(cudaMemsetAsync(B->d_counter + 2 * wi, 0, 2 * sizeof(unsigned long long), s));
-    B_CUDA(fdd::launch_mac_batch(w.d_sets, static_cast<int>(w.h_sets.size()), w.n_items,
-                                 B->d_counter + 2 * wi, B->variant, B->ctas, B->p.n_chan, B->max_n_dm, s));
+    B_CUDA(launch_groups(B, w, w.d_sets, B->d_counter + 2 * wi, s));
     if (w.n_tail_items)
       B_CUDA(fdd::launch_mac_batch(w.d_tail, static_cast<int>(w.h_tail.size()), w.n_tail_items,
                                    B->d_counter + 2 * wi + 1, B->tail_variant, B->tail_ctas,
-                                   B->p.n_chan, B->max_n_dm, s));
+                                   B->p.n_chan, 0, s));
   }
   return FDD_OK;
 }
@@ -614,7 +632,6 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
     in_acc += d.n_t * static_cast<int64_t>(p->n_chan);
     out_acc += g.n_chunks * g.n_bins * static_cast<int64_t>(d.n_dm);
     L_max = std::max(L_max, g.fft_len);
-    B->max_n_dm = std::max(B->max_n_dm, d.n_dm);
     fdd::CoreGeometry cg;
     if ((st = fdd::core_geometry(&q, &cg)) != FDD_OK) return st;
     for (int c = 0; c < p->n_chan; ++c)
@@ -733,15 +750,33 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
       wv.h_tail.clear();
       wv.tail_beam.clear();
       wv.tail_chunk.clear();
-      long long items = 0, t_items = 0;
-      for (int i = 0; i < wv.count; ++i) {
-        const int b = wv.first + i;
+      wv.groups.clear();
+      long long t_items = 0;
+      // The G12 tile's passes of up to 4096 trials cost 2.3 times those of up
+      // to 512 whatever their filling, so its beams are launched by the form
+      // that their trials take: six beams of 512 to 4096 trials x 1536 channels
+      // in four launches 9.6 ms, in one (of the widest form) 11.4.
+      std::vector<int> order(wv.count);
+      for (int i = 0; i < wv.count; ++i) order[i] = wv.first + i;
+      auto form = [&](int b) { return g12 ? fdd::mac_split_form(B->beams[b].n_dm) : 0; };
+      std::stable_sort(order.begin(), order.end(),
+                       [&](int x, int y) { return form(x) > form(y); });
+      int last_form = -1;
+      for (const int b : order) {
         const int n_dm = B->beams[b].n_dm;
+        if (form(b) != last_form) {
+          wv.groups.emplace_back();
+          wv.groups.back().first = static_cast<int>(wv.h_sets.size());
+          last_form = form(b);
+        }
+        fdd_batch_s::Group& group = wv.groups.back();
+        group.max_n_dm = std::max(group.max_n_dm, n_dm);
+        long long& items = group.n_items;
         const int full = n_dm / dms, rem = n_dm % dms;
         const bool tail = tails && rem > 0 && rem <= dms / 2;
         int blocks = full + (rem > 0 && !tail ? 1 : 0), tiles = 0;
         if (g12)
-          fdd::mac_split_batch_shape(B->max_n_dm, n_dm, B->n_bins[b], &tiles, &blocks);
+          fdd::mac_split_batch_shape(n_dm, B->n_bins[b], &tiles, &blocks);
         else
           tiles = static_cast<int>((B->n_bins[b] + bins_per_cta - 1) / bins_per_cta);
         for (int64_t c = 0; c < B->n_chunks[b]; ++c) {
@@ -754,6 +789,7 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
           bs.item_begin = items;
           items += static_cast<long long>(tiles) * blocks;
           wv.h_sets.push_back(bs);
+          ++group.n_sets;
           wv.set_beam.push_back(b);
           wv.set_chunk.push_back(static_cast<int>(c));
           if (tail) {
@@ -772,7 +808,8 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
           }
         }
       }
-      wv.n_items = items;
+      wv.n_items = 0;
+      for (const auto& g : wv.groups) wv.n_items += g.n_items;
       wv.n_tail_items = t_items;
     }
     return FDD_OK;
@@ -846,13 +883,13 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
       // the persistent grid rank the tiles whatever the wave's size), scaled
       // to the whole wave: main launch plus, for a tile with one, tail launch.
       auto timed = [&](fdd::BatchSet* sets, int n_sets, long long n_items, int tile, int ctas,
-                       unsigned long long* counter) -> double {
+                       unsigned long long* counter, int max_n_dm) -> double {
         const long long part = std::min<long long>(n_items, 8LL * ctas);
         float ms = 0.f;
         for (int rep = 0; rep < 2; ++rep) {  // the first launch is a warm-up
           cudaMemset(counter, 0, sizeof(unsigned long long));
           cudaEventRecord(e0);
-          fdd::launch_mac_batch(sets, n_sets, part, counter, tile, ctas, p->n_chan, B->max_n_dm,
+          fdd::launch_mac_batch(sets, n_sets, part, counter, tile, ctas, p->n_chan, max_n_dm,
                                 nullptr);
           cudaEventRecord(e1);
           cudaEventSynchronize(e1);
@@ -860,11 +897,13 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
         }
         return static_cast<double>(ms) * static_cast<double>(n_items) / static_cast<double>(part);
       };
-      double tot = timed(w0.d_sets, static_cast<int>(w0.h_sets.size()), w0.n_items, v, B->ctas,
-                         B->d_counter);
+      double tot = 0.0;
+      for (const auto& g : w0.groups)
+        tot += timed(w0.d_sets + g.first, g.n_sets, g.n_items, v, B->ctas, B->d_counter,
+                     g.max_n_dm);
       if (w0.n_tail_items)
         tot += timed(w0.d_tail, static_cast<int>(w0.h_tail.size()), w0.n_tail_items,
-                     B->tail_variant, B->tail_ctas, B->d_counter + 1);
+                     B->tail_variant, B->tail_ctas, B->d_counter + 1, 0);
       if (cudaGetLastError() != cudaSuccess) {
         tst = report_error(FDD_ERR_CUDA, "autotune launch failed");
         break;
@@ -1064,12 +1103,11 @@ fdd_status fdd_batch_execute_stream(fdd_batch_t b, fdd_source_fn source, void* s
     fdd::BatchSet* d_sets = b->d_sets_slot[k][wi];
     B_CUDA(cudaMemsetAsync(b->d_counter + 2 * wi, 0, 2 * sizeof(unsigned long long), s));
     const int n_sets = static_cast<int>(w.h_sets.size());
-    B_CUDA(fdd::launch_mac_batch(d_sets, n_sets, w.n_items, b->d_counter + 2 * wi, b->variant,
-                                 b->ctas, b->p.n_chan, b->max_n_dm, s));
+    B_CUDA(launch_groups(b, w, d_sets, b->d_counter + 2 * wi, s));
     if (w.n_tail_items)
       B_CUDA(fdd::launch_mac_batch(d_sets + n_sets, static_cast<int>(w.h_tail.size()),
                                    w.n_tail_items, b->d_counter + 2 * wi + 1, b->tail_variant,
-                                   b->tail_ctas, b->p.n_chan, b->max_n_dm, s));
+                                   b->tail_ctas, b->p.n_chan, 0, s));
     const int64_t origin = b->out_off[w.first];
     void* release = nullptr;
     for (int i = 0; i < w.count; ++i) {

@@ -89,8 +89,8 @@ cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s);
 size_t mac_smem_bytes(int variant, int n_chan);
 
 // The G12_4X8 tile (fdd_mac_split.cu): split-FP16 operands on the tensor
-// cores.  Batches are shaped by their largest trial count (the trials a pass
-// can hold and the bins a CTA works on together follow from it):
+// cores.  A batch's sets go into one launch by the form of their passes
+// (mac_split_form of their trials; max_n_dm: any of the launch's);
 // mac_split_batch_shape gives a set's bin groups and passes, whose product
 // numbers its items pass-major; the persistent launch deals them out in turn.
 size_t mac_split_smem_bytes();
@@ -98,7 +98,8 @@ cudaError_t mac_split_prepare();
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s);
 // whether the series of one launch share passes at this trial count
 bool mac_split_series_share(int n_dm);
-void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes);
+int mac_split_form(int n_dm);
+void mac_split_batch_shape(int n_dm, long long n_bins, int* bin_groups, int* passes);
 cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
                                    int max_n_dm, int n_ctas, cudaStream_t s);
 

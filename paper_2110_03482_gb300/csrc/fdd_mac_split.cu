@@ -1058,8 +1058,10 @@ cudaError_t mac_split_prepare() {
 
 bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2, n_dm)).sets > 1; }
 
-void mac_split_batch_shape(int max_n_dm, int n_dm, long long n_bins, int* bin_groups, int* passes) {
-  const FormInfo f = form_info(form_for(max_n_dm, 1, max_n_dm));
+int mac_split_form(int n_dm) { return form_for(n_dm, 1, n_dm); }
+
+void mac_split_batch_shape(int n_dm, long long n_bins, int* bin_groups, int* passes) {
+  const FormInfo f = form_info(form_for(n_dm, 1, n_dm));
   *bin_groups = static_cast<int>((n_bins + f.bins - 1) / f.bins);
   *passes = (n_dm + f.pass_trials - 1) / f.pass_trials;
 }

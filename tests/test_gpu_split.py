@@ -169,3 +169,25 @@ def test_plans_that_take_two_at_a_time_give_the_same_bits(n_beams, n_t, chunk_le
             limit = fdd.fdd_plan_geometry(fdd.Params(**kw))["workspace_bytes"] - 1
     assert held[1] < held[0]
     assert torch.equal(outs[0], outs[1])
+
+
+def test_batch_beams_have_the_bits_of_their_own_plans():
+    """Beams of one batch are launched by the form of their trial counts (up to
+    512, 1024, 2048, more): each equals a plan of its own."""
+    counts = [300, 4096, 512, 513, 2049, 1024, 1025, 700, 2048, 1]
+    kw = dict(n_chan=40, nu_lo_mhz=1200.0, dnu_mhz=7.5, t_samp_s=1e-3, in_dtype=fdd.FDD_IN_F32,
+              output=fdd.FDD_OUT_SPECTRA, chunk_len=0, mac_variant=1 + fdd.FDD_MAC_G12_4X8)
+    n_t = [2048 if i % 2 else 1024 for i in range(len(counts))]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    xs = [torch.randn(n * 40, generator=g, device="cuda") for n in n_t]
+    with fdd.Batch([(t, 1.0, 0.02, d) for t, d in zip(n_t, counts)], autotune=False, **kw) as batch:
+        out = torch.full((batch.info["out_elems"], 2), 7.0, device="cuda")
+        batch.execute(torch.cat(xs), out)
+        torch.cuda.synchronize()
+        for i, d in enumerate(counts):
+            with fdd.Plan(n_t=n_t[i], dm_list=1.0 + 0.02 * np.arange(d), **kw) as plan:
+                one = torch.full((plan.info["out_elems"], 2), 9.0, device="cuda")
+                plan.execute(xs[i], one)
+                torch.cuda.synchronize()
+            at = batch.out_offsets[i]
+            assert torch.equal(out[at:at + one.shape[0]], one), i

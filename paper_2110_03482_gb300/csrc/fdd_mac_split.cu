@@ -98,10 +98,11 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 constexpr int kCh = 64;     // channels per stage (four K steps of 16)
 constexpr int kRows = 128;  // Cb, Sb of 64 b's: sixteen b's Cb, then their Sb, and so on
 // Up to this many channels the columns' phasors come from the Taylor series,
-// too (2.1e-7 to 2.4e-7 of the result instead of 3.2e-7): over so few the
-// FP32 multiply-adds' sums lost little, and reached 3.0e-7.  A call of 63
-// channels x 277 trials x 347 bins takes 13 us either way.
-constexpr int kFewChan = 128;
+// too: over so few the FP32 multiply-adds' sums lost little (3.9e-7 of the
+// spectra, 5.1e-7 of the power at 167 channels; this product 3.4e-7 and 5.2e-7
+// with the hardware's columns, 2.5e-7 and 3.7e-7 with these).  167 channels x 911
+// trials x 1829 bins take 39.0 us, 37.3 with the hardware's, 80 before.
+constexpr int kFewChan = 256;
 constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's (twin: half)
 constexpr int kBlockAls = 8;      // al's of a whole block (2048 trials)
 

@@ -721,8 +721,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       q += kPrepWarps;
     };
+    // (Past the CTA's last stage the loads repeat addresses of its last item; a
+    // warp without a first stage has no item to load from.)
     Fetched next;
-    fetch(next);
+    if (p < total) fetch(next);
     for (uint32_t n = p; n < total; n += kPrepWarps) {
       const uint32_t s = n % T;
       const uint4 pc[2] = {next.pc[0], next.pc[1]};

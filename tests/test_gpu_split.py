@@ -191,3 +191,25 @@ def test_batch_beams_have_the_bits_of_their_own_plans():
                 torch.cuda.synchronize()
             at = batch.out_offsets[i]
             assert torch.equal(out[at:at + one.shape[0]], one), i
+
+
+@pytest.mark.parametrize("n_chan", [1, 16, 63, 64])
+@pytest.mark.parametrize("n_dm,n_series", [(3000, 1), (700, 4), (700, 6), (2000, 2), (2000, 3)])
+def test_one_stage_items_match_oracle(n_chan, n_dm, n_series):
+    """Up to 64 channels and one bin at a time, an item is one stage; with
+    fewer items than CTAs the second of the two warps that make the stages'
+    tables has none, and the loads that it starts ahead must be real ones."""
+    L, dms = 1 << 12, 3.7 + 0.31 * np.arange(n_dm)
+    b0, nb = 1021, 3
+    rng = np.random.default_rng(n_chan + n_dm + n_series)
+    X = (rng.standard_normal((n_series, n_chan, nb)) +
+         1j * rng.standard_normal((n_series, n_chan, nb))).astype(np.complex64)
+    with _plan(n_chan, L, dms) as plan:
+        dX = complex_to_device(X, nb)
+        dY = torch.full((n_series, n_dm, nb, 2), 7.0, device="cuda")
+        plan.dedisperse_spectra_bins(dX, nb, n_series, b0, nb, 0, n_dm, dY, nb)
+        torch.cuda.synchronize()
+        plan.query()
+    for s in range(n_series):
+        ref = _reference(X[s].astype(np.complex128), np.arange(b0, b0 + nb), L, n_chan, dms)
+        assert rel_l2(device_to_complex(dY, nb)[s], ref) <= TOL, s

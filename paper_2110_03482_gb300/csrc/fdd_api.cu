@@ -1108,6 +1108,20 @@ long long launches_so_far() { return g_launches.load(std::memory_order_relaxed);
 // fdd_debug_fail_alloc: allocations to let through before one fails (-1: none).
 std::atomic<int> g_fail_alloc{-1};
 
+cudaError_t allow_smem(const void* fn, size_t bytes) {
+  cudaFuncAttributes at;
+  int dev = 0, per_block = 0;
+  cudaError_t e = cudaFuncGetAttributes(&at, fn);
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&per_block, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e != cudaSuccess) return e;
+  const int most = per_block - static_cast<int>(at.sharedSizeBytes);
+  if (static_cast<long long>(bytes) > most) return cudaErrorInvalidValue;
+  if (at.maxDynamicSharedSizeBytes >= most) return cudaSuccess;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 bool injected_alloc_failure() {
   int k = g_fail_alloc.load();
   while (k >= 0)

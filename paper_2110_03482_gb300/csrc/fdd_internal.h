@@ -224,6 +224,13 @@ cudaError_t launch_mac_spin(const MacArgs& a, const SpinGeometry& sg, const Phas
 // allocation is to fail; every library allocator asks before cudaMalloc.
 bool injected_alloc_failure();
 
+// Lets launches of the kernel `fn` on the current device take up to `bytes` of
+// dynamic shared memory a block.  CUDA keeps one limit per kernel and device,
+// the last one set: it is raised to the most that the kernel can have, not to
+// `bytes`, so that plans of any sizes made in any order (or by any threads)
+// can run side by side.  cudaErrorInvalidValue where no block can have `bytes`.
+cudaError_t allow_smem(const void* fn, size_t bytes);
+
 // Kernels this library has launched (process wide): every launch wrapper
 // adds to it; the profiling calls report the count over a profiled region.
 void note_launches(int n);

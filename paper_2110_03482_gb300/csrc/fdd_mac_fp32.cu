@@ -790,14 +790,12 @@ size_t mac_smem_bytes(int variant, int n_chan) {
 cudaError_t mac_prepare(int variant, int n_chan) {
   if (variant == MAC_G12_4x8) return mac_split_prepare();
   const VariantInfo vi = variant_info(variant);
-  const int bytes = static_cast<int>(mac_smem_bytes(variant, n_chan));
-  cudaError_t e = cudaFuncSetAttribute(vi.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const size_t bytes = mac_smem_bytes(variant, n_chan);
+  cudaError_t e = allow_smem(vi.fn, bytes);
   if (e == cudaSuccess && variant == MAC_Q_4x4 && SplitQ::smem(n_chan) <= kMaxSmem)
-    e = cudaFuncSetAttribute(reinterpret_cast<const void*>(&mac_parts_kernel),
-                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(SplitQ::smem(n_chan)));
+    e = allow_smem(reinterpret_cast<const void*>(&mac_parts_kernel), SplitQ::smem(n_chan));
   if (e != cudaSuccess || !vi.batch_fn) return e;
-  return cudaFuncSetAttribute(vi.batch_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return allow_smem(vi.batch_fn, bytes);
 }
 
 int mac_variant_bins_per_cta(int variant) { return variant_info(variant).bins(); }

@@ -269,8 +269,7 @@ size_t tdd_smem_bytes(int win) {
 }
 
 cudaError_t tdd_prepare(int win) {
-  return cudaFuncSetAttribute(tdd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(tdd_smem_bytes(win)));
+  return allow_smem(reinterpret_cast<const void*>(&tdd_kernel), tdd_smem_bytes(win));
 }
 
 cudaError_t launch_tdd(const TddArgs& a, cudaStream_t s) {
@@ -289,8 +288,7 @@ size_t tdd8_smem_bytes(int win) {
 }
 
 cudaError_t tdd8_prepare(int win) {
-  return cudaFuncSetAttribute(tdd8_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(tdd8_smem_bytes(win)));
+  return allow_smem(reinterpret_cast<const void*>(&tdd8_kernel), tdd8_smem_bytes(win));
 }
 
 cudaError_t launch_tdd8(const Tdd8Args& a, cudaStream_t s) {

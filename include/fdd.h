@@ -420,7 +420,8 @@ fdd_status fdd_tdd_execute(fdd_plan_t plan, const void* d_in, void* d_out, fdd_s
  * status word, releases what it holds and returns.
  *
  * fdd_debug_stall_test runs the plan's waiting phase-rotate-and-sum kernel
- * (the warp-specialised FP32 tile, or the tensor-core kernel) on one bin,
+ * (the G12_4X8 tile, the tensor-core kernel, or W12_8X8 for FP32 plans of the
+ * other tiles, of which it alone waits) on one bin,
  * one trial and one series, with its producers withholding every "stage
  * filled" arrival, so the consumers' waits run out.  It blocks until the
  * kernel has returned (about 2 s); the next fdd_query then reports

@@ -1365,6 +1365,8 @@ fdd_status fdd_debug_stall_test(fdd_plan_t plan, fdd_stream_t stream) {
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // One bin, one trial, one series: a single CTA whose producers withhold
   // every arrival; the plan's spectra buffer serves as (unread-for-value) X.
+  // FP32 plans whose own tile has no waits run the W12 tile.
+  const bool g12 = !plan->tc && plan->info.mac_variant == FDD_MAC_G12_4X8;
   void* y = nullptr;
   FDD_CUDA(cudaMalloc(&y, 64));
   fdd::MacArgs m{};
@@ -1386,14 +1388,16 @@ fdd_status fdd_debug_stall_test(fdd_plan_t plan, fdd_stream_t stream) {
   m.real_bin_a = -1;
   m.real_bin_b = -1;
   m.status = plan->d_status;
+  m.of_n_dm = plan->p.n_dm;
   m.test_withhold = 1;
   cudaError_t e;
   if (plan->tc) {
     e = fdd::launch_mac_tc(m, plan->p.precision, plan->n_sms, plan->d_tcx,
                            plan->tcx_bytes, s);
   } else {
-    e = fdd::mac_prepare(fdd::MAC_W12_8x8, plan->p.n_chan);
-    if (e == cudaSuccess) e = fdd::launch_mac_fp32(m, fdd::MAC_W12_8x8, s);
+    const int tile = g12 ? fdd::MAC_G12_4x8 : fdd::MAC_W12_8x8;
+    e = fdd::mac_prepare(tile, plan->p.n_chan);
+    if (e == cudaSuccess) e = fdd::launch_mac_fp32(m, tile, s);
   }
   const cudaError_t es = cudaStreamSynchronize(s);
   cudaFree(y);

@@ -952,7 +952,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&sm.full[s]);
+        if (!a.test_withhold) mbar_arrive(&sm.full[s]);  // (never set for a batch)
         mbar_arrive(&sm.pfree[ts]);
       }
     }

@@ -107,3 +107,33 @@ def test_injected_allocation_failures_leak_nothing():
         plan.execute_host(h_in, h_out)  # the next call allocates and runs
         torch.cuda.synchronize()
         assert np.isfinite(h_out.numpy()).all()
+
+
+@pytest.mark.parametrize("n_chan,n_dm", [(64, 300), (200, 3000), (8300, 700)])
+def test_stalled_g12_tile_times_out_and_the_plan_recovers(n_chan, n_dm):
+    """The tile that FP32 plans take from 257 trials, in both its forms for one
+    trial (two bins a stage in plans of up to 512), with fewer stages than its
+    ring and more; 8300 channels are beyond the tile that other FP32 plans
+    stall.  Tensor memory is given back: the plan then runs on every SM."""
+    nu, dms, n_t = oracle.channel_centres(n_chan, 1200.0, 300.0 / n_chan), 0.01 * np.arange(n_dm), 2048
+    fb = np.random.default_rng(n_chan).standard_normal((n_t, n_chan)).astype(np.float32)
+    with fdd.Plan(n_chan=n_chan, nu_lo_mhz=1200.0, dnu_mhz=300.0 / n_chan, t_samp_s=1e-3, n_t=n_t,
+                  dm_list=dms, in_dtype=fdd.FDD_IN_F32, output=fdd.FDD_OUT_SPECTRA) as plan:
+        assert plan.info["mac_variant"] == fdd.FDD_MAC_G12_4X8
+        t0 = time.perf_counter()
+        plan.debug_stall_test()
+        dt = time.perf_counter() - t0
+        assert 0.5 < dt < 60.0, dt
+        with pytest.raises(fdd.FddError) as e:
+            plan.query()
+        assert e.value.status == fdd.FDD_ERR_TIMEOUT
+        plan.query()  # reported once
+        out = torch.full((n_dm, n_t // 2 + 1, 2), 7.0, device="cuda")
+        plan.execute(torch.from_numpy(fb).cuda(), out)
+        torch.cuda.synchronize()
+        plan.query()
+    bins = np.array([0, 1, 511, n_t // 2])
+    ref = oracle.fdd_bins(np.fft.rfft(fb.astype(np.float64), axis=0).T[:, bins], bins, n_t,
+                          oracle.delays(nu, dms, 1e-3))
+    got = out.cpu().numpy().astype(np.float64)[:, bins]
+    assert rel_l2(got[..., 0] + 1j * got[..., 1], ref) <= FP32_REL_L2

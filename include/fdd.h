@@ -142,7 +142,13 @@ typedef struct fdd_params {
   int32_t precision;      /* FDD_PREC_*                                              */
   int32_t mac_variant;    /* phase-rotate-and-sum kernel: 0 chooses automatically;
                              1 + FDD_MAC_* forces that variant                      */
-  size_t workspace_limit; /* device bytes the plan may hold; 0 = library default    */
+  size_t workspace_limit; /* device bytes the plan may hold; 0 = library default
+                             (16 GiB).  Plans of the G12_4X8 tile with 513 to
+                             2048 trials and two or more beams or chunks hold a
+                             second one's spectra (and dedispersed spectra, for
+                             time output) where they fit: fdd_execute then takes
+                             two through a launch; a limit just below
+                             fdd_plan_geometry's workspace_bytes leaves them out */
   int32_t downsample;     /* FDD_OUT_TIME: shorten the inverse transform by this
                              power-of-two factor f (0 or 1: none; Sect. 2.2, last
                              paragraph): only the bins k <= L/(2f) are dedispersed
@@ -430,8 +436,9 @@ fdd_status fdd_tdd_execute(fdd_plan_t plan, const void* d_in, void* d_out, fdd_s
  *
  * fdd_debug_fail_alloc makes the library's device allocations after the
  * next `after` ones fail once with FDD_ERR_ALLOC (plans and batch plans
- * release what they hold and report it); after < 0 turns it off.  Process
- * wide.  Always FDD_OK.
+ * release what they hold and report it; the second spectra of a plan that
+ * could take two beams or chunks at a time are left out instead, and it takes
+ * them one by one); after < 0 turns it off.  Process wide.  Always FDD_OK.
  */
 fdd_status fdd_debug_stall_test(fdd_plan_t plan, fdd_stream_t stream);
 fdd_status fdd_debug_fail_alloc(int32_t after);

@@ -818,11 +818,16 @@ fdd_status run(fdd_plan_s* P, const Io& io, cudaStream_t s) {
     auto chunk = [&](int i) { return (u + i) % g.n_chunks; };
     float2* const X[2] = {P->d_X, P->d_X2};
     float2* const Y[2] = {P->d_Y, P->d_Y2};
+    // elements from one allocation to another (both aligned to 256 bytes)
+    auto apart = [](const float2* from, const float2* to) {
+      return (reinterpret_cast<intptr_t>(to) - reinterpret_cast<intptr_t>(from)) /
+             static_cast<intptr_t>(sizeof(float2));
+    };
     for (int i = 0; i < n_u; ++i)
       if ((st = transform(P, io, beam(i), chunk(i), X[i], s)) != FDD_OK) return st;
     fdd::MacArgs m{};
     m.X = X[0];
-    m.x_series_stride = n_u == 2 ? X[1] - X[0] : 0;
+    m.x_series_stride = n_u == 2 ? apart(X[0], X[1]) : 0;
     m.x_chan_stride = g.bin_pitch;
     m.pc = P->d_pc;
     m.n_chan = p.n_chan;
@@ -840,7 +845,7 @@ fdd_status run(fdd_plan_s* P, const Io& io, cudaStream_t s) {
         m.j_begin = j0;
         m.n_dm = nb;
         m.Y = Y[0];
-        m.y_series_stride = n_u == 2 ? Y[1] - Y[0] : 0;
+        m.y_series_stride = n_u == 2 ? apart(Y[0], Y[1]) : 0;
         m.y_dm_stride = g.bin_pitch;
         m.out_kind = 1;
         m.real_bin_a = 0;                           // DC and Nyquist of a real
@@ -1315,17 +1320,13 @@ fdd_status plan_create(const fdd_params* p, void* arena, size_t arena_bytes, fdd
     if (P->has_c2r_tail) FDD_CUFFT(cufftSetWorkArea(P->c2r_tail, P->d_fftwork));
   }
   if (pair_bytes > 0 && !P->arena) {
-    // (the plan runs one by one where the device has no room for two)
+    // (not an error where the device has no room for two: the plan runs one by one)
     const size_t x = sizeof(float2) * size_t(nc) * g.bin_pitch;
-    void* two[2] = {};
-    if (cudaMalloc(&two[0], x) != cudaSuccess ||
-        (pair_bytes > x && cudaMalloc(&two[1], pair_bytes - x) != cudaSuccess)) {
-      cudaGetLastError();
-      if (two[0]) cudaFree(two[0]);
-    } else {
-      P->d_X2 = static_cast<float2*>(two[0]);
-      P->d_Y2 = static_cast<float2*>(two[1]);
-      P->bytes_held += pair_bytes;
+    if (dev_alloc(P, reinterpret_cast<void**>(&P->d_X2), x) == FDD_OK && pair_bytes > x &&
+        dev_alloc(P, reinterpret_cast<void**>(&P->d_Y2), pair_bytes - x) != FDD_OK) {
+      cudaFree(P->d_X2);
+      P->d_X2 = nullptr;
+      P->bytes_held -= x;
     }
   }
   g.workspace_bytes = static_cast<int64_t>(P->bytes_held);

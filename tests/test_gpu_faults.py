@@ -137,3 +137,38 @@ def test_stalled_g12_tile_times_out_and_the_plan_recovers(n_chan, n_dm):
                           oracle.delays(nu, dms, 1e-3))
     got = out.cpu().numpy().astype(np.float64)[:, bins]
     assert rel_l2(got[..., 0] + 1j * got[..., 1], ref) <= FP32_REL_L2
+
+
+@pytest.mark.parametrize("output,optional", [(fdd.FDD_OUT_TIME, 2), (fdd.FDD_OUT_POWER, 1)])
+def test_plans_without_room_for_two_at_a_time_run_one_by_one(output, optional):
+    """The second (beam, chunk)'s buffers are the only allocations whose failure
+    leaves a working plan: it holds less and gives the same bytes."""
+    kw = dict(n_chan=40, nu_lo_mhz=1200.0, dnu_mhz=7.5, t_samp_s=1e-3, n_t=9000, chunk_len=1 << 12,
+              in_dtype=fdd.FDD_IN_F32, dm_list=1.0 + 0.05 * np.arange(600), output=output)
+    x = torch.randn(9000 * 40, generator=torch.Generator(device="cuda").manual_seed(3), device="cuda")
+
+    def run(plan):
+        out = torch.full((plan.info["out_elems"],), 7.0, device="cuda")
+        plan.execute(x, out)
+        torch.cuda.synchronize()
+        plan.query()
+        return out
+
+    with fdd.Plan(**kw) as plan:
+        held, expected = plan.info["workspace_bytes"], run(plan)
+    free0 = torch.cuda.mem_get_info()[0]
+    failed = one_by_one = 0
+    for after in range(20):
+        fdd.fdd_debug_fail_alloc(after)
+        try:
+            with fdd.Plan(**kw) as plan:
+                fdd.fdd_debug_fail_alloc(-1)
+                assert torch.equal(run(plan), expected)
+                one_by_one += plan.info["workspace_bytes"] < held
+        except fdd.FddError as e:
+            assert e.status == fdd.FDD_ERR_ALLOC
+            failed += 1
+        finally:
+            fdd.fdd_debug_fail_alloc(-1)
+    assert failed >= 4 and one_by_one == optional
+    assert abs(torch.cuda.mem_get_info()[0] - free0) < (64 << 20)

@@ -913,6 +913,7 @@ fdd_status run_spin(fdd_plan_s* P, const Io& io, cudaStream_t s) {
     m.pc = P->d_pc;
     m.n_chan = p.n_chan;
     m.n_series = 1;
+    m.of_n_dm = p.n_dm;
     m.status = P->d_status;
     m.scale = 1.0f;
     if (p.output == FDD_OUT_TIME) {

@@ -110,3 +110,24 @@ def test_spin_rejects_what_it_does_not_run():
         with pytest.raises(fdd.FddError) as e:
             fdd.Plan(**params_for(w, **kw))
         assert e.value.status == status
+
+
+@pytest.mark.parametrize("n_dm", [64, 300, 512, 700])
+def test_bins_below_the_first_group_have_the_bits_of_an_fp32_plan(n_dm):
+    """Whole path: the bins that follow Eq. 7 exactly run the FP32 plan's own
+    kernel and form (two bins a stage in plans of 257 to 512 trials)."""
+    w = _workload(40, 4096, 0.0, 0.1, n_dm)
+    K = 2049
+    fb, _ = synth.filterbank(w, seed=4)
+    d_in = torch.from_numpy(fb).cuda()
+    outs = []
+    for kw in (dict(), dict(precision=fdd.FDD_PREC_FP16, spin_group=16, spin_tol=0.02)):
+        with fdd.Plan(**params_for(w, **kw)) as plan:
+            k_min = plan.info["spin_k_min"]
+            out = torch.full((n_dm, K, 2), 7.0, device="cuda")
+            plan.execute(d_in, out)
+            torch.cuda.synchronize()
+            plan.query()
+            outs.append(out)
+    assert k_min == 750
+    assert torch.equal(outs[0][:, :k_min], outs[1][:, :k_min])

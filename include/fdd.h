@@ -90,7 +90,9 @@ typedef enum fdd_status {
                                matrix product (half the multiplications and
                                phasors of the complex form); hi + lo FP16 operands,
                                three products, FP32 sums; passes of up to 4096
-                               trials (default from 257 trials)                 */
+                               trials (default from 257 trials).  A sample that
+                               is infinite or NaN leaves no finite trial in its
+                               bin, and the other bins as they are              */
 #define FDD_MAC_VARIANTS 6
 #define FDD_MAC_TC 100      /* fdd_info.mac_variant of the tensor-core form: one
                                CTA per SM, a pass over the channels covering

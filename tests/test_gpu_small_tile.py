@@ -65,3 +65,36 @@ def test_edges_match_oracle(n_chan, n_dm, n_series):
     for s in range(n_series):
         ref = oracle.fdd_bins(X[s].astype(np.complex128), np.arange(b0, b0 + nb), L, d)
         assert rel_l2(Y[s], ref) <= TOL, s
+
+
+@pytest.mark.parametrize("n_chan,n_dm,tol", [
+    (128, 5, TOL), (129, 130, TOL), (160, 128, TOL), (161, 40, TOL), (300, 129, TOL),
+    (1024, 256, TOL), (11200, 33, 5e-6), (11201, 33, 5e-6),
+])
+def test_long_parts_match_oracle(n_chan, n_dm, tol):
+    """A part of more than 32 channels goes round the ring of X; 11200 channels
+    are the most whose phase table fits beside the swap areas, above them one
+    warp takes a bin's channels.  Sums of n terms round to 2^-25 sqrt(n / 2) of
+    the result: 3.4e-7 for a quarter of 1024 channels, 1.1e-6 for one of 11200,
+    2.2e-6 for 11201 in one sum, beside the phasors' 2.4e-7."""
+    L, dms = 1 << 12, 3.7 + 0.31 * np.arange(n_dm)
+    dnu = (BAND[1] - BAND[0]) / n_chan
+    nu = oracle.channel_centres(n_chan, BAND[0] + 0.5 * dnu, dnu)
+    rng = np.random.default_rng(n_chan)
+    b0, nb = 700, 13
+    X = (rng.standard_normal((2, n_chan, nb)) +
+         1j * rng.standard_normal((2, n_chan, nb))).astype(np.complex64)
+    with fdd.Plan(n_chan=n_chan, nu_lo_mhz=BAND[0] + 0.5 * dnu, dnu_mhz=dnu, t_samp_s=2e-3, n_t=L,
+                  dm_list=dms, in_dtype=fdd.FDD_IN_F32, output=fdd.FDD_OUT_SPECTRA) as plan:
+        assert plan.info["mac_variant"] == fdd.FDD_MAC_Q_4X4
+        dX = complex_to_device(X, nb + 2)
+        dY = torch.full((2, n_dm, nb + 1, 2), 7.0, device="cuda")
+        plan.dedisperse_spectra_bins(dX, nb + 2, 2, b0, nb, 0, n_dm, dY, nb + 1)
+        torch.cuda.synchronize()
+        plan.query()
+    assert torch.all(dY[:, :, nb:] == 7.0)
+    Y = device_to_complex(dY, nb)
+    d = oracle.delays(nu, dms, 2e-3)
+    for s in range(2):
+        ref = oracle.fdd_bins(X[s].astype(np.complex128), np.arange(b0, b0 + nb), L, d)
+        assert rel_l2(Y[s], ref) <= tol, s

@@ -213,3 +213,26 @@ def test_one_stage_items_match_oracle(n_chan, n_dm, n_series):
     for s in range(n_series):
         ref = _reference(X[s].astype(np.complex128), np.arange(b0, b0 + nb), L, n_chan, dms)
         assert rel_l2(device_to_complex(dY, nb)[s], ref) <= TOL, s
+
+
+@pytest.mark.parametrize("n_dm", [300, 700, 2048, 3000])
+def test_infinite_samples_stay_in_their_bin(n_dm):
+    """An infinity takes every trial of its own bin and series (not a finite
+    value anywhere: the split makes NaN of it) and none of another's."""
+    n_chan, nb, n_series, b0 = 70, 9, 2, 333
+    X = torch.randn((n_series, n_chan, nb, 2), device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(n_dm))
+    with _plan(n_chan, 1 << 12, 0.5 * np.arange(n_dm)) as plan:
+        clean, dY = (torch.empty((n_series, n_dm, nb, 2), device="cuda") for _ in range(2))
+        plan.dedisperse_spectra_bins(X, nb, n_series, b0, nb, 0, n_dm, clean, nb)
+        X[0, 3, 1, 0], X[1, 69, 6, 1] = float("inf"), -float("inf")
+        plan.dedisperse_spectra_bins(X, nb, n_series, b0, nb, 0, n_dm, dY, nb)
+        dP = torch.empty((n_series, n_dm, nb), device="cuda")
+        plan.dedisperse_spectra_bins(X, nb, n_series, b0, nb, 0, n_dm, dP, nb, fdd.FDD_OUT_POWER)
+        torch.cuda.synchronize()
+        plan.query()
+    hit = torch.zeros((n_series, nb), dtype=torch.bool, device="cuda")
+    hit[0, 1] = hit[1, 6] = True
+    hit = hit[:, None].expand(n_series, n_dm, nb)
+    assert not torch.any(torch.isfinite(dY[hit])) and not torch.any(torch.isfinite(dP[hit]))
+    assert torch.equal(dY[~hit], clean[~hit])

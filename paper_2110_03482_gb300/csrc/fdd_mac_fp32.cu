@@ -293,15 +293,17 @@ __global__ void __launch_bounds__(W * 32, 1) mac_kernel(const MacArgs a) {
 // for its own results five cycles of six.  So kParts warps share the bins, each
 // with a part of the channels, and add their sums up at the end; a warp
 // evaluates a group of kGroup channels while it accumulates the group before;
-// and X arrives kXAhead batches of eight channels early.  Groups of two keep
-// the swap areas small enough for three CTAs an SM.  The split depends on
+// and X and the phase constants arrive kXAhead batches of eight channels early.
+// Groups of two, and no table of all channels' constants, keep a CTA's shared
+// memory small enough for three CTAs an SM whatever the channels.  The split depends on
 // nothing but the channels, so calls on parts of the bins or trials agree
-// bit for bit.  Against a warp taking all the channels one by one: 64 channels
-// x 128 trials x 2049 bins 21.2 -> 10.6 us a call (8 of which the host takes),
-// 1024 channels x 250 trials x 500 bins 279 -> 76, x 186 trials x 4096 bins
-// 393 -> 301, 100 channels x 128 trials x 9000 bins 44.8 -> 44.7.  (Groups of four, two
-// CTAs an SM: 10.7, 76, 340 and 50 us; evaluating ahead alone, without the
-// split: 18.7, 217, 492, 43.)
+// bit for bit.  Against a warp taking all the channels one by one (table in
+// shared memory): 64 channels x 128 trials x 500 bins 21.5 -> 8.2 us a call (the
+// host's time), x 4096 bins 22.6 -> 16.4, 1024 channels x 256 trials x 500 bins
+// 277 -> 60, x 200 trials x 4096 bins 391 -> 281, 4096 channels x 200 trials x
+// 4096 bins 1543 -> 1099.  (With the table beside the swap areas, one CTA an SM
+// of 4096 channels: 17.4, 74, 299, 1964.  Groups of four, two CTAs an SM, or
+// evaluating ahead without the split were slower, too.)
 constexpr int kParts = 4, kBinSets = 2;  // warps per four bins; fours of bins per CTA
 constexpr int kGroup = 2, kXAhead = 4;
 struct SplitQ {
@@ -310,13 +312,13 @@ struct SplitQ {
   static constexpr int kWarpsOf = kParts * kBinSets;
   static constexpr int kStage = Gm::NG * M::GFL;            // floats of a channel
   static constexpr int kSwap = 2 * kGroup * kStage;         // of a warp's two swap areas
-  static constexpr int kRing = 2 * 32 * kXAhead;            // and its X ring
+  static constexpr int kRing = 2 * 32 * kXAhead;            // its ring of X
+  static constexpr int kConsts = 4 * 8 * kXAhead;           // and of phase constants
+  static constexpr int kWarpFloats = kSwap + kRing + kConsts;
   static constexpr int kSums = 2 * Gm::AT * Gm::BT * 32;    // the sums, over the swap areas
   static_assert(kSums <= kSwap, "sums fit the swap areas");
-  static size_t smem(int n_chan) {
-    return sizeof(PhaseConst) * static_cast<size_t>(n_chan) +
-           sizeof(float) * static_cast<size_t>(kWarpsOf) * (kSwap + kRing);
-  }
+  static_assert(sizeof(PhaseConst) == 16, "a batch's constants are a word a lane");
+  static constexpr int kSmem = 4 * kWarpsOf * kWarpFloats;
 };
 
 __global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(const MacArgs a) {
@@ -325,13 +327,13 @@ __global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(con
   constexpr int kStage = SplitQ::kStage;
   static_assert(Gm::NG == 4 && 8 % (2 * kGroup) == 0, "a batch of X is eight channels x four bins");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  PhaseConst* pcs = reinterpret_cast<PhaseConst*>(smem_raw);
-  float* areas = reinterpret_cast<float*>(smem_raw + sizeof(PhaseConst) * a.n_chan);
+  float* areas = reinterpret_cast<float*>(smem_raw);
   const int warp = threadIdx.x >> 5;
   const int lane = threadIdx.x & 31;
   const int part = warp % kParts, set = warp / kParts;
-  float* const swap = areas + warp * (SplitQ::kSwap + SplitQ::kRing);
+  float* const swap = areas + warp * SplitQ::kWarpFloats;
   float2* const ring = reinterpret_cast<float2*>(swap + SplitQ::kSwap);
+  PhaseConst* const pcs = reinterpret_cast<PhaseConst*>(swap + SplitQ::kSwap + SplitQ::kRing);
   const int g = lane / Gm::G, lg = lane % Gm::G;
   const int ga = lg / Gm::GB, gb = lg % Gm::GB;
   const int k4 = (blockIdx.x * kBinSets + set) * 4;  // the four bins
@@ -345,18 +347,21 @@ __global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(con
   const int k_mine = k4 + (lane & 3);
   const float2* x_mine = a.X + static_cast<int64_t>(series) * a.x_series_stride +
                          (k_mine < a.n_bins ? k_mine : 0);  // (idle bins: bin 0, not stored)
-  auto fetch = [&](int c0) {  // an element a lane (zeros beyond the part)
+  const uint32_t* pc_mine = reinterpret_cast<const uint32_t*>(a.pc) + (lane & 3);
+  auto fetch = [&](int c0) {  // an element and a word of the constants a lane (zeros beyond the part)
     const int c = c0 + (lane >> 2);
     const bool in = c < n_c;
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
-                     dev::smem_u32(ring + (c0 / 8 % kXAhead) * 32 + lane)),
+    const int at = (c0 / 8 % kXAhead) * 32 + lane;
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dev::smem_u32(ring + at)),
                  "l"(x_mine + static_cast<int64_t>(in ? c_lo + c : 0) * a.x_chan_stride), "r"(in ? 8 : 0)
+                 : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                     dev::smem_u32(reinterpret_cast<uint32_t*>(pcs) + at)),
+                 "l"(pc_mine + 4 * (in ? c_lo + c : 0)), "r"(in ? 4 : 0)
                  : "memory");
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   for (int b = 0; b < kXAhead; ++b) fetch(8 * b);
-  for (int i = threadIdx.x; i < a.n_chan; i += SplitQ::kWarpsOf * 32) pcs[i] = a.pc[i];
-  __syncthreads();
 
   Generator<Gm, M> gen;
   gen.init(static_cast<uint32_t>(a.k_begin + (k < a.n_bins ? k : 0)), lg, a.j_begin + jblk);
@@ -367,7 +372,8 @@ __global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(con
 #pragma unroll
     for (int i = 0; i < kGroup; ++i)
       if (c0 + i < n_c)
-        gen.run(pcs[c_lo + c0 + i], ring[(c0 / 8 % kXAhead) * 32 + (c0 % 8 + i) * 4 + g],
+        gen.run(pcs[c0 / 8 % kXAhead * 8 + c0 % 8 + i],
+                ring[(c0 / 8 % kXAhead) * 32 + (c0 % 8 + i) * 4 + g],
                 grp0 + (area * kGroup + i) * kStage);
   };
   auto accumulate = [&](int c0, int area) {
@@ -414,7 +420,7 @@ __global__ void __launch_bounds__(SplitQ::kWarpsOf * 32, 3) mac_parts_kernel(con
 #pragma unroll
     for (int q = 0; q < kParts; ++q)
       v = __fadd2_rn(v, reinterpret_cast<const float2*>(
-                            areas + (set * kParts + q) * (SplitQ::kSwap + SplitQ::kRing))[
+                            areas + (set * kParts + q) * SplitQ::kWarpFloats)[
                             (part * Gm::BT + jj) * 32 + lane]);
     const int jl = jblk + (ga * Gm::AT + part) * Gm::TW + gb * Gm::BT + jj;
     if (jl < a.n_dm) {
@@ -792,8 +798,8 @@ cudaError_t mac_prepare(int variant, int n_chan) {
   const VariantInfo vi = variant_info(variant);
   const size_t bytes = mac_smem_bytes(variant, n_chan);
   cudaError_t e = allow_smem(vi.fn, bytes);
-  if (e == cudaSuccess && variant == MAC_Q_4x4 && SplitQ::smem(n_chan) <= kMaxSmem)
-    e = allow_smem(reinterpret_cast<const void*>(&mac_parts_kernel), SplitQ::smem(n_chan));
+  if (e == cudaSuccess && variant == MAC_Q_4x4)
+    e = allow_smem(reinterpret_cast<const void*>(&mac_parts_kernel), SplitQ::kSmem);
   if (e != cudaSuccess || !vi.batch_fn) return e;
   return allow_smem(vi.batch_fn, bytes);
 }
@@ -838,12 +844,11 @@ cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s) {
   VariantInfo vi = variant_info(variant);
   size_t smem = mac_smem_bytes(variant, a.n_chan);
   int bins_per_cta = vi.bins();
-  // (up to 11,000 channels, whose table fits beside the swap areas)
-  if (variant == MAC_Q_4x4 && SplitQ::smem(a.n_chan) <= kMaxSmem) {
+  if (variant == MAC_Q_4x4) {
     vi.fn = reinterpret_cast<const void*>(&mac_parts_kernel);
     vi.warps = SplitQ::kWarpsOf;
     bins_per_cta = 4 * kBinSets;
-    smem = SplitQ::smem(a.n_chan);
+    smem = SplitQ::kSmem;
   }
   dim3 grid((a.n_bins + bins_per_cta - 1) / bins_per_cta, (a.n_dm + vi.dms - 1) / vi.dms,
             a.n_series);

@@ -72,11 +72,10 @@ def test_edges_match_oracle(n_chan, n_dm, n_series):
     (1024, 256, TOL), (11200, 33, 5e-6), (11201, 33, 5e-6),
 ])
 def test_long_parts_match_oracle(n_chan, n_dm, tol):
-    """A part of more than 32 channels goes round the ring of X; 11200 channels
-    are the most whose phase table fits beside the swap areas, above them one
-    warp takes a bin's channels.  Sums of n terms round to 2^-25 sqrt(n / 2) of
-    the result: 3.4e-7 for a quarter of 1024 channels, 1.1e-6 for one of 11200,
-    2.2e-6 for 11201 in one sum, beside the phasors' 2.4e-7."""
+    """A part of more than 32 channels goes round the rings of X and of phase
+    constants.  Sums of n terms round to 2^-25 sqrt(n / 2) of the result: 3.4e-7 for a quarter of 1024
+    channels, 1.1e-6 for one of 11200, 2.2e-6 were they one sum, beside the
+    phasors' 2.4e-7."""
     L, dms = 1 << 12, 3.7 + 0.31 * np.arange(n_dm)
     dnu = (BAND[1] - BAND[0]) / n_chan
     nu = oracle.channel_centres(n_chan, BAND[0] + 0.5 * dnu, dnu)

@@ -304,8 +304,14 @@ __global__ void __launch_bounds__(W * 32, 1) mac_kernel(const MacArgs a) {
 // 4096 bins 1543 -> 1099.  (With the table beside the swap areas, one CTA an SM
 // of 4096 channels: 17.4, 74, 299, 1964.  Groups of four, two CTAs an SM, or
 // evaluating ahead without the split were slower, too.)
+// Up to kFewQ channels one warp takes them all: a part would have four at
+// most, fewer than its own start costs.  4096 bins x 3 series x 128 trials:
+// 1 channel 8.2 us against 12.7 in parts, 8 12.5 and 14.6, 16 16.5 and 18.5,
+// 20 18.6 and 18.6, 32 26.7 and 23.5; 500 bins: 16 channels 8.9 and 8, 20 10.2
+// and 8.
 constexpr int kParts = 4, kBinSets = 2;  // warps per four bins; fours of bins per CTA
 constexpr int kGroup = 2, kXAhead = 4;
+constexpr int kFewQ = 16;
 struct SplitQ {
   using Gm = G4x4;
   using M = PackedCompact<G4x4>;
@@ -844,7 +850,7 @@ cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s) {
   VariantInfo vi = variant_info(variant);
   size_t smem = mac_smem_bytes(variant, a.n_chan);
   int bins_per_cta = vi.bins();
-  if (variant == MAC_Q_4x4) {
+  if (variant == MAC_Q_4x4 && a.n_chan > kFewQ) {
     vi.fn = reinterpret_cast<const void*>(&mac_parts_kernel);
     vi.warps = SplitQ::kWarpsOf;
     bins_per_cta = 4 * kBinSets;

@@ -69,11 +69,13 @@ def test_edges_match_oracle(n_chan, n_dm, n_series):
 
 @pytest.mark.parametrize("n_chan,n_dm,tol", [
     (128, 5, TOL), (129, 130, TOL), (160, 128, TOL), (161, 40, TOL), (300, 129, TOL),
-    (1024, 256, TOL), (11200, 33, 5e-6), (11201, 33, 5e-6),
+    (1024, 256, TOL), (11200, 33, 5e-6), (11201, 33, 5e-6), (15, 3, TOL), (16, 200, TOL),
+    (17, 200, TOL),
 ])
 def test_long_parts_match_oracle(n_chan, n_dm, tol):
     """A part of more than 32 channels goes round the rings of X and of phase
-    constants.  Sums of n terms round to 2^-25 sqrt(n / 2) of the result: 3.4e-7 for a quarter of 1024
+    constants; up to 16 channels one warp takes them all.  Sums of n terms
+    round to 2^-25 sqrt(n / 2) of the result: 3.4e-7 for a quarter of 1024
     channels, 1.1e-6 for one of 11200, 2.2e-6 were they one sum, beside the
     phasors' 2.4e-7."""
     L, dms = 1 << 12, 3.7 + 0.31 * np.arange(n_dm)

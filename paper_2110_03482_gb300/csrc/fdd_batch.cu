@@ -758,7 +758,7 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
       // in four launches 9.6 ms, in one (of the widest form) 11.4.
       std::vector<int> order(wv.count);
       for (int i = 0; i < wv.count; ++i) order[i] = wv.first + i;
-      auto form = [&](int b) { return g12 ? fdd::mac_split_form(B->beams[b].n_dm) : 0; };
+      auto form = [&](int b) { return g12 ? fdd::mac_split_form(B->beams[b].n_dm, p->n_chan) : 0; };
       std::stable_sort(order.begin(), order.end(),
                        [&](int x, int y) { return form(x) > form(y); });
       int last_form = -1;
@@ -776,7 +776,7 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
         const bool tail = tails && rem > 0 && rem <= dms / 2;
         int blocks = full + (rem > 0 && !tail ? 1 : 0), tiles = 0;
         if (g12)
-          fdd::mac_split_batch_shape(n_dm, B->n_bins[b], &tiles, &blocks);
+          fdd::mac_split_batch_shape(n_dm, p->n_chan, B->n_bins[b], &tiles, &blocks);
         else
           tiles = static_cast<int>((B->n_bins[b] + bins_per_cta - 1) / bins_per_cta);
         for (int64_t c = 0; c < B->n_chunks[b]; ++c) {

@@ -96,12 +96,13 @@ size_t mac_smem_bytes(int variant, int n_chan);
 size_t mac_split_smem_bytes();
 cudaError_t mac_split_prepare();
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s);
-// whether the series of one launch share passes at this trial count
+// whether the series of one launch share passes at this trial count (with few
+// channels they share the launch only)
 bool mac_split_series_share(int n_dm);
-int mac_split_form(int n_dm);
-void mac_split_batch_shape(int n_dm, long long n_bins, int* bin_groups, int* passes);
+int mac_split_form(int n_dm, int n_chan);
+void mac_split_batch_shape(int n_dm, int n_chan, long long n_bins, int* bin_groups, int* passes);
 cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
-                                   int max_n_dm, int n_ctas, cudaStream_t s);
+                                   int max_n_dm, int n_chan, int n_ctas, cudaStream_t s);
 
 // Tensor-core phase-rotate-and-sum (fdd_mac_tc.cu): 16-bit (or FP8)
 // phasors and data, FP32 accumulation in tensor memory; persistent CTAs (one

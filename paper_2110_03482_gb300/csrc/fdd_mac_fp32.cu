@@ -834,7 +834,7 @@ cudaError_t launch_mac_batch(const BatchSet* d_sets, int n_sets, long long n_ite
                              unsigned long long* d_counter, int variant, int n_ctas, int n_chan,
                              int max_n_dm, cudaStream_t s) {
   if (variant == MAC_G12_4x8)
-    return launch_mac_split_batch(d_sets, n_sets, n_items, max_n_dm, n_ctas, s);
+    return launch_mac_split_batch(d_sets, n_sets, n_items, max_n_dm, n_chan, n_ctas, s);
   const VariantInfo vi = variant_info(variant);
   if (!vi.batch_fn) return cudaErrorInvalidValue;
   if (n_items <= 0) return cudaSuccess;

@@ -60,6 +60,7 @@
 // loop unrolled by stage (334: instruction fetch), lo hi as an MMA of its own
 // (307), four more warps to store, with the producers at 80 registers (335).
 #include <atomic>
+#include <climits>
 
 #include <cuda_fp16.h>
 
@@ -1003,11 +1004,23 @@ FormInfo form_info(Form f) {
 // may depend on the series only among those whose results are the same bits.
 // 4096 bins x 1024 channels x 512 trials take 190 us in twin stages, 249 in
 // those for 1024.
-Form form_for(int n_dm, int n_series, int of_n_dm) {
+// With few channels the rows cost little and storing the sums is what counts,
+// which a pass of more bins does in fewer and longer pieces: there more than
+// 2048 trials go through passes of 2048, and series by themselves (in one
+// launch), with the same bits.  4096 bins x 8192 trials: 1 channel 159 us in
+// passes of 2048 and 378 of 4096, 64 channels 184 and 381, 128 246 and 336
+// (3000 trials 119 and 135), 192 340 and 359 (3000 trials 165 and 150).  4096
+// bins x 3 series x 700 trials: 1 channel 62 us alone and 72 shared, 32 67 and
+// 76, 64 79 and 84 (but 4 series x 600 trials 8 % slower alone); x 2048 trials
+// 120 and 169, 124 and 172, 138 and 173, 100 channels 178 and 206 (but 2 series
+// x 1100 trials 10 % slower alone).
+constexpr int kFewForPass = 128, kFewForTwo2048 = 64, kFewFor1024 = 32;
+Form form_for(int n_dm, int n_series, int of_n_dm, int n_chan) {
   const int total = (n_dm + kPairTrials - 1) / kPairTrials;
-  if (total > 8) return kUpTo4096;
+  if (total > 8) return n_chan > kFewForPass ? kUpTo4096 : kUpTo2048;
   if (of_n_dm > 0 && of_n_dm <= 2 * kPairTrials) return kUpTo512;
-  if (total > 4) return n_series >= 2 ? kTwoUpTo2048 : kUpTo2048;
+  if (total > 4) return n_series >= 2 && n_chan > kFewForTwo2048 ? kTwoUpTo2048 : kUpTo2048;
+  if (n_chan <= kFewFor1024) return kUpTo1024;
   return n_series >= 4 ? kFourUpTo1024 : n_series >= 2 ? kTwoUpTo1024 : kUpTo1024;
 }
 
@@ -1059,22 +1072,22 @@ cudaError_t mac_split_prepare() {
   return e;
 }
 
-bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2, n_dm)).sets > 1; }
+bool mac_split_series_share(int n_dm) { return form_info(form_for(n_dm, 2, n_dm, INT_MAX)).sets > 1; }
 
-int mac_split_form(int n_dm) { return form_for(n_dm, 1, n_dm); }
+int mac_split_form(int n_dm, int n_chan) { return form_for(n_dm, 1, n_dm, n_chan); }
 
-void mac_split_batch_shape(int n_dm, long long n_bins, int* bin_groups, int* passes) {
-  const FormInfo f = form_info(form_for(n_dm, 1, n_dm));
+void mac_split_batch_shape(int n_dm, int n_chan, long long n_bins, int* bin_groups, int* passes) {
+  const FormInfo f = form_info(form_for(n_dm, 1, n_dm, n_chan));
   *bin_groups = static_cast<int>((n_bins + f.bins - 1) / f.bins);
   *passes = (n_dm + f.pass_trials - 1) / f.pass_trials;
 }
 
 cudaError_t launch_mac_split_batch(const BatchSet* d_sets, int n_sets, long long n_items,
-                                   int max_n_dm, int n_ctas, cudaStream_t s) {
+                                   int max_n_dm, int n_chan, int n_ctas, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   if (n_items > kMaxItems) return cudaErrorInvalidConfiguration;
   return launch_split(MacArgs{}, d_sets, n_sets, static_cast<int>(n_items),
-                      form_info(form_for(max_n_dm, 1, max_n_dm)), n_ctas, s);
+                      form_info(form_for(max_n_dm, 1, max_n_dm, n_chan)), n_ctas, s);
 }
 
 cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
@@ -1084,7 +1097,7 @@ cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
   const size_t y_elem = a.out_kind == 2 ? sizeof(float) : sizeof(float2);
   // series in groups that share passes, then the rest by themselves
   for (int s0 = 0; s0 < a.n_series;) {
-    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0, a.of_n_dm));
+    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0, a.of_n_dm, a.n_chan));
     const long long per_set = static_cast<long long>((a.n_bins + f.bins - 1) / f.bins) *
                               ((a.n_dm + f.pass_trials - 1) / f.pass_trials);
     if (per_set > kMaxItems) return cudaErrorInvalidConfiguration;

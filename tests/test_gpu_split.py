@@ -236,3 +236,32 @@ def test_infinite_samples_stay_in_their_bin(n_dm):
     hit = hit[:, None].expand(n_series, n_dm, nb)
     assert not torch.any(torch.isfinite(dY[hit])) and not torch.any(torch.isfinite(dP[hit]))
     assert torch.equal(dY[~hit], clean[~hit])
+
+
+@pytest.mark.parametrize("nb", [5, 260])
+@pytest.mark.parametrize("n_dm", [700, 2048, 2049, 5000, 9000])
+@pytest.mark.parametrize("n_chan", [32, 33, 64, 65, 128, 129])
+def test_forms_by_channel_count_give_the_same_bits(n_chan, n_dm, nb):
+    """On both sides of the channel counts at which series begin to share
+    passes and passes of 4096 trials begin, in one launch of few bins and in
+    several of more: a series among five has the bits it has alone, and blocks
+    of 2048 trials those of the whole call."""
+    n_series, L = 5, 1 << 12
+    dms = 0.25 * np.arange(n_dm)
+    rng = np.random.default_rng(n_chan + n_dm)
+    X = (rng.standard_normal((n_series, n_chan, nb)) +
+         1j * rng.standard_normal((n_series, n_chan, nb))).astype(np.complex64)
+    dX = complex_to_device(X, nb)
+    with _plan(n_chan, L, dms) as plan:
+        whole = torch.full((n_series, n_dm, nb, 2), 7.0, device="cuda")
+        plan.dedisperse_spectra_bins(dX, nb, n_series, 999, nb, 0, n_dm, whole, nb)
+        for j in range(0, n_dm, 2048):
+            n = min(2048, n_dm - j)
+            for s in (0, 4):
+                part = torch.full((n, nb, 2), 7.0, device="cuda")
+                plan.dedisperse_spectra_bins(dX[s].contiguous(), nb, 1, 999, nb, j, n, part, nb)
+                assert torch.equal(part, whole[s, j:j + n]), (j, s)
+        torch.cuda.synchronize()
+        plan.query()
+    ref = _reference(X[2, :, :5].astype(np.complex128), np.arange(999, 1004), L, n_chan, dms)
+    assert rel_l2(device_to_complex(whole[2, :, :5], 5), ref) <= TOL

@@ -1095,14 +1095,27 @@ cudaError_t launch_mac_split(const MacArgs& a, cudaStream_t s) {
   cudaError_t e = sm_count(&n_sms);
   if (e != cudaSuccess) return e;
   const size_t y_elem = a.out_kind == 2 ? sizeof(float) : sizeof(float2);
-  // series in groups that share passes, then the rest by themselves
+  auto items = [&](const FormInfo& f) {
+    return static_cast<long long>((a.n_bins + f.bins - 1) / f.bins) *
+           ((a.n_dm + f.pass_trials - 1) / f.pass_trials);
+  };
+  // Series in groups that share passes, then the rest in smaller groups, in
+  // launches one after another; or all by themselves in one launch, where that
+  // takes no more than one item per SM (of two stages of channels at most, no
+  // more than launches saved).  3 series x 600 trials x 48 channels x 200
+  // bins: 10 us in one launch, 19 in two; 1024 channels x 64 bins 41 and 70.
   for (int s0 = 0; s0 < a.n_series;) {
-    const FormInfo f = form_info(form_for(a.n_dm, a.n_series - s0, a.of_n_dm, a.n_chan));
-    const long long per_set = static_cast<long long>((a.n_bins + f.bins - 1) / f.bins) *
-                              ((a.n_dm + f.pass_trials - 1) / f.pass_trials);
+    const int left = a.n_series - s0;
+    FormInfo f = form_info(form_for(a.n_dm, left, a.of_n_dm, a.n_chan));
+    const FormInfo alone = form_info(form_for(a.n_dm, 1, a.of_n_dm, a.n_chan));
+    int launches = 0;
+    for (int l = left; l > 0; ++launches) l %= form_info(form_for(a.n_dm, l, a.of_n_dm, a.n_chan)).sets;
+    if (launches > 1 && left * items(alone) <= (a.n_chan > kFewForPass ? 1 : launches) * n_sms)
+      f = alone;
+    const long long per_set = items(f);
     if (per_set > kMaxItems) return cudaErrorInvalidConfiguration;
     // (as many as leave item numbers in an int)
-    long long sets = (a.n_series - s0) / f.sets;
+    long long sets = left / f.sets;
     if (sets > kMaxItems / per_set) sets = kMaxItems / per_set;
     MacArgs c = a;
     c.n_series = static_cast<int>(sets) * f.sets;

@@ -450,8 +450,7 @@ fdd_status compute_plan(const fdd_params* p, fdd_info* g, fdd::CoreGeometry* cor
     return n > pass2 / 2 && (r == 0 || r > pass2 / 2);
   };
   bool pair = tc && p->spin_group == 0 && pair_wins(p->n_dm);
-  if (!tc && fdd::mac_smem_bytes(g->mac_variant, nc) > kMaxSmem)
-    return fail(FDD_ERR_UNSUPPORTED, "n_chan %d needs more shared memory than a CTA has", nc);
+  if (!tc && (st = fdd::mac_variant_check(g->mac_variant, nc)) != FDD_OK) return st;
 
   const size_t spectra_sets = tc ? static_cast<size_t>(p->n_beams) : 1;
   const size_t fixed = sizeof(fdd::PhaseConst) * nc + sizeof(float) * size_t(nc) * L +
@@ -1276,8 +1275,7 @@ fdd_status plan_create(const fdd_params* p, void* arena, size_t arena_bytes, fdd
     P->spin_scratch_bytes = fdd::spin_scratch_bytes(P->spin, nc, g.n_bins);
     if ((st = ws_alloc(P, &P->d_spin_scratch, P->spin_scratch_bytes))) return st;
     P->spin_fp32_variant = fdd::mac_variant_for(p->n_dm, nc);
-    if (fdd::mac_smem_bytes(P->spin_fp32_variant, nc) > kMaxSmem)
-      return fail(FDD_ERR_UNSUPPORTED, "n_chan %d needs more shared memory than a CTA has", nc);
+    if ((st = fdd::mac_variant_check(P->spin_fp32_variant, nc)) != FDD_OK) return st;
     FDD_CUDA(fdd::mac_prepare(P->spin_fp32_variant, nc));
   }
   FDD_CUDA(cudaMemset(P->d_status, 0, 256));

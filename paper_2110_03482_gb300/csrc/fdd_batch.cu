@@ -834,7 +834,7 @@ fdd_status fdd_batch_plan(const fdd_params* p, const fdd_beam_desc* beams, int32
   }
 
   auto tile_fits = [&](int v) {
-    if (fdd::mac_smem_bytes(v, p->n_chan) > 227 * 1024) return false;
+    if (!fdd::mac_variant_takes(v, p->n_chan)) return false;
     if (fdd::mac_prepare(v, p->n_chan) != cudaSuccess) {
       cudaGetLastError();
       return false;

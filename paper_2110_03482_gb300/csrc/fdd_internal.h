@@ -87,6 +87,10 @@ int mac_variant_trials_per_block(int variant);
 cudaError_t mac_prepare(int variant, int n_chan);  // kernel attributes (host, once)
 cudaError_t launch_mac_fp32(const MacArgs& a, int variant, cudaStream_t s);
 size_t mac_smem_bytes(int variant, int n_chan);
+// Whether plans of n_chan channels may take the tile; reports why not
+// (FDD_ERR_UNSUPPORTED) otherwise.
+bool mac_variant_takes(int variant, int n_chan);
+fdd_status mac_variant_check(int variant, int n_chan);
 
 // The G12_4X8 tile (fdd_mac_split.cu): split-FP16 operands on the tensor
 // cores.  A batch's sets go into one launch by the form of their passes

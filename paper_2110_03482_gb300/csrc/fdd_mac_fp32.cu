@@ -36,6 +36,8 @@
 // Lanes are numbered lane = ga * GB + gb, so each quarter warp reads a single
 // Z row (a broadcast) and GB distinct P rows; the P rows are padded so that
 // those reads fall in distinct shared-memory banks.
+#include <cstdio>
+
 #include "fdd_device.cuh"
 #include "fdd_internal.h"
 
@@ -770,7 +772,7 @@ VariantInfo variant_info(int v) {
 // four-product warp-specialised tile W12_8x8 measured 0.621 on the same
 // launch, Q12_8x8, the 2048-trial tile on the plain schedule, 0.553.)
 int mac_variant_for(int n_dm, int n_chan) {
-  if (n_dm > 256 && mac_smem_bytes(MAC_G12_4x8, n_chan) <= kMaxSmem) return MAC_G12_4x8;
+  if (n_dm > 256 && mac_variant_takes(MAC_G12_4x8, n_chan)) return MAC_G12_4x8;
   struct Tile {
     int variant, block;
     double rate;
@@ -780,7 +782,7 @@ int mac_variant_for(int n_dm, int n_chan) {
   int best = MAC_W12_8x8;  // (the smallest shared-memory need of the 2048-trial tiles)
   double best_cost = 0.0;
   for (const Tile& t : tiles) {
-    if (mac_smem_bytes(t.variant, n_chan) > kMaxSmem) continue;
+    if (!mac_variant_takes(t.variant, n_chan)) continue;
     const double cost = (n_dm + t.block - 1) / t.block * t.block / t.rate;
     if (best_cost == 0.0 || cost < best_cost) {
       best = t.variant;
@@ -795,8 +797,23 @@ int mac_variant_trials_per_block(int variant) {
 }
 
 size_t mac_smem_bytes(int variant, int n_chan) {
-  if (variant == MAC_G12_4x8) return n_chan <= kG12MaxChan ? mac_split_smem_bytes() : kMaxSmem + 1;
+  if (variant == MAC_G12_4x8) return mac_split_smem_bytes();
   return sizeof(PhaseConst) * static_cast<size_t>(n_chan) + variant_info(variant).swap_bytes;
+}
+
+bool mac_variant_takes(int variant, int n_chan) {
+  return variant == MAC_G12_4x8 ? n_chan <= kG12MaxChan : mac_smem_bytes(variant, n_chan) <= kMaxSmem;
+}
+
+fdd_status mac_variant_check(int variant, int n_chan) {
+  if (mac_variant_takes(variant, n_chan)) return FDD_OK;
+  char text[96];
+  if (variant == MAC_G12_4x8)
+    std::snprintf(text, sizeof text, "n_chan %d is above the %d channels that the G12_4X8 tile is used for",
+                  n_chan, kG12MaxChan);
+  else
+    std::snprintf(text, sizeof text, "n_chan %d needs more shared memory than a CTA has", n_chan);
+  return report_error(FDD_ERR_UNSUPPORTED, text);
 }
 
 cudaError_t mac_prepare(int variant, int n_chan) {

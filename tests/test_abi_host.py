@@ -170,6 +170,22 @@ def test_variant_choice():
     assert g["mac_variant"] not in (fdd.FDD_MAC_G12_4X8, fdd.FDD_MAC_TC)
 
 
+@pytest.mark.parametrize("variant,n_chan,text", [
+    (fdd.FDD_MAC_G12_4X8, 8381, None), (fdd.FDD_MAC_G12_4X8, 8382, "8381"),
+    (fdd.FDD_MAC_Q_4X4, 13000, None), (fdd.FDD_MAC_Q_4X4, 14000, "shared memory")])
+def test_tiles_refuse_channels_for_their_own_reason(variant, n_chan, text):
+    w = synth.WORKLOADS["fdd_1024ch_2p20t_2048dm"]
+    p = _params(w, n_chan=n_chan, dnu_mhz=0.02, workspace_limit=250 << 30, mac_variant=1 + variant)
+    if text is None:
+        assert fdd.fdd_plan_geometry(p)["mac_variant"] == variant
+        return
+    with pytest.raises(fdd.FddError) as e:
+        fdd.fdd_plan_geometry(p)
+    assert e.value.status == fdd.FDD_ERR_UNSUPPORTED
+    assert text in fdd.fdd_last_error() and ("shared memory" in text or
+                                             "shared memory" not in fdd.fdd_last_error())
+
+
 def test_tensor_core_form_geometry():
     """The tensor-core form holds the spectra of every beam at once and batches
     DMs in whole trial passes when the workspace is bounded (below one pass,

@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&sm.pfree[i], C::kTasks);
     }
     for (int i = 0; i < S; ++i) {
-      mbar_init(&sm.full[i], C::kTasks);
+      mbar_init(&sm.full[i], C::kTasks + (a.test_withhold ? 1 : 0));  // (never all: stalled)
       mbar_init(&sm.done[i], 1);
     }
     for (int i = 0; i < C::kAccs; ++i) mbar_init(&sm.acc_free[i], kEpiWarps);
@@ -953,7 +953,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
       if (lane == 0) {
-        if (!a.test_withhold) mbar_arrive(&sm.full[s]);  // (never set for a batch)
+        mbar_arrive(&sm.full[s]);
         mbar_arrive(&sm.pfree[ts]);
       }
     }

@@ -108,7 +108,10 @@ typedef enum fdd_status {
                                workspace_limit                                 */
 
 /* fdd_params.precision */
-#define FDD_PREC_FP32 0      /* FP32 phasors and accumulation (CUDA cores)       */
+#define FDD_PREC_FP32 0      /* FP32 accuracy: FP32 operands on CUDA cores, or two
+                                FP16 terms per operand (22 bits) on tensor cores
+                                with FP32 sums (G12_4X8; relative error of the
+                                spectra 2.4e-7 to 3.5e-7)                        */
 #define FDD_PREC_BF16_HILO 1 /* tensor cores (tcgen05), the direction of Sect. 5:
                                 BF16 hi+lo phasors, BF16 data, FP32 accumulation;
                                 all beams of a chunk share each bin's phasors    */
@@ -145,7 +148,11 @@ typedef struct fdd_params {
   int32_t mac_variant;    /* phase-rotate-and-sum kernel: 0 chooses automatically;
                              1 + FDD_MAC_* forces that variant                      */
   size_t workspace_limit; /* device bytes the plan may hold; 0 = library default
-                             (16 GiB).  Plans of the G12_4X8 tile with 513 to
+                             (16 GiB).  It bounds the trials per batch or block;
+                             with spectra or power output the spectra of one
+                             chunk (tensor-core forms: of every beam, twice for
+                             one of them, and their scratch) are held even
+                             where they exceed it.  Plans of the G12_4X8 tile with 513 to
                              2048 trials and two or more beams or chunks hold a
                              second one's spectra (and dedispersed spectra, for
                              time output) where they fit: fdd_execute then takes
@@ -413,7 +420,8 @@ fdd_status fdd_dedisperse_spectra_bins(fdd_plan_t plan, const void* d_X, int64_t
  *   d_in  : as fdd_execute (u8 or f32, either layout, n_beams beams).
  *   d_out : float [n_beams][n_dm][n_t - d_max].
  * The first call builds the shift tables and a channel-major copy of one
- * beam (n_chan x n_t floats) in plan memory; later calls reuse them.
+ * beam (n_chan x n_t floats; bytes for 8-bit input of up to 65793 channels,
+ * whose sums are exact either way) in plan memory; later calls reuse them.
  * Asynchronous on the stream.  Errors: FDD_ERR_INVALID_ARG (NULL pointers,
  * n_t <= d_max), FDD_ERR_UNSUPPORTED (a block of 32 trials spans more than
  * ~3300 samples of delay in one channel, or more than 2^24 output samples),
@@ -535,7 +543,9 @@ typedef struct fdd_batch_info {
  * fixed part (n_chan x max L floats of staging, the phase tables and a
  * 64 MiB reserve for the FFT work area);
  * each wave is one persistent launch of the phase-rotate-and-sum whose CTAs
- * take (beam, chunk, bin tile, trial block) work items from a counter.  With
+ * take (beam, chunk, bin tile, trial block) work items from a counter (with
+ * the G12_4X8 tile one launch for each of the up to four sizes of its passes
+ * that the beams' trial counts take).  With
  * mac_variant 0 and autotune != 0 the candidate kernel tiles are timed on the
  * batch's own shapes and the fastest is kept (remembered per shape in the
  * process, and in the text file named by the FDD_AUTOTUNE_CACHE environment

@@ -350,7 +350,7 @@ size_t spin_plan_bytes(const fdd_params* p, const fdd::CoreGeometry& cg, int64_t
 
 // Bytes a plan holds to take two (beam, chunk)s through each launch of the
 // phase-rotate-and-sum: the G12 tile's series share its cosine and sine rows
-// (1024 channels x 2048 trials: 73 ns a bin one by one, 52 in twos).  Only what
+// (1024 channels x 2048 trials: 73 ns a bin one by one, 55 in twos).  Only what
 // fits the limit beside the rest, with every trial in one batch, as the
 // batches' order is the same then; 0 where there is nothing to share or no room.
 size_t pairing_bytes(const fdd_params* p, const fdd_info* g) {

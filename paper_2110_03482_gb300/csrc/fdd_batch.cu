@@ -6,8 +6,9 @@
 // wave the beams are unpacked and transformed one by one, whole or in their
 // own overlap-save chunks (one cuFFT plan per distinct transform length),
 // then ONE persistent launch of the FP32 phase-rotate-and-sum serves the
-// whole wave (the G12 tile: one per form of its passes): its CTAs pull (beam,
-// chunk, bin tile, trial block) items from a counter.  The whole execute is captured once as a
+// whole wave: its CTAs pull (beam, chunk, bin tile, trial block) items from a
+// counter (the G12 tile: one launch per form of its passes, whose items are
+// dealt out in turn).  The whole execute is captured once as a
 // CUDA graph and replayed.  At plan time an autotuner times the candidate
 // kernel tiles on the batch's real shapes and keeps the fastest.
 #include <cufft.h>

@@ -763,12 +763,13 @@ VariantInfo variant_info(int v) {
 // Default tile for a trial count.  From 257 trials on the G12 tile while the
 // channels allow it: on 4096 bins x 1024 channels its passes of up to 512,
 // 1024, 2048 and 4096 trials take 190, 250, 300 and 430 us whatever their filling,
-// the 128-trial tile 310 us at 256 trials and more with every 128.  (From 129 to
+// the 128-trial tile 281 us at 256 trials and more with every 128.  (From 129 to
 // 256 trials the G12 tile would be the faster one too with many channels; plans
-// have always reported Q_4X4 there, and keep to it.)  Otherwise the tile with the least time for the padded trial
-// blocks, ceil(n_dm / block) * block / rate, with each tile's rate measured
-// kernel-only (fraction of the FP32 peak, 1024 channels, 131073 bins): Q_4x8
-// 0.493 (1024-trial blocks), Q_8x8_512 0.415 (512), Q_4x4 0.347 (128).  (The
+// have always reported Q_4X4 there, and keep to it.)  Otherwise the tile with
+// the least time for the padded trial blocks, ceil(n_dm / block) * block /
+// rate, with each tile's rate measured kernel-only (fraction of the FP32 peak,
+// 1024 channels, 131073 bins): Q_4x8 0.493 (1024-trial blocks), Q_8x8_512 0.415
+// (512), Q_4x4 0.347 (128; before its warps shared the channels).  (The
 // four-product warp-specialised tile W12_8x8 measured 0.621 on the same
 // launch, Q12_8x8, the 2048-trial tile on the plain schedule, 0.553.)
 int mac_variant_for(int n_dm, int n_chan) {

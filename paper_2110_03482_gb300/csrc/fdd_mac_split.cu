@@ -27,10 +27,11 @@
 // formed as hi hi + (hi lo + lo hi) on tcgen05 with FP32 accumulators.  The
 // tensor cores round their sums toward zero, so an accumulator only lives for
 // one stage; the stages' sums are added in FP32 registers (to nearest).  The
-// error against FP64 is 3.2e-7 of the result whatever the channel count (rows
-// and columns from the hardware sine, 1.6e-7 each); the FP32 multiply-adds
-// this replaces rounded every sum: 3.2e-7 at 64 channels, 4.2e-7 at 200,
-// 7.7e-7 at 1024.
+// error of the spectra against FP64 is 2.4e-7 of the result at 64 channels and
+// 2.5e-7 at 256 (rows from the hardware sine, columns from a series), 3.4e-7 from 257
+// to 512, 3.5e-7 at 1024 and 2048 (both from the hardware sine); the FP32
+// multiply-adds this replaces rounded every sum: 3.1e-7 at 64 channels, 4.5e-7
+// at 256, 7.7e-7 at 1024, 1.1e-6 at 2048.
 //
 // Sixty-four channels of a bin are a stage.  Two warps turn the spectra and
 // phase constants into a table per stage, thirteen evaluate and split rows and
@@ -38,11 +39,11 @@
 // four add the stages up and store.  4096 bins x 1024 channels x 2048 trials
 // take 300 us, against 1185 us for the FP32 multiply-adds (three real products
 // per complex one) at 0.75 of the FP32 peak; 301 bins x 4096 channels x 8192
-// trials 210 against 1292 us; 701 trials of 2 x 387 channels 140 against 560 us.
-// What bounds it: writing and reading the operands in shared memory (71 % of
-// its cycles, the MMAs' reads and the producers' stores about equal) beside
-// 50 warp instructions per bin and channel (61 % of the issue slots), most of
-// them phasors and splits of the 128 rows.  Hence the wide passes: the rows
+// trials 212 against 1292 us; 701 trials of 2 x 387 channels 151 against 560 us.
+// What bounds it (two series of 2048 trials a pass): writing and reading the
+// operands in shared memory (82 % of its cycles, 24 of them the MMAs' reads)
+// beside 65 warp instructions per bin and channel (55 % of the issue slots),
+// most of them phasors and splits of the 128 rows.  Hence the wide passes: the rows
 // serve all columns of a pass, up to 4096 trials of one series.  Several series
 // share them too (two, or four up to 1024 trials), each with its own columns
 // and scales and the bits it has alone: 4096 (bin, series) x 1024 channels of
@@ -99,10 +100,14 @@ __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volati
 constexpr int kCh = 64;     // channels per stage (four K steps of 16)
 constexpr int kRows = 128;  // Cb, Sb of 64 b's: sixteen b's Cb, then their Sb, and so on
 // Up to this many channels the columns' phasors come from the Taylor series,
-// too: over so few the FP32 multiply-adds' sums lost little (3.9e-7 of the
-// spectra, 5.1e-7 of the power at 167 channels; this product 3.4e-7 and 5.2e-7
-// with the hardware's columns, 2.5e-7 and 3.7e-7 with these).  167 channels x 911
-// trials x 1829 bins take 39.0 us, 37.3 with the hardware's, 80 before.
+// too: over so few the FP32 multiply-adds' sums lost little, and the product with
+// the hardware's columns would lose more.  Error of the power against FP64,
+// FP32 multiply-adds, hardware's columns, series: 64 channels 4.2, 5.0 and
+// 3.5e-7, 128 4.8, 5.1 and 3.7, 200 5.3, 5.2 and 3.7, 256 5.7, 5.3 and 3.7, 512
+// 7.2, 5.3 and 3.8 (of the spectra the hardware's columns lose more up to some
+// 80 channels).  The series costs (911 trials x 1829 bins) nothing at 64 and 128
+// channels, 42.0 against 41.0 us at 200, 44.8 against 43.1 at 256, 78.3 against
+// 76.6 at 512; the line is the next whole stage above 200.
 constexpr int kFewChan = 256;
 constexpr int kPairTrials = 256;  // trials per al: s, t = +-1, 64 b's (twin: half)
 constexpr int kBlockAls = 8;      // al's of a whole block (2048 trials)
@@ -142,7 +147,7 @@ struct Cfg {
   static constexpr int kStages = kNa == 16 ? 4 : 5;
   // (tables run further ahead than operands)
   static constexpr int kTables = 8;
-  static constexpr uint32_t kATile = kRows * kCh * 2;  // 8 KB per term
+  static constexpr uint32_t kATile = kRows * kCh * 2;  // 16 KB per term
   static constexpr uint32_t kBTile = kN * kCh * 2;
   static constexpr uint32_t kStageBytes = 2 * (kATile + kBTile);
   // tasks of a stage, dealt to the producer warps in turn: the columns (sixteen
@@ -277,7 +282,7 @@ __device__ __forceinline__ void split2(float2 v, uint32_t& hi, uint32_t& lo) {
 // x^8 and x^9 on |x| <= pi / 4 (truncation below 3e-8, rounding of the order
 // of 2^-24), two phases per instruction.  The stage tables use it: their
 // phasors multiply every row and column of a channel, where the hardware
-// sine's 2^-21 would be seen twice.
+// sine's 2^-21 would be seen twice; and the columns of calls of few channels.
 __device__ __forceinline__ void sincos2(uint32_t p0, uint32_t p1, float2& cs, float2& sn) {
   const uint32_t q0 = (p0 + 0x20000000u) >> 30, q1 = (p1 + 0x20000000u) >> 30;
   const float2 r = make_float2(static_cast<float>(static_cast<int>(p0 - (q0 << 30))),

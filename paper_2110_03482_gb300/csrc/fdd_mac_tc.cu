@@ -416,9 +416,9 @@ __global__ void __launch_bounds__(kThreads, 1) mac_tc_kernel(const MacArgs a) {
       // descriptors come from uniform registers: issued by a lone thread of a
       // divided warp an MMA takes up to 260 cycles to issue, twice as long as
       // it runs (128 at N = 256).  16 beams x 4096 channels x 8192 trials x
-      // 129 bins in BF16 hi + lo 858 -> 793 us, 32 beams x 1024 channels x 4096
+      // 129 bins in BF16 hi + lo 858 -> 810 us, 32 beams x 1024 channels x 4096
       // trials x 1025 bins in FP16 (bound by the producers and the read-out)
-      // 1637 -> 1606 us.
+      // 1629 -> 1598 us.
       const uint32_t el = elect_one();
       const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
       const uint32_t ring = __shfl_sync(0xffffffffu, smem_u32(base), 0);
